@@ -363,7 +363,7 @@ lsw_status lsw_solve_sweep(const lsw_grid* grid, const double* velocity, const d
                            lsw_sweep_info* info, lsw_solve_info* sinfo, void* stream);
 
 /* Measure the operator's pass variants for this grid and precision on
- * nbatch fields -- 0: register radix-8 FFT passes, 1: the same with
+ * nbatch fields -- 0: register FFT passes, 1: the same with
  * 512-thread row blocks in the x pass, 2: shared-memory Stockham passes --
  * and use the fastest for this (2nz, 2nx, precision) from now on in this
  * process.  *variant (may be NULL) receives the choice, ms3 (may be NULL)

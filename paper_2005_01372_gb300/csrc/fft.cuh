@@ -22,14 +22,28 @@ __device__ __forceinline__ C twiddle(const C* __restrict__ tw, int m, bool inv) 
     return w;
 }
 
-// multiply by -i (forward) or +i (inverse)
-template <typename C>
-__device__ __forceinline__ C rot90(C a, bool inv) { return inv ? mk(-a.y, a.x) : mk(a.y, -a.x); }
+// Complex sums of the butterflies: for FP32 one packed instruction per
+// complex entry instead of two.
+template <typename C> __device__ __forceinline__ C vadd(C a, C b) { return cadd(a, b); }
+template <typename C> __device__ __forceinline__ C vsub(C a, C b) { return csub(a, b); }
+template <> __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+template <> __device__ __forceinline__ float2 vsub(float2 a, float2 b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;"
+        : "=l"(r)
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+    return reinterpret_cast<const float2&>(r);
+}
 
 template <typename C>
 __device__ __forceinline__ void dft4(C& v0, C& v1, C& v2, C& v3, bool inv) {
-    C t0 = cadd(v0, v2), t1 = csub(v0, v2), t2 = cadd(v1, v3), t3 = rot90(csub(v1, v3), inv);
-    v0 = cadd(t0, t2); v2 = csub(t0, t2); v1 = cadd(t1, t3); v3 = csub(t1, t3);
+    const C t0 = vadd(v0, v2), t1 = vsub(v0, v2), t2 = vadd(v1, v3), t3 = vsub(v1, v3);
+    v0 = vadd(t0, t2);
+    v2 = vsub(t0, t2);
+    // t1 +- (-i) t3 (forward) or (+i) t3
+    const C a = mk(t1.x + t3.y, t1.y - t3.x), b = mk(t1.x - t3.y, t1.y + t3.x);
+    v1 = inv ? b : a;
+    v3 = inv ? a : b;
 }
 
 template <typename C>
@@ -42,13 +56,14 @@ __device__ __forceinline__ void dft8(C* v, bool inv) {
     typedef decltype(o0.x) R;
     const R s = (R)0.70710678118654752440;
     // w8^1 = (1 -+ i)/sqrt2, w8^2 = -+ i, w8^3 = (-1 -+ i)/sqrt2
-    C w1o1 = inv ? mk((o1.x - o1.y) * s, (o1.x + o1.y) * s) : mk((o1.x + o1.y) * s, (o1.y - o1.x) * s);
-    C w2o2 = rot90(o2, inv);
-    C w3o3 = inv ? mk((-o3.x - o3.y) * s, (o3.x - o3.y) * s) : mk((o3.y - o3.x) * s, (-o3.x - o3.y) * s);
-    v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
-    v[1] = cadd(e1, w1o1); v[5] = csub(e1, w1o1);
-    v[2] = cadd(e2, w2o2); v[6] = csub(e2, w2o2);
-    v[3] = cadd(e3, w3o3); v[7] = csub(e3, w3o3);
+    const C w1o1 = inv ? mk((o1.x - o1.y) * s, (o1.x + o1.y) * s) : mk((o1.x + o1.y) * s, (o1.y - o1.x) * s);
+    const C w3o3 = inv ? mk((-o3.x - o3.y) * s, (o3.x - o3.y) * s) : mk((o3.y - o3.x) * s, (-o3.x - o3.y) * s);
+    v[0] = vadd(e0, o0); v[4] = vsub(e0, o0);
+    v[1] = vadd(e1, w1o1); v[5] = vsub(e1, w1o1);
+    const C a = mk(e2.x + o2.y, e2.y - o2.x), b = mk(e2.x - o2.y, e2.y + o2.x);
+    v[2] = inv ? b : a;
+    v[6] = inv ? a : b;
+    v[3] = vadd(e3, w3o3); v[7] = vsub(e3, w3o3);
 }
 
 // One radix-R stage over nlines lines of length P (line l at s + l*lstride).
@@ -113,72 +128,176 @@ __device__ void smem_fft(C* s, int lstride, int nlines, int P, int logP,
 }
 
 // ------------------------------------------------------------------------
-// Register-resident line FFT.  A line of length P = 2^logP (8 <= P <= 2048)
-// is held by T = P / 8 threads, thread t owning v[r] = x[t + r T].  One
-// radix-2 or radix-4 stage (when log2 P is not a multiple of 3) is followed
-// by radix-8 stages; between stages the line passes once through shared
-// memory, indexed with one pad slot per 8 entries so that the strided
-// Stockham stores spread over the banks.  The result comes back in the same
-// layout, v[r] = X[t + r T]; the last stage needs no exchange.
-__device__ __forceinline__ int pad8(int i) { return i + (i >> 3); }
+// Line FFTs of N = 2^LOGN points (8 <= N <= 1024) held by T threads of one
+// warp, E = N / T entries each, T <= E: thread t owns v[a] = x[T a + t].  The
+// transform is an E-point DFT in registers, one twiddle, one transpose
+// through shared memory inside the warp (no block barrier) and E / T T-point
+// DFTs in registers; the result has the input's layout, v[a] = X[T a + t].
+// The transposed line is stored with T + 1 slots per row, which spreads both
+// the writes (consecutive lanes) and the reads (stride T + 1) over the banks.
+template <int LOGN> struct LineCfg {
+    static constexpr int N = 1 << LOGN;
+    static constexpr int E = LOGN >= 9 ? 32 : LOGN >= 7 ? 16 : LOGN >= 5 ? 8 : 4;
+    static constexpr int T = N / E;
+    static constexpr int XCH = E * (T + 1);       // entries of a line's transpose buffer
+    static_assert(T <= E && T <= 32 && E % T == 0, "one transpose");
+};
 
-template <typename C>
-__device__ __forceinline__ void exch(C v[8], C* s, int t, int T) {
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = s[pad8(t + r * T)];
-    __syncthreads();
+// cos(pi k / 16), 0 <= k <= 8
+__host__ __device__ constexpr double cos16(int k) {
+    return k == 0 ? 1.0 : k == 1 ? 0.98078528040323044913 : k == 2 ? 0.92387953251128675613
+         : k == 3 ? 0.83146961230254523708 : k == 4 ? 0.70710678118654752440 : k == 5 ? 0.55557023301960222474
+         : k == 6 ? 0.38268343236508977173 : k == 7 ? 0.19509032201612826785 : 0.0;
+}
+__host__ __device__ constexpr double cos32(int k) {      // cos(2 pi k / 32), 0 <= k < 32
+    return k <= 8 ? cos16(k) : k <= 16 ? -cos16(16 - k) : k <= 24 ? -cos16(k - 16) : cos16(32 - k);
 }
 
-template <typename C, int LOGP>
-__device__ __forceinline__ void fft_line(C v[8], C* s, int t, const C* __restrict__ tw, int twstep, bool inv) {
-    constexpr int P = 1 << LOGP;
-    constexpr int T = P >> 3;
-    constexpr int B = 1 << (LOGP % 3);
-    int Ns = 1;
-    if (B == 2) {
-        // four radix-2 butterflies j = t + qT: inputs v[q], v[q + 4]; outputs y[2j], y[2j + 1]
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const C a = v[q], c = v[q + 4];
-            const int j = t + q * T;
-            s[pad8(2 * j)] = cadd(a, c);
-            s[pad8(2 * j + 1)] = csub(a, c);
-        }
-        exch(v, s, t, T);
-        Ns = 2;
-    } else if (B == 4) {
-        // two radix-4 butterflies j = t + qT: inputs v[q + 2r]; outputs y[4j + r]
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            C a0 = v[q], a1 = v[q + 2], a2 = v[q + 4], a3 = v[q + 6];
-            dft4(a0, a1, a2, a3, inv);
-            const int j = t + q * T;
-            s[pad8(4 * j)] = a0;
-            s[pad8(4 * j + 1)] = a1;
-            s[pad8(4 * j + 2)] = a2;
-            s[pad8(4 * j + 3)] = a3;
-        }
-        exch(v, s, t, T);
-        Ns = 4;
-    }
-    constexpr int NST = LOGP / 3;          // radix-8 stages
-#pragma unroll
-    for (int st = 0; st < NST; ++st) {
-        const int k = t & (Ns - 1);
-        if (Ns > 1) {
-            const int m = k * ((P >> 3) / Ns) * twstep;
-#pragma unroll
-            for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], twiddle(tw, r * m, inv));
-        }
-        dft8(v, inv);
-        if (st == NST - 1) break;
-        const int base = (t - k) * 8 + k;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) s[pad8(base + r * Ns)] = v[r];
-        exch(v, s, t, T);
-        Ns *= 8;
+// cos(2 pi k / 64) for odd k, 0 < k < 64 (even k: cos32)
+__host__ __device__ constexpr double cos64(int k) {
+    return k % 2 == 0 ? cos32((k / 2) % 32) : k > 32 ? cos64(64 - k) : k > 16 ? -cos64(32 - k)
+         : k == 1 ? 0.99518472667219688624 : k == 3 ? 0.95694033573220886494 : k == 5 ? 0.88192126434835502971
+         : k == 7 ? 0.77301045336273696081 : k == 9 ? 0.63439328416364549822 : k == 11 ? 0.47139673682599764856
+         : k == 13 ? 0.29028467725446236764 : 0.09801714032956060199;
+}
+
+// v times exp(-2 pi i K / 32) (forward) or its conjugate (inverse)
+template <int K, bool INV, typename C>
+__device__ __forceinline__ C rot32(C v) {
+    typedef decltype(v.x) R;
+    constexpr int k = (INV ? 32 - (K % 32) : K) % 32;
+    if constexpr (k == 0) return v;
+    else if constexpr (k == 8) return mk(v.y, -v.x);
+    else if constexpr (k == 16) return mk(-v.x, -v.y);
+    else if constexpr (k == 24) return mk(-v.y, v.x);
+    else if constexpr (k % 8 == 4) {
+        constexpr R s = (R)0.70710678118654752440;
+        if constexpr (k == 4) return mk((v.x + v.y) * s, (v.y - v.x) * s);
+        else if constexpr (k == 12) return mk((v.y - v.x) * s, -(v.x + v.y) * s);
+        else if constexpr (k == 20) return mk(-(v.x + v.y) * s, (v.x - v.y) * s);
+        else return mk((v.x - v.y) * s, (v.x + v.y) * s);
+    } else {
+        constexpr R c = (R)cos32(k), s = (R)cos32((k + 24) % 32);     // cos(x - pi/2) = sin x
+        // (x + iy)(c - is)
+        return mk(v.x * c + v.y * s, v.y * c - v.x * s);
     }
 }
+
+// rows b = 1, 2, 3 of the M / 4 entries c times w_M^(b c)
+template <int M, bool INV, int LEFT, typename C>
+__device__ __forceinline__ void rot_rows(C* y1, C* y2, C* y3) {
+    if constexpr (LEFT > 1) {
+        constexpr int c = LEFT - 1, S = 32 / M;
+        y1[c] = rot32<S * c, INV>(y1[c]);
+        y2[c] = rot32<S * 2 * c, INV>(y2[c]);
+        y3[c] = rot32<S * 3 * c, INV>(y3[c]);
+        rot_rows<M, INV, LEFT - 1>(y1, y2, y3);
+    }
+}
+
+// DFT of M entries (2, 4, 8, 16, 32) of a register array, in natural order
+template <int M, bool INV, typename C>
+__device__ __forceinline__ void reg_dft(C* v) {
+    if constexpr (M == 2) {
+        const C a = v[0];
+        v[0] = vadd(a, v[1]);
+        v[1] = vsub(a, v[1]);
+    } else if constexpr (M == 4) {
+        dft4(v[0], v[1], v[2], v[3], INV);
+    } else if constexpr (M == 8) {
+        dft8(v, INV);
+    } else {
+        // n = 4 a + b: DFT over a, twiddle w_M^(b c), DFT over b -> X[c + (M / 4) d]
+        constexpr int Q = M / 4;
+        C y[4][Q];
+#pragma unroll
+        for (int a = 0; a < Q; ++a) {
+            y[0][a] = v[4 * a];
+            y[1][a] = v[4 * a + 1];
+            y[2][a] = v[4 * a + 2];
+            y[3][a] = v[4 * a + 3];
+        }
+        reg_dft<Q, INV>(y[0]);
+        reg_dft<Q, INV>(y[1]);
+        reg_dft<Q, INV>(y[2]);
+        reg_dft<Q, INV>(y[3]);
+        rot_rows<M, INV, Q>(y[1], y[2], y[3]);
+#pragma unroll
+        for (int c = 0; c < Q; ++c) {
+            dft4(y[0][c], y[1][c], y[2][c], y[3][c], INV);
+            v[c] = y[0][c];
+            v[c + Q] = y[1][c];
+            v[c + 2 * Q] = y[2][c];
+            v[c + 3 * Q] = y[3][c];
+        }
+    }
+}
+
+// v[a] times exp(-2 pi i a / (2 M)) (forward) or its conjugate, a < M <= 32
+template <int M, bool INV, int LEFT = M, typename C>
+__device__ __forceinline__ void half_shift(C* v) {
+    if constexpr (LEFT > 1) {
+        constexpr int a = LEFT - 1;
+        if constexpr (M <= 16) {
+            v[a] = rot32<a * (16 / M), INV>(v[a]);
+        } else {
+            typedef decltype(v->x) R;
+            constexpr R c = (R)cos64(a), s = (R)cos64((a + 48) % 64);
+            v[a] = INV ? mk(v[a].x * c - v[a].y * s, v[a].y * c + v[a].x * s)
+                       : mk(v[a].x * c + v[a].y * s, v[a].y * c - v[a].x * s);
+        }
+        half_shift<M, INV, LEFT - 1>(v);
+    }
+}
+
+// The line transform.  buf: the line's transpose buffer (XCH entries, used by
+// this line's threads alone, all in one warp).  Every lane of the warp calls
+// it.  odd (the same for the whole warp): the input (forward) or the output
+// (inverse) is also multiplied by the half-sample shift w_2N^n or its
+// conjugate, n = T a + t.  Of that factor the part that depends on the
+// register index is a constant, and the part that depends on the lane
+// commutes with the register DFT next to it, so it is part of the twiddle
+// table and costs no load.  lt (line_table): w_N^(c t), w_2N^((2c + 1) t) or
+// w_2N^(c (2t + 1)) at c T + t.  Both parities run the same code but for the
+// constants: with a copy for each, the passes' code outgrew the instruction
+// cache.
+template <int LOGN, bool INV, typename C>
+__device__ __forceinline__ void line_fft(C (&v)[LineCfg<LOGN>::E], C* buf, int t, int odd, const C* __restrict__ lt) {
+    constexpr int N = LineCfg<LOGN>::N, E = LineCfg<LOGN>::E, T = LineCfg<LOGN>::T, J = E / T;
+    if (!INV && odd) half_shift<E, false>(v);
+    reg_dft<E, INV>(v);
+    const C* tw = lt + (odd ? (INV ? 2 * N : N) : 0) + t;
+#pragma unroll
+    for (int c = 0; c < E; ++c) {
+        if (c || !INV) {
+            C w = tw[c * T];
+            if (INV) w.y = -w.y;
+            v[c] = cmul(v[c], w);
+        }
+        buf[c * (T + 1) + t] = v[c];
+    }
+    __syncwarp();
+    C x[E];
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+#pragma unroll
+        for (int b = 0; b < T; ++b) x[j * T + b] = buf[(t + T * j) * (T + 1) + b];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < J; ++j) reg_dft<T, INV>(x + j * T);
+    if (INV && odd) {
+#pragma unroll
+        for (int j = 0; j < J; ++j) half_shift<T, true>(x + j * T);
+    }
+    // X[(t + T j) + E d]: entry a = j + J d of the layout T a + t
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+#pragma unroll
+        for (int d = 0; d < T; ++d) v[j + J * d] = x[j * T + d];
+}
+
+// Tables of the line transforms, N = 8 .. 1024: three of N entries each.
+__host__ __device__ constexpr int line_table(int N) { return 3 * N - 24; }   // first entry of N's tables
+constexpr int kLineTables = line_table(2048);                                // entries in all
 
 }  // namespace lsw

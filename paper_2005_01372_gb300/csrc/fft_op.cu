@@ -33,6 +33,20 @@ template <> struct FftCfg<double> { static constexpr int NT = 256, MB4 = 4; };
 // elements of one CTA's line set: nlines * P <= 4 * NT * MB4
 template <typename R> constexpr int fft_capacity() { return 4 * FftCfg<R>::NT * FftCfg<R>::MB4; }
 
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gmem), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// 16-byte accesses: two complex64 entries or one complex128
+template <typename C> struct Vec16;
+template <> struct Vec16<float2> { typedef float4 T; };
+template <> struct Vec16<double2> { typedef double2 T; };
+
 struct DevGeom {
     int bz, bx, logbz;
     const double* chi;
@@ -168,167 +182,309 @@ k_pass_c(const typename Cx<R>::T* __restrict__ T, DevGeom geo, int pz, int logpz
 }
 
 // ------------------------------------------------- register-FFT passes
-// The same three passes with register-resident radix-8 line FFTs, for
-// 8 <= 2bz, 2bx <= 2048.  Here T holds, per field, the 2bz x bx spectrum in
-// kz-blocks: the kblk rows kz = kblk j .. kblk j + kblk - 1 (64 bytes of one
-// column) lie next to each other for ix = 0, 1, ..., bx - 1, and the blocks
-// follow each other.  A column's write (pass A) and read (pass C) then move
-// whole 64-byte segments, and pass B reads and writes every kz-block as one
-// contiguous run.
+// The same three passes with register-resident line FFTs, for box sides of
+// 8 .. 1024 cells.  A line of N cells zero-padded to 2N has the spectrum
+//   X[2k] = DFT_N(x)[k],   X[2k + 1] = DFT_N(x w_2N^n)[k],
+// and the first N entries of an inverse transform of length 2N are
+//   y[n] = IDFT_N(Y[even])[n] + conj(w_2N^n) IDFT_N(Y[odd])[n],
+// so the padding costs no butterfly: the two halves (parities) of a line are
+// N-point transforms, run by two thread groups of T threads (LineCfg) that
+// meet only where their results are added.
+//
+// T holds, per field, the rows kz' = parity * bz + k (kz = 2k + parity) in
+// blocks: kblk rows (64 bytes of one column) lie next to each other for
+// ix = 0, 1, ..., bx - 1, and the blocks follow each other.  A column's write
+// (pass A) and read (pass C) move whole 64-byte segments, and pass B reads
+// and writes its rows of a block in runs of at least 32 bytes.
+//
+// What bounds them: shared-memory wavefronts (63% of peak in pass B) and FP32
+// issue, at the 16 - 32 warps the registers leave; FP64 is bound by its pipe
+// (85% busy).  A line's transform moves every entry twice through shared
+// memory (one transpose, inside a warp) where the radix-8 passes these
+// replaced moved it six times with two block barriers each.  RESIDUAL on one
+// GB300, before -> now: 256^2, 32 fields 95 -> 55 us; 1024^2, 16 fields 1098 ->
+// 539 us; ADJOINT 256 x 1024, 30 fields 487 -> 216 us; FP64 256^2, 32 fields
+// 1401 -> 1352 us.
 template <typename C> __host__ __device__ constexpr int kblk() { return 64 / (int)sizeof(C); }
 template <typename C> __device__ __forceinline__ long long tile_index(int kz, int ix, int bx) {
     constexpr int KB = kblk<C>();
     return (long long)(kz / KB) * bx * KB + (long long)ix * KB + (kz % KB);
 }
-template <typename R, int LOGP>
-__global__ void __launch_bounds__(256)
-k_fa(const typename Cx<R>::T* __restrict__ u, DevGeom geo, const typename Cx<R>::T* __restrict__ tw,
-     int twstep, int adjoint, typename Cx<R>::T* __restrict__ T) {
+// entries between the buffers of two lines: the transpose buffer and, in pass
+// B, a row, rounded so that the transposing stores of 2 (c64: pairs) or 1
+// (c128) rows per lane fall into different banks
+template <typename C, int LOGN, int ROWS> __host__ __device__ constexpr int line_stride() {
+    constexpr int need = LineCfg<LOGN>::XCH > LineCfg<LOGN>::N ? LineCfg<LOGN>::XCH : LineCfg<LOGN>::N;
+    constexpr int want = sizeof(C) == 16 ? 2 : ROWS >= kblk<C>() ? 10 : 4, mod = sizeof(C) == 16 ? 8 : 16;
+    return need + ((want - need) % mod + mod) % mod;
+}
+// A line's two halves after the inverse transforms: group par keeps the
+// entries a = par E / 2 .. of the sum (v[0 .. E / 2)), handing the others to
+// its partner (buffer `other`) in its own buffer.  Called by the whole CTA.
+template <int LOGN, typename C>
+__device__ __forceinline__ void add_parities(C (&v)[LineCfg<LOGN>::E], C* buf, const C* other, int t, int par) {
+    constexpr int E = LineCfg<LOGN>::E, T = LineCfg<LOGN>::T, EH = E / 2;
+    if (par) {
+#pragma unroll
+        for (int a = 0; a < EH; ++a) buf[T * a + t] = v[a];
+    } else {
+#pragma unroll
+        for (int a = EH; a < E; ++a) buf[T * a + t] = v[a];
+    }
+    __syncthreads();
+    if (par) {
+#pragma unroll
+        for (int a = 0; a < EH; ++a) v[a] = cadd(other[T * (EH + a) + t], v[EH + a]);
+    } else {
+#pragma unroll
+        for (int a = 0; a < EH; ++a) v[a] = cadd(v[a], other[T * a + t]);
+    }
+}
+// T is read and written past L1 (every sector is used once per pass; L1 is
+// left to the twiddles), u0 and y evict first from L2, where T is to stay.
+constexpr int kFftThreads = 256;
+// launch bounds: CTAs per SM the registers are to allow (E complex entries
+// and about as many temporaries per thread, more in pass B)
+template <typename R, int LOGN, bool PASS_B> constexpr int fft_ctas() {
+    return sizeof(R) == 8 ? (LineCfg<LOGN>::E == 32 ? 1 : 2)
+                          : (LineCfg<LOGN>::E == 32 ? 2 : LineCfg<LOGN>::E == 16 && PASS_B ? 3 : 4);
+}
+
+// Pass A: a CTA takes COLS columns of `per` consecutive fields.  chi is kept
+// as R in shared memory for all of them: the FP64 -> FP32 conversion runs on
+// the FP64 pipe (2 lanes per SM and cycle) and was 42% of its time when both
+// parity groups converted every cell of every field.
+// Programmatic dependent launch: the passes follow each other on one stream,
+// and each is launched while its predecessor still runs.  A pass lets its
+// successor's CTAs start as soon as all of its own have, and touches nothing
+// an earlier kernel writes (or writes anything one reads) before
+// pdl_wait(), which returns once the whole preceding grid has finished.
+__device__ __forceinline__ void pdl_start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename R, int LOGN>
+__global__ void __launch_bounds__(kFftThreads, (fft_ctas<R, LOGN, false>()))
+k_fa(const typename Cx<R>::T* __restrict__ u, DevGeom geo, const typename Cx<R>::T* __restrict__ lt, int adjoint,
+     typename Cx<R>::T* __restrict__ T_, int nbatch, int per) {
     typedef typename Cx<R>::T C;
+    typedef LineCfg<LOGN> L;
+    constexpr int N = L::N, E = L::E, T = L::T, COLS = kFftThreads / (2 * T);
+    constexpr int LS = line_stride<C, LOGN, kblk<C>()>();
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    constexpr int pz = 1 << LOGP, Tz = pz >> 3, lpc = 256 / Tz;
-    const int l = threadIdx.x / Tz, t = threadIdx.x - l * Tz;
-    C* s = reinterpret_cast<C*>(sm_raw) + l * (pad8(pz) + 1);
-    const int b = blockIdx.y;
-    const int ix = blockIdx.x * lpc + l;
+    const int t = threadIdx.x % T, line = threadIdx.x / T;
+    const int par = line / COLS, l = line - par * COLS;
+    C* buf = reinterpret_cast<C*>(sm_raw) + line * LS;
+    R* chs = reinterpret_cast<R*>(reinterpret_cast<C*>(sm_raw) + 2 * COLS * LS);    // COLS x N
+    const int ix0 = blockIdx.x * COLS, ix = ix0 + l;
     const bool valid = ix < geo.bx;
-    const int2 org = box_origin(geo, b);
-    const C* ub = u + (long long)b * geo.bz * geo.bx + (long long)ix * geo.bz;
-    C v[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int iz = t + r * Tz;
-        C x = czero<C>();
-        if (valid && iz < geo.bz) {
-            x = ub[iz];
-            if (adjoint) {
-                x.y = -x.y;
-            } else {
-                const R ch = (R)geo.chi[(long long)(org.y + ix) * geo.chi_ld + org.x + iz];
-                x = cscale(x, ch);
+    const int b0 = blockIdx.y * per, b1 = min(nbatch, b0 + per);
+    pdl_start_next();
+    pdl_wait();
+    int box = -1;
+    for (int b = b0; b < b1; ++b) {
+        if (!adjoint && (geo.origin ? b / geo.vpb : 0) != box) {
+            box = geo.origin ? b / geo.vpb : 0;
+            const int2 org = box_origin(geo, b);
+            if (b != b0) __syncthreads();
+#pragma unroll 4
+            for (int e = threadIdx.x; e < COLS * N; e += kFftThreads) {
+                const int c = e / N, iz = e % N;
+                if (ix0 + c < geo.bx) chs[e] = (R)geo.chi[(long long)(org.y + ix0 + c) * geo.chi_ld + org.x + iz];
             }
+            __syncthreads();
         }
-        v[r] = x;
-    }
-    fft_line<C, LOGP>(v, s, t, tw, twstep, false);
-    if (valid) {
-        C* Tb = T + (long long)b * pz * geo.bx;
+        const C* ub = u + ((long long)b * geo.bx + (valid ? ix : 0)) * N;
+        C v[E];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) Tb[tile_index<C>(t + r * Tz, ix, geo.bx)] = v[r];
+        for (int a = 0; a < E; ++a) v[a] = ub[T * a + t];
+        if (adjoint) {
+#pragma unroll
+            for (int a = 0; a < E; ++a) v[a].y = -v[a].y;
+        } else {
+#pragma unroll
+            for (int a = 0; a < E; ++a) v[a] = cscale(v[a], chs[l * N + T * a + t]);
+        }
+        line_fft<LOGN, false>(v, buf, t, par, lt);
+        if (valid) {
+            C* Tb = T_ + (long long)b * 2 * N * geo.bx;
+#pragma unroll
+            for (int a = 0; a < E; ++a) __stcg(Tb + tile_index<C>(par * N + T * a + t, ix, geo.bx), v[a]);
+        }
     }
 }
 
-// Pass B on kz-blocks.  A CTA owns nblk consecutive kz-blocks of one field
-// (kblk rows each): it reads them as one contiguous run of memory, turns them
-// into rows of a shared-memory tile (odd row stride), runs the x transforms
-// of RC rows at a time (Tx threads per row, register radix-8 lines), and
-// writes the run back.  Rows past the field's last kz-block are transformed
-// as zeros and not stored, so every thread meets every barrier.
-template <typename R, int LOGP, int NTB>
-__global__ void __launch_bounds__(NTB)
-k_fb(typename Cx<R>::T* __restrict__ T, int pz, int nblk, const typename Cx<R>::T* __restrict__ spt,
-     const typename Cx<R>::T* __restrict__ tw, int twstep) {
+// Pass B: a CTA takes ROWS consecutive rows kz' of one field, turns them into
+// rows of a shared-memory tile, and two groups of T threads per row transform,
+// multiply by the spectrum and transform back one parity each; the odd group
+// hands its half over in shared memory.  The even group's transposes reuse the
+// row itself, once both groups have read it.  Rows past the field's end are
+// transformed as they lie in shared memory and not stored.
+template <typename R, int LOGN, int NTB>
+__global__ void __launch_bounds__(NTB, (NTB == 256 ? fft_ctas<R, LOGN, true>() : 1))
+k_fb(typename Cx<R>::T* __restrict__ T_, int bz, const typename Cx<R>::T* __restrict__ spt,
+     const typename Cx<R>::T* __restrict__ lt) {
     typedef typename Cx<R>::T C;
+    typedef LineCfg<LOGN> L;
+    constexpr int N = L::N, E = L::E, T = L::T, ROWS = NTB / (2 * T), KB = kblk<C>();
+    constexpr int RB = ROWS < KB ? ROWS : KB;           // rows of one kz-block in this CTA
+    constexpr int PK = sizeof(C) == 16 ? 1 : 2;         // rows per 16-byte access
+    constexpr int LS = line_stride<C, LOGN, ROWS>();
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    constexpr int px = 1 << LOGP, bx = px >> 1, Tx = px >> 3, RC = NTB / Tx;
-    constexpr int KB = kblk<C>();
-    constexpr int TS = bx + 1;                                   // odd: transposing stores spread over banks
-    C* tile = reinterpret_cast<C*>(sm_raw);                      // nblk * KB rows of TS
-    const int l = threadIdx.x / Tx, t = threadIdx.x - l * Tx;
-    C* s = tile + (size_t)nblk * KB * TS + (size_t)l * (pad8(px) + 1);
-    const int b = blockIdx.y;
-    const int kb0 = blockIdx.x * nblk;
-    const int nb = min(nblk, pz / KB - kb0);                     // kz-blocks of this CTA
-    const int nrows = nb * KB;
-    C* run = T + (long long)b * pz * bx + (long long)kb0 * bx * KB;
-    const int nrun = nrows * bx;
-    for (int e = threadIdx.x; e < nrun; e += NTB) {
-        const int blk = e / (bx * KB), w = e - blk * (bx * KB);
-        const int ix = w / KB, r = w - ix * KB;
-        tile[(blk * KB + r) * TS + ix] = run[e];
+    C* tile = reinterpret_cast<C*>(sm_raw);             // ROWS rows, then ROWS buffers of the odd groups
+    C* spec = tile + 2 * ROWS * LS;                     // the rows' spectra, N + 1 entries each
+    const int row0 = blockIdx.x * ROWS, pz = 2 * bz;
+    const int nrun = (min(ROWS, pz - row0) / PK) * N;   // 16-byte accesses
+    C* Tb = T_ + (long long)blockIdx.y * pz * N;
+    // access e: rows r, r + 1 (c128: r) of kz-block blk at ix
+    auto where = [&](int e, int& r, int& ix) -> C* {
+        const int rp = e % (RB / PK), q = e / (RB / PK);
+        const int blk = q / N;
+        ix = q - blk * N;
+        r = blk * KB + rp * PK;
+        return Tb + ((long long)(row0 / KB + blk) * N + ix) * KB + (row0 % KB) + rp * PK;
+    };
+    // the spectra arrive asynchronously behind the rows
+    for (int r = threadIdx.x >> 5; r < ROWS; r += NTB / 32) {
+        // kz = 2k + (kz parity) of row kz'; the spectrum's row holds the even
+        // qx (N / 2 + 1 entries) and then the odd ones
+        const int kr = min(row0 + r, pz - 1);
+        const int kz = kr < bz ? 2 * kr : 2 * (kr - bz) + 1;
+        const C* sp = spt + (long long)min(kz, pz - kz) * (N + 1);
+        for (int e = threadIdx.x & 31; e <= N; e += 32) cp_async<sizeof(C)>(spec + r * (N + 1) + e, sp + e);
     }
-    __syncthreads();
-    const int rows_all = nblk * KB;
-    for (int r0 = 0; r0 < rows_all; r0 += RC) {
-        const int row = r0 + l;
-        const bool live = row < nrows;
-        const int kz = kb0 * KB + row;
-        C v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int kx = t + q * Tx;
-            v[q] = (live && kx < bx) ? tile[row * TS + kx] : czero<C>();
-        }
-        fft_line<C, LOGP>(v, s, t, tw, twstep, false);
-        const int qzz = live ? min(kz, pz - kz) : 0;
-        const C* sp = spt + (long long)qzz * (bx + 1);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int kx = t + q * Tx;
-            v[q] = cmul(v[q], sp[min(kx, px - kx)]);
-        }
-        fft_line<C, LOGP>(v, s, t, tw, twstep, true);
-        if (live) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int kx = t + q * Tx;
-                if (kx < bx) tile[row * TS + kx] = v[q];
-            }
+    pdl_start_next();
+    pdl_wait();
+#pragma unroll 8
+    for (int e = threadIdx.x; e < nrun; e += NTB) {
+        int r, ix;
+        const C* p = where(e, r, ix);
+        const auto w = __ldcg(reinterpret_cast<const typename Vec16<C>::T*>(p));
+        if constexpr (PK == 2) {
+            tile[r * LS + ix] = mk(w.x, w.y);
+            tile[(r + 1) * LS + ix] = mk(w.z, w.w);
+        } else {
+            tile[r * LS + ix] = w;
         }
     }
     __syncthreads();
+    const int t = threadIdx.x % T, line = threadIdx.x / T;
+    const int par = line / ROWS, row = line - par * ROWS;
+    C* rowp = tile + row * LS;
+    C* buf = tile + line * LS;
+    C v[E];
+#pragma unroll
+    for (int a = 0; a < E; ++a) v[a] = rowp[T * a + t];
+    cp_async_wait_all();
+    __syncthreads();
+    line_fft<LOGN, false>(v, buf, t, par, lt);
+    const C* sp = spec + row * (N + 1) + par * (N / 2 + 1);
+#pragma unroll
+    for (int a = 0; a < E; ++a) v[a] = cmul(v[a], sp[min(T * a + t, N - par - (T * a + t))]);
+    line_fft<LOGN, true>(v, buf, t, par, lt);
+    add_parities<LOGN>(v, buf, buf + (par ? -ROWS * LS : ROWS * LS), t, par);
+    // both groups' halves of the row
+    constexpr int EH = E / 2;
+#pragma unroll
+    for (int a = 0; a < EH; ++a) rowp[T * (par * EH + a) + t] = v[a];
+    __syncthreads();
+#pragma unroll 8
     for (int e = threadIdx.x; e < nrun; e += NTB) {
-        const int blk = e / (bx * KB), w = e - blk * (bx * KB);
-        const int ix = w / KB, r = w - ix * KB;
-        run[e] = tile[(blk * KB + r) * TS + ix];
+        int r, ix;
+        C* p = where(e, r, ix);
+        typename Vec16<C>::T w;
+        if constexpr (PK == 2) {
+            const C w0 = tile[r * LS + ix], w1 = tile[(r + 1) * LS + ix];
+            w.x = w0.x; w.y = w0.y; w.z = w1.x; w.w = w1.y;
+        } else {
+            w = tile[r * LS + ix];
+        }
+        __stcg(reinterpret_cast<typename Vec16<C>::T*>(p), w);
     }
 }
 
-template <typename R, int LOGP>
-__global__ void __launch_bounds__(256)
-k_fc(const typename Cx<R>::T* __restrict__ T, DevGeom geo, const typename Cx<R>::T* __restrict__ tw,
-     int twstep, int mode, const typename Cx<R>::T* __restrict__ u, const typename Cx<R>::T* __restrict__ u0,
+template <typename R, int LOGN>
+__global__ void __launch_bounds__(kFftThreads, (fft_ctas<R, LOGN, false>()))
+k_fc(const typename Cx<R>::T* __restrict__ T_, DevGeom geo, const typename Cx<R>::T* __restrict__ lt, int mode,
+     const typename Cx<R>::T* __restrict__ u, const typename Cx<R>::T* __restrict__ u0,
      typename Cx<R>::T* __restrict__ y) {
     typedef typename Cx<R>::T C;
+    typedef LineCfg<LOGN> L;
+    constexpr int N = L::N, E = L::E, T = L::T, COLS = kFftThreads / (2 * T);
+    constexpr int LS = line_stride<C, LOGN, kblk<C>()>();
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    constexpr int pz = 1 << LOGP, Tz = pz >> 3, lpc = 256 / Tz;
-    const int l = threadIdx.x / Tz, t = threadIdx.x - l * Tz;
-    C* s = reinterpret_cast<C*>(sm_raw) + l * (pad8(pz) + 1);
-    const int b = blockIdx.y;
-    const int ix = blockIdx.x * lpc + l;
+    const int t = threadIdx.x % T, line = threadIdx.x / T;
+    const int par = line / COLS, l = line - par * COLS;
+    C* buf = reinterpret_cast<C*>(sm_raw) + line * LS;
+    const int b = blockIdx.y, ix = blockIdx.x * COLS + l;
     const bool valid = ix < geo.bx;
-    const C* Tb = T + (long long)b * pz * geo.bx;
-    C v[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = valid ? Tb[tile_index<C>(t + r * Tz, ix, geo.bx)] : czero<C>();
-    fft_line<C, LOGP>(v, s, t, tw, twstep, true);
-    if (!valid) return;
-    const int2 org = box_origin(geo, b);
-    const long long base = (long long)b * geo.bz * geo.bx + (long long)ix * geo.bz;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int iz = t + r * Tz;
-        if (iz >= geo.bz) continue;
-        const long long idx = base + iz;
-        const C g = v[r];
-        C out;
-        switch (mode) {
-            case LSW_OP_FORWARD:
-                out = u0 ? cadd(u0[idx], g) : g;
-                break;
-            case LSW_OP_RESIDUAL:
-                out = csub(u[idx], g);
-                if (u0) out = csub(out, u0[idx]);
-                break;
-            case LSW_OP_ADJOINT: {
-                const R ch = (R)geo.chi[(long long)(org.y + ix) * geo.chi_ld + org.x + iz];
-                out = mk(g.x * ch, -g.y * ch);
-                break;
-            }
-            default:
-                out = g;
+    const C* Tb = T_ + (long long)b * 2 * N * geo.bx;
+    pdl_start_next();
+    pdl_wait();
+    if (valid && (mode == LSW_OP_RESIDUAL || mode == LSW_OP_FORWARD)) {
+        // the fields this half of the column is combined with: into L2 while
+        // the transform runs
+        const long long lo = ((long long)b * geo.bx + ix) * N + par * (N / 2);
+        for (int i = t * (128 / (int)sizeof(C)); i < N / 2; i += T * (128 / (int)sizeof(C))) {
+            if (mode == LSW_OP_RESIDUAL) prefetch_l2(u + lo + i);
+            if (u0) prefetch_l2(u0 + lo + i);
         }
-        y[idx] = out;
+    }
+    C v[E];
+#pragma unroll
+    for (int a = 0; a < E; ++a) v[a] = __ldcg(Tb + tile_index<C>(par * N + T * a + t, valid ? ix : 0, geo.bx));
+    line_fft<LOGN, true>(v, buf, t, par, lt);
+    add_parities<LOGN>(v, buf, buf + (par ? -COLS * LS : COLS * LS), t, par);
+    if (!valid) return;
+    // entry a of this group's half lies at off + T a; the fields it is
+    // combined with are all loaded before the first is used
+    constexpr int EH = E / 2;
+    const int iz0 = par * EH * T + t;
+    const long long off = ((long long)b * geo.bx + ix) * N + iz0;
+    if (mode == LSW_OP_RESIDUAL) {
+        C x[EH];
+#pragma unroll
+        for (int a = 0; a < EH; ++a) x[a] = __ldcs(u + off + T * a);
+#pragma unroll
+        for (int a = 0; a < EH; ++a) v[a] = csub(x[a], v[a]);
+        if (u0) {
+#pragma unroll
+            for (int a = 0; a < EH; ++a) x[a] = __ldcs(u0 + off + T * a);
+#pragma unroll
+            for (int a = 0; a < EH; ++a) v[a] = csub(v[a], x[a]);
+        }
+    } else if (mode == LSW_OP_FORWARD) {
+        if (u0) {
+            C x[EH];
+#pragma unroll
+            for (int a = 0; a < EH; ++a) x[a] = __ldcs(u0 + off + T * a);
+#pragma unroll
+            for (int a = 0; a < EH; ++a) v[a] = cadd(x[a], v[a]);
+        }
+    } else if (mode == LSW_OP_ADJOINT) {
+        const int2 org = box_origin(geo, b);
+        const double* ch = geo.chi + (long long)(org.y + ix) * geo.chi_ld + org.x + iz0;
+        R x[EH];
+#pragma unroll
+        for (int a = 0; a < EH; ++a) x[a] = (R)ch[T * a];
+#pragma unroll
+        for (int a = 0; a < EH; ++a) v[a] = mk(v[a].x * x[a], -v[a].y * x[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < EH; ++a) __stcs(y + off + T * a, v[a]);
+}
+
+// line twiddles and half-sample shifts of every line length (line_table)
+__global__ void k_line_tables(double2* t64, float2* t32) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kLineTables; e += gridDim.x * blockDim.x) {
+        int N = 8;
+        while (line_table(2 * N) <= e) N *= 2;
+        const int E = N >= 512 ? 32 : N >= 128 ? 16 : N >= 32 ? 8 : 4, T = N / E;      // LineCfg
+        const int i = e - line_table(N);
+        double s, c;
+        const int which = i / N, cc = (i - which * N) / T, t = i % T;
+        sincospi(-(double)(which == 0 ? 2 * cc * t : which == 1 ? (2 * cc + 1) * t : cc * (2 * t + 1)) / N, &s, &c);
+        t64[e] = make_double2(c, s);
+        t32[e] = make_float2((float)c, (float)s);
     }
 }
 
@@ -402,8 +558,10 @@ __global__ void k_quarter(const double2* __restrict__ F, int bz, int bx, double2
         const float2 f = make_float2((float)w.x, (float)w.y);
         q64[e] = w;
         q32[e] = f;
-        t64[qz * (bx + 1) + qx] = w;
-        t32[qz * (bx + 1) + qx] = f;
+        // kz-major rows: the even qx, then the odd ones
+        const int p = qz * (bx + 1) + ((qx & 1) ? bx / 2 + 1 : 0) + (qx >> 1);
+        t64[p] = w;
+        t32[p] = f;
     }
 }
 
@@ -440,8 +598,6 @@ __global__ void k_point_sources(const double2* __restrict__ table, int nz, int n
     }
 }
 
-inline size_t pad8h(int i) { return (size_t)i + (size_t)(i >> 3); }
-
 // Algorithmic bytes of one batched apply: per field read u (and u0) and
 // write y; chi (FP64) and the quarter spectrum once per batch.
 double op_bytes(size_t elem, int bz, int bx, int nb, bool has_u0, int) {
@@ -467,7 +623,7 @@ int grid_for(long long n, int bs = 256) {
 template <typename K>
 lsw_status set_smem(K k, std::atomic<bool>& done) {
     if (!done) {
-        LSW_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
+        LSW_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
         done = true;
     }
     return LSW_OK;
@@ -483,44 +639,75 @@ lsw_status set_smem(K k, std::atomic<bool>& done) {
         case 8: { constexpr int L_ = 8; __VA_ARGS__; break; }   \
         case 9: { constexpr int L_ = 9; __VA_ARGS__; break; }   \
         case 10: { constexpr int L_ = 10; __VA_ARGS__; break; } \
-        case 11: { constexpr int L_ = 11; __VA_ARGS__; break; } \
         default: return LSW_ERR_UNSUPPORTED_SIZE;        \
     }
 
+template <typename K, typename... A>
+lsw_status launch_pdl(K k, dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    LSW_CUDA(cudaLaunchKernelEx(&cfg, k, args...));
+    LSW_LAUNCH_CHECK();
+    return LSW_OK;
+}
+
+// log2 box sides lz, lx: 3 .. 10
 template <typename R>
-lsw_status launch_fa(int lg, dim3 grid, size_t sm, cudaStream_t st, const typename Cx<R>::T* u, DevGeom dg,
-                     const typename Cx<R>::T* tw, int tws, int adj, typename Cx<R>::T* work) {
-    static std::atomic<bool> done[12];
-    LSW_LOG_SWITCH(lg, {
+lsw_status launch_fa(int lz, int nbatch, cudaStream_t st, const typename Cx<R>::T* u, const DevGeom& dg,
+                     const typename Cx<R>::T* tab, int adj, typename Cx<R>::T* work) {
+    typedef typename Cx<R>::T C;
+    static std::atomic<bool> done[11];
+    LSW_LOG_SWITCH(lz, {
+        constexpr int lines = kFftThreads / LineCfg<L_>::T, cols = lines / 2;
         LSW_TRY(set_smem(k_fa<R, L_>, done[L_]));
-        k_fa<R, L_><<<grid, 256, sm, st>>>(u, dg, tw, tws, adj, work);
-        LSW_LAUNCH_CHECK();
+        // fields per CTA: up to 4 while about four CTAs per SM slot remain
+        const int gx = (dg.bx + cols - 1) / cols;
+        const int per = std::max(1, std::min(4, (int)((long long)gx * nbatch / (152 * 8))));
+        LSW_TRY(launch_pdl(k_fa<R, L_>, dim3(gx, (nbatch + per - 1) / per), kFftThreads,
+                           sizeof(C) * lines * line_stride<C, L_, kblk<C>()>() + sizeof(R) * cols * LineCfg<L_>::N, st,
+                           u, dg, tab + line_table(1 << L_), adj, work, nbatch, per));
     })
     return LSW_OK;
 }
+
+// 512 threads: twice the rows, where they fit in shared memory and registers
+template <typename R, int LOGN> constexpr bool fb_wide() { return sizeof(R) == 4 || LineCfg<LOGN>::E < 32; }
 
 template <typename R, int NTB>
-lsw_status launch_fb(int lg, dim3 grid, size_t sm, cudaStream_t st, typename Cx<R>::T* work, int pz, int nblk,
-                     const typename Cx<R>::T* spt, const typename Cx<R>::T* tw, int tws) {
-    static std::atomic<bool> done[12];
-    LSW_LOG_SWITCH(lg, {
-        if (L_ < 4 && NTB > 256) return LSW_ERR_UNSUPPORTED_SIZE;
-        LSW_TRY(set_smem(k_fb<R, L_, NTB>, done[L_]));
-        k_fb<R, L_, NTB><<<grid, NTB, sm, st>>>(work, pz, nblk, spt, tw, tws);
-        LSW_LAUNCH_CHECK();
+lsw_status launch_fb(int lx, int bz, int nbatch, cudaStream_t st, typename Cx<R>::T* work,
+                     const typename Cx<R>::T* spt, const typename Cx<R>::T* tab) {
+    typedef typename Cx<R>::T C;
+    static std::atomic<bool> done[11];
+    LSW_LOG_SWITCH(lx, {
+        constexpr int NT = fb_wide<R, L_>() ? NTB : 256, rows = NT / (2 * LineCfg<L_>::T);
+        LSW_TRY(set_smem(k_fb<R, L_, NT>, done[L_]));
+        LSW_TRY(launch_pdl(k_fb<R, L_, NT>, dim3((2 * bz + rows - 1) / rows, nbatch), NT,
+                           sizeof(C) * rows * (2 * line_stride<C, L_, rows>() + LineCfg<L_>::N + 1), st, work, bz, spt,
+                           tab + line_table(1 << L_)));
     })
     return LSW_OK;
 }
 
 template <typename R>
-lsw_status launch_fc(int lg, dim3 grid, size_t sm, cudaStream_t st, const typename Cx<R>::T* work, DevGeom dg,
-                     const typename Cx<R>::T* tw, int tws, int mode, const typename Cx<R>::T* u,
-                     const typename Cx<R>::T* u0, typename Cx<R>::T* y) {
-    static std::atomic<bool> done[12];
-    LSW_LOG_SWITCH(lg, {
+lsw_status launch_fc(int lz, int nbatch, cudaStream_t st, const typename Cx<R>::T* work, const DevGeom& dg,
+                     const typename Cx<R>::T* tab, int mode, const typename Cx<R>::T* u, const typename Cx<R>::T* u0,
+                     typename Cx<R>::T* y) {
+    typedef typename Cx<R>::T C;
+    static std::atomic<bool> done[11];
+    LSW_LOG_SWITCH(lz, {
+        constexpr int lines = kFftThreads / LineCfg<L_>::T, cols = lines / 2;
         LSW_TRY(set_smem(k_fc<R, L_>, done[L_]));
-        k_fc<R, L_><<<grid, 256, sm, st>>>(work, dg, tw, tws, mode, u, u0, y);
-        LSW_LAUNCH_CHECK();
+        LSW_TRY(launch_pdl(k_fc<R, L_>, dim3((dg.bx + cols - 1) / cols, nbatch), kFftThreads,
+                           sizeof(C) * lines * line_stride<C, L_, kblk<C>()>(), st, work, dg, tab + line_table(1 << L_),
+                           mode, u, u0, y));
     })
     return LSW_OK;
 }
@@ -567,26 +754,16 @@ lsw_status op_apply(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, i
     DevGeom dg{bz, bx, ilog2(bz), geo.chi, geo.chi_ld, geo.origin, geo.vpb > 0 ? geo.vpb : 1};
     const int logpz = ilog2(pz), logpx = ilog2(px);
     const int variant = op_variant(pz, px, (int)sizeof(R));
-    if (variant != 2 && pz >= 8 && px >= 8 && pz <= 2048 && px <= 2048 && sp.t32 && sp.t64) {
+    if (variant != 2 && bz >= 8 && bx >= 8 && bz <= 1024 && bx <= 1024 && sp.t32 && sp.t64) {
         const C* spt = reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)sp.t64 : (const void*)sp.t32);
-        const int ntb = (variant == 1 && px >= 16) ? 512 : 256;
-        const int lz = 256 / (pz >> 3), lx = ntb / (px >> 3);
-        const size_t smA = sizeof(C) * (size_t)lz * (pad8h(pz) + 1);
-        // pass B: kz-blocks per CTA so that a CTA holds >= lx rows and about
-        // 4096 entries, within the field's pz / kblk blocks
-        constexpr int KB = kblk<C>();
-        const int nkb = pz / KB;
-        int nblk = std::max((lx + KB - 1) / KB, 4096 / (KB * bx));
-        nblk = std::max(1, std::min(nblk, nkb));
-        const size_t smB = sizeof(C) * ((size_t)nblk * KB * (bx + 1) + (size_t)lx * (pad8h(px) + 1));
-        const int twz = g->twP / pz, twx = g->twP / px;
-        dim3 gA((bx + lz - 1) / lz, nbatch), gB((nkb + nblk - 1) / nblk, nbatch);
+        const C* tab = reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)g->lt64 : (const void*)g->lt32);
         KTimer kt(sizeof(R) == 8 ? "operator_c128" : "operator_c64", st, op_bytes(sizeof(C), bz, bx, nbatch, u0 != nullptr, mode),
                   op_flops(bz, bx, nbatch));
-        LSW_TRY(launch_fa<R>(logpz, gA, smA, st, u, dg, tw, twz, mode == LSW_OP_ADJOINT, work));
-        if (ntb == 512) LSW_TRY((launch_fb<R, 512>(logpx, gB, smB, st, work, pz, nblk, spt, tw, twx)));
-        else LSW_TRY((launch_fb<R, 256>(logpx, gB, smB, st, work, pz, nblk, spt, tw, twx)));
-        LSW_TRY(launch_fc<R>(logpz, gA, smA, st, work, dg, tw, twz, mode, u, u0, y));
+        const int lz = logpz - 1, lx = logpx - 1;
+        LSW_TRY(launch_fa<R>(lz, nbatch, st, u, dg, tab, mode == LSW_OP_ADJOINT, work));
+        if (variant == 1) LSW_TRY((launch_fb<R, 512>(lx, bz, nbatch, st, work, spt, tab)));
+        else LSW_TRY((launch_fb<R, 256>(lx, bz, nbatch, st, work, spt, tab)));
+        LSW_TRY(launch_fc<R>(lz, nbatch, st, work, dg, tab, mode, u, u0, y));
         return LSW_OK;
     }
     // columns per CTA for passes A and C, rows per CTA for pass B
@@ -686,6 +863,10 @@ lsw_status green_init(lsw_green* g, cudaStream_t st) {
     LSW_CUDA(cudaMalloc(&g->tw64, g->twP * sizeof(double2)));
     LSW_CUDA(cudaMalloc(&g->tw32, g->twP * sizeof(float2)));
     k_twiddles<<<grid_for(g->twP), 256, 0, st>>>(g->tw64, g->tw32, g->twP);
+    LSW_LAUNCH_CHECK();
+    LSW_CUDA(cudaMalloc(&g->lt64, kLineTables * sizeof(double2)));
+    LSW_CUDA(cudaMalloc(&g->lt32, kLineTables * sizeof(float2)));
+    k_line_tables<<<grid_for(kLineTables), 256, 0, st>>>(g->lt64, g->lt32);
     LSW_LAUNCH_CHECK();
     LSW_TRY(build_spectrum(g, g->nz, g->nx, &g->full, st));
     LSW_CUDA(cudaStreamSynchronize(st));
