@@ -33,14 +33,6 @@ template <> struct FftCfg<double> { static constexpr int NT = 256, MB4 = 4; };
 // elements of one CTA's line set: nlines * P <= 4 * NT * MB4
 template <typename R> constexpr int fft_capacity() { return 4 * FftCfg<R>::NT * FftCfg<R>::MB4; }
 
-template <int BYTES>
-__device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gmem), "n"(BYTES) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // 16-byte accesses: two complex64 entries or one complex128
 template <typename C> struct Vec16;

@@ -1,6 +1,7 @@
 // Fourier neural operator used as a learned right preconditioner: forward,
 // backward (G = dL/dRe + i dL/dIm convention), Adam, and the preconditioner
-// apply, all in FP32 complex on the library's batched GEMMs.
+// apply, all in FP32 complex: fused passes (fno_passes.cuh) and the library's
+// batched GEMMs.
 //
 // Network (complex): v = P x + p;  v <- sigma(K_l v + W_l v + b_l) for
 // l < L (no sigma on the last layer);  y = x0 + Q v + q.  K_l keeps the 2m x 2m
@@ -16,11 +17,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <new>
 #include <vector>
 
+#include "fno_passes.cuh"
 #include "lsw_internal.cuh"
 
 struct lsw_fno {
@@ -35,6 +38,9 @@ struct lsw_fno {
     float2* Fz = nullptr;        // M x nz   rows of the DFT
     float2* FxT = nullptr;       // nx x M   (F_x)^T
     float2* Fxc = nullptr;       // M x nx   conj(F_x)
+    bool fast = false;           // truncated transforms by register DFTs (fno_passes.cuh)
+    float2* twz = nullptr;       // their line twiddles, nz and nx entries
+    float2* twx = nullptr;
     // offsets into params
     long long oPT, op, oQT, oq;
     std::vector<long long> oR, oWT, ob;
@@ -50,11 +56,6 @@ int gridn(long long n, int bs = 256) {
 
 __host__ __device__ inline float2 c1() { return make_float2(1.f, 0.f); }
 __host__ __device__ inline float2 c0() { return make_float2(0.f, 0.f); }
-
-__device__ __forceinline__ float gelu_f(float t) { return t * 0.5f * (1.f + erff(t * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_g(float t) {
-    return 0.5f * (1.f + erff(t * 0.70710678118654752f)) + t * expf(-0.5f * t * t) * 0.3989422804014327f;
-}
 
 // rows of the DFT for the retained wavenumbers: F[a][i] = exp(-2 pi i k_a i / n)
 __global__ void k_dft_rows(float2* F, int n, int m, int ld_rows_first) {
@@ -74,40 +75,6 @@ __global__ void k_dft_rows(float2* F, int n, int m, int ld_rows_first) {
 __global__ void k_conj(const float2* a, float2* b, long long n) {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         b[e] = make_float2(a[e].x, -a[e].y);
-}
-
-// v[b][w][i] += bias[w]
-__global__ void k_bias(float2* v, const float2* __restrict__ bias, long long n, int W, int B) {
-    const long long tot = n * W * B;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-        const int w = (int)((e / n) % W);
-        v[e].x += bias[w].x;
-        v[e].y += bias[w].y;
-    }
-}
-
-// z += bias; keep z; v = split-GELU(z) (or z)
-__global__ void k_bias_act(float2* __restrict__ z, const float2* __restrict__ bias, float2* __restrict__ v, long long n,
-                           int W, int B, int act) {
-    const long long tot = n * W * B;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-        const int w = (int)((e / n) % W);
-        float2 t = z[e];
-        t.x += bias[w].x;
-        t.y += bias[w].y;
-        z[e] = t;
-        v[e] = act ? make_float2(gelu_f(t.x), gelu_f(t.y)) : t;
-    }
-}
-
-__global__ void k_act_grad(const float2* __restrict__ z, float2* __restrict__ g, long long tot) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-        const float2 t = z[e];
-        float2 a = g[e];
-        a.x *= gelu_g(t.x);
-        a.y *= gelu_g(t.y);
-        g[e] = a;
-    }
 }
 
 // [b][w][mode] <-> [mode][b][w]: per mode a W x B column-major matrix
@@ -147,31 +114,6 @@ __global__ void k_loss(const float2* __restrict__ y, const float2* __restrict__ 
         double a = 0;
         for (int i = 0; i < 8; ++i) a += red[i];
         part[blockIdx.x] = a;
-    }
-}
-
-// out[w] = sum over b, i of g[b][w][i]   (one CTA per w)
-__global__ void k_chan_sum(const float2* __restrict__ g, float2* __restrict__ out, long long n, int W, int B) {
-    const int w = blockIdx.x;
-    float sx = 0, sy = 0;
-    for (int b = 0; b < B; ++b) {
-        const float2* p = g + ((long long)b * W + w) * n;
-        for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-            sx += p[i].x;
-            sy += p[i].y;
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
-    }
-    __shared__ float2 red[8];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(sx, sy);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float2 a = c0();
-        for (int i = 0; i < 8; ++i) { a.x += red[i].x; a.y += red[i].y; }
-        out[w] = a;
     }
 }
 
@@ -294,12 +236,13 @@ __global__ void k_sqrt_inv(const double* __restrict__ n2, double* __restrict__ n
 }  // namespace
 
 // ------------------------------------------------------------- forward
-// Activations kept for the backward pass.
+// Activations: the scratch of a forward pass and, when keep is set, what the
+// backward pass reads.
 struct FnoTape {
     int B = 0;
+    bool keep = false;
     std::vector<DevBuf*> bufs;
-    float2 *x = nullptr, *y = nullptr;
-    std::vector<float2*> v, z, Vh;     // v[0..L], z[0..L-1], Vh[0..L-1] ([b][w][mode])
+    std::vector<float2*> v, z, Vt;     // v[0..L], z[0..L-2], Vt[0..L-1] ([mode][b][w])
     ~FnoTape() { for (auto* b : bufs) delete b; }
     float2* get(size_t elems, cudaStream_t st, lsw_status* s) {
         DevBuf* b = new (std::nothrow) DevBuf();
@@ -311,129 +254,215 @@ struct FnoTape {
     }
 };
 
+namespace {
+
+bool fno_fast(int nz, int nx, int M) {
+    if (M != 8 && M != 16 && M != 32) return false;
+    if (nz % M || nx % M) return false;
+    const int qz = nz / M, qx = nx / M;
+    return is_pow2(qz) && is_pow2(qx) && qz <= M && qx <= M &&
+           sizeof(float2) * M * (size_t)(nx + 1) <= 200 * 1024;
+}
+
+// scratch of the spectral passes
+struct SpecWork {
+    float2 *T1, *Vh, *Zt, *Zh;
+};
+
+// Vt[mode][b][w] = scale * truncated transform of the B W fields of v
+lsw_status fno_analysis(const lsw_fno* f, const float2* v, int B, float scale, const SpecWork& wk, float2* Vt,
+                        cudaStream_t st) {
+    const int W = f->W, M = f->M, MM = M * M, nz = f->nz, nx = f->nx;
+    if (f->fast) {
+        const size_t smem = sizeof(float2) * M * (size_t)(nx + 1);
+        static std::atomic<bool> attr{false};
+        if (!attr.load()) {
+            for (auto k : {k_fno_analysis<8>, k_fno_analysis<16>, k_fno_analysis<32>})
+                LSW_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+            attr.store(true);
+        }
+        auto k = M == 8 ? k_fno_analysis<8> : M == 16 ? k_fno_analysis<16> : k_fno_analysis<32>;
+        k<<<B * W, 256, smem, st>>>(v, nz, nx, B * W, f->twz, f->twx, scale, Vt);
+        LSW_LAUNCH_CHECK();
+        return LSW_OK;
+    }
+    // Vh = Fz v FxT   (per sample and channel: M x M)
+    LSW_TRY(gemm<float>('N', 'N', M, nx, nz, c1(), f->Fz, M, 0, v, nz, f->n, c0(), wk.T1, M, (long long)M * nx, B * W, st));
+    LSW_TRY(gemm<float>('N', 'N', M, M, nx, make_float2(scale, 0.f), wk.T1, M, (long long)M * nx, f->FxT, nx, 0, c0(),
+                        wk.Vh, M, MM, B * W, st));
+    k_bwm_to_mwb<<<gridn((long long)B * W * MM), 256, 0, st>>>(wk.Vh, Vt, B, W, MM);
+    LSW_LAUNCH_CHECK();
+    return LSW_OK;
+}
+
+// out = sigma(inverse transform of Zt / scale^-1 + pointwise map of v + bias)
+lsw_status fno_synthesis(const lsw_fno* f, const float2* Zt, int B, float scale, const SpecWork& wk, float2* zin,
+                         PointwiseArgs a, cudaStream_t st) {
+    const int W = f->W, M = f->M, MM = M * M, nz = f->nz, nx = f->nx, og = (W + 7) / 8;
+    a.n = f->n;
+    a.nz = nz;
+    a.W = W;
+    // the fused z transform needs whole columns in a tile
+    const int cells = 4 * pw_cells(og);
+    const bool fused = f->fast && cells % nz == 0;
+    if (f->fast) {
+        auto k = M == 8 ? k_fno_synth_x<8> : M == 16 ? k_fno_synth_x<16> : k_fno_synth_x<32>;
+        k<<<B * W, 256, 0, st>>>(Zt, nx, B * W, f->twx, scale, wk.T1);
+        LSW_LAUNCH_CHECK();
+    } else {
+        k_mwb_to_bwm<<<gridn((long long)B * W * MM), 256, 0, st>>>(Zt, wk.Zh, B, W, MM);
+        LSW_LAUNCH_CHECK();
+        LSW_TRY(gemm<float>('N', 'N', M, nx, M, make_float2(scale, 0.f), wk.Zh, M, MM, f->Fxc, M, 0, c0(), wk.T1, M,
+                            (long long)M * nx, B * W, st));
+    }
+    if (!fused)
+        LSW_TRY(gemm<float>('C', 'N', nz, nx, M, c1(), f->Fz, M, 0, wk.T1, M, (long long)M * nx, c0(), zin, nz, f->n,
+                            B * W, st));
+    a.T1 = wk.T1;
+    a.twz = f->twz;
+    a.zin = zin;
+    const int nt = pw_threads(og);
+    const int Mk = fused ? M : 0;
+    const size_t smem = sizeof(float2) * W * (size_t)(8 * og + cells + 8);
+    const dim3 grid((unsigned)((f->n + cells - 1) / cells), B);
+    typedef void (*Kern)(PointwiseArgs);
+    static const Kern kerns[2][4] = {{k_fno_pointwise<0, 256>, k_fno_pointwise<8, 256>, k_fno_pointwise<16, 256>,
+                                      k_fno_pointwise<32, 256>},
+                                     {k_fno_pointwise<0, 512>, k_fno_pointwise<8, 512>, k_fno_pointwise<16, 512>,
+                                      k_fno_pointwise<32, 512>}};
+    static std::atomic<bool> attr{false};
+    if (!attr.load()) {
+        for (auto& by_m : kerns)
+            for (Kern k : by_m)
+                LSW_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        attr.store(true);
+    }
+    const Kern k = kerns[nt == 512][Mk == 0 ? 0 : Mk == 8 ? 1 : Mk == 16 ? 2 : 3];
+    k<<<grid, nt, smem, st>>>(a);
+    LSW_LAUNCH_CHECK();
+    return LSW_OK;
+}
+
+bool fno_zin_needed(const lsw_fno* f) { return !f->fast || (4 * pw_cells((f->W + 7) / 8)) % f->nz != 0; }
+
+lsw_status fno_spec_work(const lsw_fno* f, int B, FnoTape& tp, SpecWork* wk, cudaStream_t st) {
+    lsw_status s = LSW_OK;
+    const size_t modes = (size_t)B * f->W * f->M * f->M;
+    wk->T1 = tp.get((size_t)B * f->W * f->M * f->nx, st, &s);
+    wk->Zt = tp.get(modes, st, &s);
+    wk->Vh = wk->Zh = nullptr;
+    if (!f->fast) {
+        wk->Vh = tp.get(modes, st, &s);
+        wk->Zh = tp.get(modes, st, &s);
+    }
+    return s;
+}
+
+}  // namespace
+
 static lsw_status fno_forward(const lsw_fno* f, const float2* x, float2* y, int B, FnoTape& tp, cudaStream_t st) {
     const long long n = f->n;
-    const int W = f->W, M = f->M, MM = M * M, nz = f->nz, nx = f->nx;
+    const int W = f->W, M = f->M, MM = M * M;
     const float2* P = f->params;
     lsw_status s = LSW_OK;
     tp.B = B;
     tp.v.assign(f->L + 1, nullptr);
     tp.z.assign(f->L, nullptr);
-    tp.Vh.assign(f->L, nullptr);
-    float2* T1 = tp.get((size_t)B * W * M * nx, st, &s);
-    float2* Vt = tp.get((size_t)B * W * MM, st, &s);
-    float2* Zt = tp.get((size_t)B * W * MM, st, &s);
-    float2* Zh = tp.get((size_t)B * W * MM, st, &s);
-    for (int l = 0; l <= f->L; ++l) tp.v[l] = tp.get((size_t)B * W * n, st, &s);
+    tp.Vt.assign(f->L, nullptr);
+    SpecWork wk;
+    LSW_TRY(fno_spec_work(f, B, tp, &wk, st));
+    const size_t act = (size_t)B * W * n, modes = (size_t)B * W * MM;
+    float2* zin = fno_zin_needed(f) ? tp.get(act, st, &s) : nullptr;
+    for (int l = 0; l <= f->L; ++l)     // without keep the pointwise map works in place
+        tp.v[l] = l == 0 || tp.keep ? tp.get(act, st, &s) : tp.v[0];
     for (int l = 0; l < f->L; ++l) {
-        tp.z[l] = tp.get((size_t)B * W * n, st, &s);
-        tp.Vh[l] = tp.get((size_t)B * W * MM, st, &s);
+        if (tp.keep && l < f->L - 1) tp.z[l] = tp.get(act, st, &s);
+        tp.Vt[l] = l == 0 || tp.keep ? tp.get(modes, st, &s) : tp.Vt[0];
     }
     if (s != LSW_OK) return s;
-    // lift: V0_b (n x W) = X_b (n x 2) P^T (2 x W) + p
-    LSW_TRY(gemm<float>('N', 'N', (int)n, W, 2, c1(), x, (int)n, 2 * n, P + f->oPT, 2, 0, c0(), tp.v[0], (int)n, W * n, B, st));
-    k_bias<<<gridn(n * W * B), 256, 0, st>>>(tp.v[0], P + f->op, n, W, B);
+    const dim3 cells((unsigned)((n + 255) / 256), B);
+    k_fno_lift<<<cells, 256, 0, st>>>(x, P + f->oPT, P + f->op, tp.v[0], n, W);
     LSW_LAUNCH_CHECK();
+    const size_t smix = sizeof(float2) * ((size_t)W * W + W * 32);
     for (int l = 0; l < f->L; ++l) {
-        float2* v = tp.v[l];
-        float2* z = tp.z[l];
-        // Vh = Fz v FxT   (per sample and channel: M x M)
-        LSW_TRY(gemm<float>('N', 'N', M, nx, nz, c1(), f->Fz, M, 0, v, nz, n, c0(), T1, M, (long long)M * nx, B * W, st));
-        LSW_TRY(gemm<float>('N', 'N', M, M, nx, c1(), T1, M, (long long)M * nx, f->FxT, nx, 0, c0(), tp.Vh[l], M, MM,
-                            B * W, st));
-        // Zh[mode] = R[mode] Vh[mode]
-        k_bwm_to_mwb<<<gridn((long long)B * W * MM), 256, 0, st>>>(tp.Vh[l], Vt, B, W, MM);
+        LSW_TRY(fno_analysis(f, tp.v[l], B, 1.f, wk, tp.Vt[l], st));
+        // Zt[mode] = R[mode] Vt[mode]
+        k_fno_mix<<<MM, 256, smix, st>>>(P + f->oR[l], tp.Vt[l], wk.Zt, W, B);
         LSW_LAUNCH_CHECK();
-        LSW_TRY(gemm<float>('N', 'N', W, B, W, c1(), P + f->oR[l], W, (long long)W * W, Vt, W, (long long)W * B, c0(), Zt,
-                            W, (long long)W * B, MM, st));
-        k_mwb_to_bwm<<<gridn((long long)B * W * MM), 256, 0, st>>>(Zt, Zh, B, W, MM);
-        LSW_LAUNCH_CHECK();
-        // z = Fz^H (Zh conj(Fx)) / n
-        LSW_TRY(gemm<float>('N', 'N', M, nx, M, c1(), Zh, M, MM, f->Fxc, M, 0, c0(), T1, M, (long long)M * nx, B * W, st));
-        const float inv_n = 1.f / (float)n;
-        LSW_TRY(gemm<float>('C', 'N', nz, nx, M, make_float2(inv_n, 0.f), f->Fz, M, 0, T1, M, (long long)M * nx, c0(), z,
-                            nz, n, B * W, st));
-        // z += V W^T; z += b; v' = sigma(z)
-        LSW_TRY(gemm<float>('N', 'N', (int)n, W, W, c1(), v, (int)n, W * n, P + f->oWT[l], W, 0, c1(), z, (int)n, W * n, B,
-                            st));
-        k_bias_act<<<gridn(n * W * B), 256, 0, st>>>(z, P + f->ob[l], tp.v[l + 1], n, W, B, l < f->L - 1);
-        LSW_LAUNCH_CHECK();
+        PointwiseArgs a = {};
+        a.v = tp.v[l];
+        a.wt = P + f->oWT[l];
+        a.bias = P + f->ob[l];
+        a.z = tp.z[l];
+        a.out = tp.v[l + 1];
+        a.act = l < f->L - 1;
+        LSW_TRY(fno_synthesis(f, wk.Zt, B, 1.f / (float)n, wk, zin, a, st));
     }
-    // project: y_b (n x 1) = x0_b + V_b Q^T + q  (the residual channel passes through)
-    LSW_CUDA(cudaMemcpy2DAsync(y, sizeof(float2) * n, x, sizeof(float2) * 2 * n, sizeof(float2) * n, B,
-                               cudaMemcpyDeviceToDevice, st));
-    LSW_TRY(gemm<float>('N', 'N', (int)n, 1, W, c1(), tp.v[f->L], (int)n, W * n, P + f->oQT, W, 0, c1(), y, (int)n, n, B,
-                        st));
-    k_bias<<<gridn(n * B), 256, 0, st>>>(y, P + f->oq, n, 1, B);
+    k_fno_project<<<cells, 256, 0, st>>>(x, tp.v[f->L], P + f->oQT, P + f->oq, y, n, W);
     LSW_LAUNCH_CHECK();
     return LSW_OK;
 }
 
 static lsw_status fno_backward(lsw_fno* f, const float2* x, const float2* Gy, int B, FnoTape& tp, cudaStream_t st) {
     const long long n = f->n;
-    const int W = f->W, M = f->M, MM = M * M, nz = f->nz, nx = f->nx;
+    const int W = f->W, M = f->M, MM = M * M;
     const float2* P = f->params;
     float2* G = f->grads;
     lsw_status s = LSW_OK;
-    FnoTape wk;
-    float2* Gv = wk.get((size_t)B * W * n, st, &s);
-    float2* Gz = wk.get((size_t)B * W * n, st, &s);
-    float2* T1 = wk.get((size_t)B * W * M * nx, st, &s);
-    float2* GZh = wk.get((size_t)B * W * MM, st, &s);
-    float2* GZt = wk.get((size_t)B * W * MM, st, &s);
-    float2* Vt = wk.get((size_t)B * W * MM, st, &s);
-    float2* GVt = wk.get((size_t)B * W * MM, st, &s);
-    float2* GVh = wk.get((size_t)B * W * MM, st, &s);
+    FnoTape own;
+    SpecWork wk;
+    LSW_TRY(fno_spec_work(f, B, own, &wk, st));
+    float2* Gv = own.get((size_t)B * W * n, st, &s);        // the activations' gradient, layer by layer in place
+    float2* zin = fno_zin_needed(f) ? own.get((size_t)B * W * n, st, &s) : nullptr;
+    float2* GZt = own.get((size_t)B * W * MM, st, &s);
+    const int chunks = (int)((n + kFnoSumChunk - 1) / kFnoSumChunk);
     // per-sample partial weight gradients (W x W at most), summed over samples
-    float2* part = wk.get((size_t)B * std::max<long long>((long long)W * W, 2LL * W), st, &s);
+    float2* part = own.get((size_t)B * std::max<long long>({(long long)W * W, 2LL * W, (long long)W * chunks}), st, &s);
     if (s != LSW_OK) return s;
-    // Q^T: sum_b V_b^H Gy_b;  q: sum Gy;  Gv = Gy Q^H... Gv_b (n x W) = Gy_b (n x 1) (Q^T)^H (1 x W)
+    const dim3 cells((unsigned)((n + 255) / 256), B);
+    // Q^T: sum_b V_b^H Gy_b;  q: sum Gy;  G = Gy conj(Q)
     LSW_TRY(gemm<float>('C', 'N', W, 1, (int)n, c1(), tp.v[f->L], (int)n, W * n, Gy, (int)n, n, c0(), part, W, W, B, st));
     k_batch_sum<<<gridn(W), 256, 0, st>>>(part, G + f->oQT, W, B);
     LSW_LAUNCH_CHECK();
-    k_chan_sum<<<1, 256, 0, st>>>(Gy, G + f->oq, n, 1, B);
-    LSW_LAUNCH_CHECK();
-    LSW_TRY(gemm<float>('N', 'C', (int)n, W, 1, c1(), Gy, (int)n, n, P + f->oQT, W, 0, c0(), Gv, (int)n, W * n, B, st));
-    for (int l = f->L - 1; l >= 0; --l) {
-        const long long tot = n * W * B;
-        LSW_CUDA(cudaMemcpyAsync(Gz, Gv, sizeof(float2) * tot, cudaMemcpyDeviceToDevice, st));
-        if (l < f->L - 1) {
-            k_act_grad<<<gridn(tot), 256, 0, st>>>(tp.z[l], Gz, tot);
-            LSW_LAUNCH_CHECK();
-        }
-        float2* v = tp.v[l];
-        k_chan_sum<<<W, 256, 0, st>>>(Gz, G + f->ob[l], n, W, B);
+    // the sums read g through the kernel's in-place argument and leave it alone (z NULL)
+    auto channel_sums = [&](float2* g, const float2* z, int chan, float2* out) -> lsw_status {
+        k_fno_act_sum<<<dim3(chunks, chan * B), 256, 0, st>>>(g, z, n, part);
         LSW_LAUNCH_CHECK();
+        k_fno_sum_channels<<<chan, 32, 0, st>>>(part, chunks, chan, B, out);
+        LSW_LAUNCH_CHECK();
+        return LSW_OK;
+    };
+    LSW_TRY(channel_sums(const_cast<float2*>(Gy), nullptr, 1, G + f->oq));
+    k_fno_project_grad<<<cells, 256, 0, st>>>(Gy, P + f->oQT, Gv, n, W);
+    LSW_LAUNCH_CHECK();
+    const size_t smix = sizeof(float2) * ((size_t)W * (W + 1) + 2 * W * 32);
+    static std::atomic<bool> attr{false};
+    if (!attr.load()) {
+        LSW_CUDA(cudaFuncSetAttribute(k_fno_mix_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+        attr.store(true);
+    }
+    for (int l = f->L - 1; l >= 0; --l) {
+        // Gz = Gv sigma'(z) and its channel sums
+        LSW_TRY(channel_sums(Gv, l < f->L - 1 ? tp.z[l] : nullptr, W, G + f->ob[l]));
         // W^T: sum_b V_b^H Gz_b
-        LSW_TRY(gemm<float>('C', 'N', W, W, (int)n, c1(), v, (int)n, W * n, Gz, (int)n, W * n, c0(), part, W,
+        LSW_TRY(gemm<float>('C', 'N', W, W, (int)n, c1(), tp.v[l], (int)n, W * n, Gv, (int)n, W * n, c0(), part, W,
                             (long long)W * W, B, st));
         k_batch_sum<<<gridn((long long)W * W), 256, 0, st>>>(part, G + f->oWT[l], (long long)W * W, B);
         LSW_LAUNCH_CHECK();
-        // G_Zh = Fz Gz FxT / n
-        const float inv_n = 1.f / (float)n;
-        LSW_TRY(gemm<float>('N', 'N', M, nx, nz, c1(), f->Fz, M, 0, Gz, nz, n, c0(), T1, M, (long long)M * nx, B * W, st));
-        LSW_TRY(gemm<float>('N', 'N', M, M, nx, make_float2(inv_n, 0.f), T1, M, (long long)M * nx, f->FxT, nx, 0, c0(), GZh,
-                            M, MM, B * W, st));
-        k_bwm_to_mwb<<<gridn((long long)B * W * MM), 256, 0, st>>>(GZh, GZt, B, W, MM);
-        LSW_LAUNCH_CHECK();
-        k_bwm_to_mwb<<<gridn((long long)B * W * MM), 256, 0, st>>>(tp.Vh[l], Vt, B, W, MM);
-        LSW_LAUNCH_CHECK();
-        // G_R[mode] = GZt[mode] Vt[mode]^H ;  GVt[mode] = R[mode]^H GZt[mode]
-        LSW_TRY(gemm<float>('N', 'C', W, W, B, c1(), GZt, W, (long long)W * B, Vt, W, (long long)W * B, c0(), G + f->oR[l],
-                            W, (long long)W * W, MM, st));
-        LSW_TRY(gemm<float>('C', 'N', W, B, W, c1(), P + f->oR[l], W, (long long)W * W, GZt, W, (long long)W * B, c0(), GVt,
-                            W, (long long)W * B, MM, st));
-        k_mwb_to_bwm<<<gridn((long long)B * W * MM), 256, 0, st>>>(GVt, GVh, B, W, MM);
+        // G_Zh = Fz Gz FxT / n;  G_R[mode] = GZt[mode] Vt[mode]^H, GVt[mode] = R[mode]^H GZt[mode]
+        LSW_TRY(fno_analysis(f, Gv, B, 1.f / (float)n, wk, GZt, st));
+        k_fno_mix_grad<<<MM, 256, smix, st>>>(P + f->oR[l], tp.Vt[l], GZt, G + f->oR[l], wk.Zt, W, B);
         LSW_LAUNCH_CHECK();
         // Gv = Fz^H GVh conj(Fx)  +  Gz (W^T)^H
-        LSW_TRY(gemm<float>('N', 'N', M, nx, M, c1(), GVh, M, MM, f->Fxc, M, 0, c0(), T1, M, (long long)M * nx, B * W, st));
-        LSW_TRY(gemm<float>('C', 'N', nz, nx, M, c1(), f->Fz, M, 0, T1, M, (long long)M * nx, c0(), Gv, nz, n, B * W, st));
-        LSW_TRY(gemm<float>('N', 'C', (int)n, W, W, c1(), Gz, (int)n, W * n, P + f->oWT[l], W, 0, c1(), Gv, (int)n, W * n, B,
-                            st));
+        PointwiseArgs a = {};
+        a.v = Gv;
+        a.wt = P + f->oWT[l];
+        a.adjoint = 1;
+        a.out = Gv;
+        LSW_TRY(fno_synthesis(f, wk.Zt, B, 1.f, wk, zin, a, st));
     }
     // lift: P^T: sum_b X_b^H Gv_b ; p: sum Gv
-    k_chan_sum<<<W, 256, 0, st>>>(Gv, G + f->op, n, W, B);
-    LSW_LAUNCH_CHECK();
+    LSW_TRY(channel_sums(Gv, nullptr, W, G + f->op));
     LSW_TRY(gemm<float>('C', 'N', 2, W, (int)n, c1(), x, (int)n, 2 * n, Gv, (int)n, W * n, c0(), part, 2, 2LL * W, B, st));
     k_batch_sum<<<gridn(2LL * W), 256, 0, st>>>(part, G + f->oPT, 2LL * W, B);
     LSW_LAUNCH_CHECK();
@@ -526,6 +555,15 @@ lsw_status lsw_fno_create(const lsw_fno_params* p, void* stream, lsw_fno** out) 
             k_conj<<<gridn((long long)f->M * f->nx), 256, 0, st>>>(tmp.as<float2>(), f->Fxc, (long long)f->M * f->nx);
         }
     }
+    f->fast = fno_fast(f->nz, f->nx, f->M);
+    if (f->fast) {
+        al(&f->twz, f->nz);
+        al(&f->twx, f->nx);
+        if (s == LSW_OK) {
+            k_line_twiddles<<<gridn(f->nz), 256, 0, st>>>(f->twz, f->nz, f->M);
+            k_line_twiddles<<<gridn(f->nx), 256, 0, st>>>(f->twx, f->nx, f->M);
+        }
+    }
     // Gaussian initial weights (Philox), scaled per tensor by 1/sqrt(fan-in); biases zero
     if (s == LSW_OK) {
         DevBuf w2, w3;
@@ -563,7 +601,7 @@ lsw_status lsw_fno_create(const lsw_fno_params* p, void* stream, lsw_fno** out) 
 
 lsw_status lsw_fno_destroy(lsw_fno* f) {
     if (!f) return LSW_ERR_INVALID_ARG;
-    for (float2* p : {f->params, f->grads, f->adam_m, f->adam_v, f->Fz, f->FxT, f->Fxc})
+    for (float2* p : {f->params, f->grads, f->adam_m, f->adam_v, f->Fz, f->FxT, f->Fxc, f->twz, f->twx})
         if (p) cudaFree(p);
     delete f;
     return LSW_OK;
@@ -601,6 +639,7 @@ lsw_status lsw_fno_loss_grad(lsw_fno* f, const void* x, const void* target, int 
     const int nblk = 512;
     LSW_TRY(part.alloc(sizeof(double) * nblk, st));
     FnoTape tp;
+    tp.keep = true;
     LSW_TRY(fno_forward(f, (const float2*)x, y.as<float2>(), batch, tp, st));
     k_loss<<<nblk, 256, 0, st>>>(y.as<float2>(), (const float2*)target, gy.as<float2>(), tot, 1.f / (float)tot,
                                  part.as<double>());
