@@ -373,7 +373,7 @@ lsw_status lsw_autotune(const lsw_green* g, int prec, int nbatch, void* stream,
                         int* variant, float* ms3);
 
 /* Process-wide switch (default on) for the tensor-core path of the FP32
- * products of H's dense leaves with blocks of up to 32 vectors (tcgen05,
+ * products of H's dense leaves with blocks of 5 to 32 vectors (tcgen05,
  * three TF32 products per real product, FP32 accumulation: results agree
  * with the CUDA-core path to FP32 rounding, not bit for bit).  Off: every
  * product runs on the CUDA cores.  Not part of the method; for A/B

@@ -24,6 +24,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "la_tiles.cuh"
 #include "lsw_internal.cuh"
 
 namespace lsw {
@@ -597,6 +598,22 @@ k_lr_partial(LrLevels<C, FT> lv, int m, int r, int k, const C* __restrict__ X, i
     }
 }
 
+// The same for FP32 factors, column-major: cn_block_f32 (65536 rows, 6 levels,
+// 20 x 32: 124 -> 81 us on one GB300).
+template <int NPRE, int MA>
+__global__ void __launch_bounds__(256)
+k_lr_partial_f32(LrLevels<float2, float2> lv, int m, int r, int k, const float2* __restrict__ X, int swapA,
+                 float2* __restrict__ P) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    int q = 0;
+    while (q + 1 < lv.nlev && (int)blockIdx.x >= lv.chunk0[q + 1]) ++q;
+    const int nb = lv.nb[q], row0 = (blockIdx.x - lv.chunk0[q]) * lv.ch[q];
+    const int j = row0 / nb, o = row0 - j * nb;
+    const int src = swapA ? (j ^ 1) : j;
+    cn_block_f32<NPRE, MA>(r, k, lv.F[q] + (long long)j * nb * r + o, nb, X + (long long)src * nb + o, m, lv.ch[q],
+                       reinterpret_cast<float2*>(sm_raw), P + (long long)blockIdx.x * r * k);
+}
+
 // T[level q][block j] = sum over the block's chunks of the partials, in order.
 template <typename C, typename FT>
 __global__ void k_lr_reduce(LrLevels<C, FT> lv, int r, int k, const C* __restrict__ P, C* __restrict__ T) {
@@ -616,27 +633,30 @@ __global__ void k_lr_reduce(LrLevels<C, FT> lv, int r, int k, const C* __restric
     }
 }
 
-// Y[i][c] += sum over levels of G_b'(row) T_b': thread (4 consecutive rows,
-// group of 8 columns); the 4 rows share their block at every level (block
-// sizes are multiples of 4), so each T entry loaded serves 4 rows.
-template <typename C, typename FT>
+// Y[i][c] += sum over levels of G_b'(row) T_b': thread (RPT consecutive rows,
+// group of UC columns); the rows share their block at every level (block
+// sizes are multiples of 4), so each T entry loaded serves all of them.  Four
+// rows and 8 columns amortise the loads; one row where the node is too small
+// to fill the GPU with four, and 4 columns where there are no more (FP64
+// issue is what bounds that type).
+template <typename C, typename FT, int RPT, int UC>
 __global__ void __launch_bounds__(128)
 k_lr_apply(LrLevels<C, FT> lv, int m, int r, int k, const C* __restrict__ T, int swapC, C* __restrict__ Y) {
-    const int ngrp = (k + 7) / 8;
+    const int ngrp = (k + UC - 1) / UC;
     const int slots = 128 / ngrp;
     const int slot = threadIdx.x % slots, g = threadIdx.x / slots;
     if (g >= ngrp) return;
-    const int i0 = (blockIdx.x * slots + slot) * 4;
+    const int i0 = (blockIdx.x * slots + slot) * RPT;
     if (i0 >= m) return;
-    const int c0 = g * 8;
+    const int c0 = g * UC;
     const long long nout = (long long)r * k;
-    // four factor columns' loads in flight (one for FP64, where registers run out)
-    constexpr int UNR = sizeof(C) == 16 ? 1 : 4;
-    C acc[4][8];
+    // four factor columns' loads in flight (one where registers run out)
+    constexpr int UNR = sizeof(C) == 16 && RPT * UC > 8 ? 1 : 4;
+    C acc[RPT][UC];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < RPT; ++a)
 #pragma unroll
-        for (int u = 0; u < 8; ++u) acc[a][u] = czero<C>();
+        for (int u = 0; u < UC; ++u) acc[a][u] = czero<C>();
     for (int q = 0; q < lv.nlev; ++q) {
         const int nb = lv.nb[q];
         const int b = i0 / nb, o = i0 - b * nb;
@@ -646,25 +666,111 @@ k_lr_apply(LrLevels<C, FT> lv, int m, int r, int k, const C* __restrict__ T, int
         const C* Tb = T + (lv.t0[q] + bb) * nout;
 #pragma unroll UNR
         for (int t = 0; t < r; ++t) {
-            C gv[4], tv[8];
+            C gv[RPT], tv[UC];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < RPT; ++a)
                 gv[a] = ldfac(glay == FAC_PLAIN ? Gb + (long long)t * nb + a
                                                 : lv.G[q] + fac_index(glay, nb, r, lv.rp, bb, o + a, t));
 #pragma unroll
-            for (int u = 0; u < 8; ++u) tv[u] = c0 + u < k ? Tb[(long long)(c0 + u) * r + t] : czero<C>();
+            for (int u = 0; u < UC; ++u) tv[u] = c0 + u < k ? Tb[(long long)(c0 + u) * r + t] : czero<C>();
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < RPT; ++a)
 #pragma unroll
-                for (int u = 0; u < 8; ++u) cfma(acc[a][u], gv[a], tv[u]);
+                for (int u = 0; u < UC; ++u) cfma(acc[a][u], gv[a], tv[u]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < UC; ++u)
+        if (c0 + u < k) {
+#pragma unroll
+            for (int a = 0; a < RPT; ++a) {
+                C* y = Y + (long long)(c0 + u) * m + i0 + a;
+                *y = cadd(*y, acc[a][u]);
+            }
+        }
+}
+
+// The same for FP32 factors, column-major, block sizes multiples of 32 RPT: a
+// CTA takes 32 RPT rows, which lie in one block at every level, and a warp per
+// group of 8 columns (lane: rows lane + 32 a).  The factor's columns stream
+// through shared memory in chunks of LRA_T columns, LRA_ST chunks ahead
+// (cp.async): with every warp loading them itself only a quarter of the bytes
+// in flight were different ones, and 65536 rows, 6 levels, 20 x 32 took
+// 104 - 136 us instead of 73.  A level's T block arrives with its first chunk, in a ring of
+// lra_ring() blocks: as many as the levels the chunks in flight can touch.
+constexpr int LRA_T = 8, LRA_ST = 4;
+__host__ __device__ inline int lra_ring(int r) {
+    const int nch = (r + LRA_T - 1) / LRA_T;
+    return nch >= 3 ? 2 : nch == 2 ? 3 : 4;
+}
+template <int RPT>
+__global__ void __launch_bounds__(256)
+k_lr_apply_f32(LrLevels<float2, float2> lv, int m, int r, int k, const float2* __restrict__ T, int swapC,
+               float2* __restrict__ Y) {
+    constexpr int ROWS = 32 * RPT;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    const int ngrp = blockDim.x >> 5, ld = 8 * ngrp + 2;        // even: 16-byte loads
+    float2* gs = reinterpret_cast<float2*>(sm_raw);             // LRA_ST x LRA_T x ROWS
+    float2* ts = gs + LRA_ST * LRA_T * ROWS;                    // ring x r x ld
+    const int g = threadIdx.x >> 5, lane = threadIdx.x & 31, c0 = 8 * g;
+    const int row0 = blockIdx.x * ROWS;
+    const int nout = r * k, nch = (r + LRA_T - 1) / LRA_T, total = lv.nlev * nch, ring = lra_ring(r);
+    auto issue = [&](int i) {
+        if (i < total) {
+            const int q = i / nch, t0 = (i - q * nch) * LRA_T, nt = min(LRA_T, r - t0);
+            const int nb = lv.nb[q], b = row0 / nb, bb = swapC ? (b ^ 1) : b;
+            const float2* Gb = lv.G[q] + ((long long)bb * r + t0) * nb + (row0 - b * nb);
+            float2* d = gs + (i % LRA_ST) * LRA_T * ROWS;
+            for (int e = threadIdx.x; e < nt * (ROWS / 2); e += blockDim.x) {
+                const int t = e / (ROWS / 2), x = e % (ROWS / 2) * 2;
+                cp_async<16>(d + t * ROWS + x, Gb + (long long)t * nb + x);
+            }
+            if (t0 == 0) {
+                const float2* Tb = T + (lv.t0[q] + bb) * nout;
+                float2* dt = ts + (q % ring) * r * ld;
+                for (int c = g; c < k; c += ngrp)
+                    for (int t = lane; t < r; t += 32) cp_async<8>(dt + t * ld + c, Tb + c * r + t);
+            }
+        }
+        cp_async_commit();
+    };
+    float2 acc[RPT][8];
+#pragma unroll
+    for (int a = 0; a < RPT; ++a)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[a][u] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < LRA_ST - 1; ++i) issue(i);
+    for (int i = 0; i < total; ++i) {
+        cp_async_wait<LRA_ST - 2>();
+        __syncthreads();                // chunk i is here, chunk i - 1 is done with
+        issue(i + LRA_ST - 1);
+        const int q = i / nch, t0 = (i - q * nch) * LRA_T, nt = min(LRA_T, r - t0);
+        const float2* gq = gs + (i % LRA_ST) * LRA_T * ROWS + lane;
+        const float2* tq = ts + (q % ring) * r * ld + t0 * ld + c0;
+#pragma unroll 2
+        for (int t = 0; t < nt; ++t) {
+            float2 gv[RPT];
+#pragma unroll
+            for (int a = 0; a < RPT; ++a) gv[a] = gq[t * ROWS + 32 * a];
+            const float4* tv = reinterpret_cast<const float4*>(tq + t * ld);
+#pragma unroll
+            for (int u = 0; u < 8; u += 2) {
+                const float4 w = tv[u / 2];
+#pragma unroll
+                for (int a = 0; a < RPT; ++a) {
+                    cfma(acc[a][u], gv[a], make_float2(w.x, w.y));
+                    cfma(acc[a][u + 1], gv[a], make_float2(w.z, w.w));
+                }
+            }
         }
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u)
         if (c0 + u < k) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                C* y = Y + (long long)(c0 + u) * m + i0 + a;
+            for (int a = 0; a < RPT; ++a) {
+                float2* y = Y + (long long)(c0 + u) * m + row0 + lane + 32 * a;
                 *y = cadd(*y, acc[a][u]);
             }
         }
@@ -680,7 +786,15 @@ lsw_status lr_launch(const LrLevels<C, FT>& lv, int m, int r, int k, const C* X,
     LSW_TRY(T.alloc(sizeof(C) * (size_t)lv.t0[lv.nlev] * nout, st));
     static std::atomic<bool> attr{false};
     if (!attr.load()) {
-        LSW_CUDA(cudaFuncSetAttribute(k_lr_partial<C, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        if constexpr (std::is_same<FT, float2>::value) {
+            for (auto kk : {k_lr_partial_f32<2, 8>, k_lr_partial_f32<4, 8>, k_lr_partial_f32<9, 8>, k_lr_partial_f32<2, 5>,
+                            k_lr_partial_f32<4, 5>, k_lr_partial_f32<9, 5>})
+                LSW_CUDA(cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+            for (auto kk : {k_lr_apply_f32<1>, k_lr_apply_f32<2>, k_lr_apply_f32<4>})
+                LSW_CUDA(cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024));
+        } else {
+            LSW_CUDA(cudaFuncSetAttribute(k_lr_partial<C, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        }
         attr.store(true);
     }
     const int rs = (r + 3) & ~3, ks = (k + 3) & ~3;
@@ -699,6 +813,14 @@ lsw_status lr_launch(const LrLevels<C, FT>& lv, int m, int r, int k, const C* X,
         if (tc) {
             if constexpr (std::is_same<C, float2>::value && std::is_same<FT, uint32_t>::value)
                 LSW_TRY(lr_partial_tc(lv, m, r, k, X, swapA, P.as<C>(), st));
+        } else if constexpr (std::is_same<FT, float2>::value) {
+            const int ma = cn_block_ma(r, k), npre = cn_block_npre(r, k, ma);
+            auto kern = ma == 8 ? (npre == 2 ? k_lr_partial_f32<2, 8> : npre == 4 ? k_lr_partial_f32<4, 8>
+                                                                                  : k_lr_partial_f32<9, 8>)
+                                : (npre == 2 ? k_lr_partial_f32<2, 5> : npre == 4 ? k_lr_partial_f32<4, 5>
+                                                                                  : k_lr_partial_f32<9, 5>);
+            kern<<<lv.chunk0[lv.nlev], 256, cn_block_smem(r, k, ma), st>>>(lv, m, r, k, X, swapA, P.as<C>());
+            LSW_LAUNCH_CHECK();
         } else {
             k_lr_partial<C, FT><<<lv.chunk0[lv.nlev], 256, smem, st>>>(lv, m, r, k, X, swapA, P.as<C>());
             LSW_LAUNCH_CHECK();
@@ -716,8 +838,30 @@ lsw_status lr_launch(const LrLevels<C, FT>& lv, int m, int r, int k, const C* X,
         if constexpr (std::is_same<C, float2>::value && std::is_same<FT, uint32_t>::value)
             return lr_apply_tc(lv, m, r, k, T.as<C>(), swapC, Y, st);
     }
-    const int rows_cta = 4 * (128 / ((k + 7) / 8));
-    k_lr_apply<C, FT><<<(m + rows_cta - 1) / rows_cta, 128, 0, st>>>(lv, m, r, k, T.as<C>(), swapC, Y);
+    if constexpr (std::is_same<FT, float2>::value) {
+        // rows per thread: 4 while that leaves two CTAs per SM, fewer below
+        int least = m;
+        for (int q = 0; q < lv.nlev; ++q) least = std::min(least, lv.nb[q]);
+        const int rpt = m >= 128 * 304 && least % 128 == 0 ? 4 : m >= 64 * 152 && least % 64 == 0 ? 2 : 1;
+        if (least % 32 == 0) {
+            const int ngrp = (k + 7) / 8;
+            const size_t sma = sizeof(float2) * ((size_t)LRA_ST * LRA_T * 32 * rpt + (size_t)lra_ring(r) * r * (8 * ngrp + 2));
+            auto kern = rpt == 4 ? k_lr_apply_f32<4> : rpt == 2 ? k_lr_apply_f32<2> : k_lr_apply_f32<1>;
+            kern<<<m / (32 * rpt), 32 * ngrp, sma, st>>>(lv, m, r, k, T.as<C>(), swapC, Y);
+            LSW_LAUNCH_CHECK();
+            return LSW_OK;
+        }
+    }
+    const int uc = sizeof(C) == 16 && k <= 4 ? 4 : 8, slots = 128 / ((k + uc - 1) / uc);
+    const int rpt = sizeof(C) == 16 && m < 4 * slots * 304 ? 1 : 4;
+    const int grid = (m + rpt * slots - 1) / (rpt * slots);
+    if constexpr (sizeof(C) == 16) {
+        auto kern = uc == 4 ? (rpt == 1 ? k_lr_apply<C, FT, 1, 4> : k_lr_apply<C, FT, 4, 4>)
+                            : (rpt == 1 ? k_lr_apply<C, FT, 1, 8> : k_lr_apply<C, FT, 4, 8>);
+        kern<<<grid, 128, 0, st>>>(lv, m, r, k, T.as<C>(), swapC, Y);
+    } else {
+        k_lr_apply<C, FT, 4, 8><<<grid, 128, 0, st>>>(lv, m, r, k, T.as<C>(), swapC, Y);
+    }
     LSW_LAUNCH_CHECK();
     return LSW_OK;
 }
@@ -740,6 +884,10 @@ lsw_status lr_levels(const HStore<R>& H, int l, int c, bool F_is_W, const typena
     if (r * k > 4096 || k > 64 || r > 64 || (m & 3)) return LSW_ERR_INVALID_ARG;
     LrLevels<C, C> lv;
     lv.nlev = L - l;
+    // rows per partial product: up to 1024, fewer on small nodes so that all
+    // levels together give about four CTAs per SM
+    int chunk = 1024;
+    while (chunk > 64 && (long long)m * lv.nlev < 608LL * chunk) chunk /= 2;
     lv.chunk0[0] = 0;
     lv.t0[0] = 0;
     for (int q = 0; q < lv.nlev; ++q) {
@@ -750,7 +898,7 @@ lsw_status lr_levels(const HStore<R>& H, int l, int c, bool F_is_W, const typena
         lv.F[q] = F_is_W ? W0 : U0;
         lv.G[q] = F_is_W ? U0 : W0;
         lv.nb[q] = nb;
-        lv.ch[q] = std::min(nb, 1024);
+        lv.ch[q] = std::min(nb, std::max(chunk, nb / 64));      // at most 64 partials to add per block
         lv.chunk0[q + 1] = lv.chunk0[q] + m / lv.ch[q];
         lv.t0[q + 1] = lv.t0[q] + cnt;
     }
@@ -775,7 +923,7 @@ lsw_status leaf_product(const typename Cx<R>::T* D0, int nL, const typename Cx<R
 template <>
 lsw_status leaf_product<float>(const float2* D0, int nL, const float2* X, int m, int k, float2* Y, int nleaf,
                                cudaStream_t st) {
-    if (tc_gemm_enabled() && tc_gemm_fits(nL, k, nL))
+    if (tc_gemm_enabled() && k > 4 && tc_gemm_fits(nL, k, nL))
         return cgemm_tc(D0, nL, (long long)nL * nL, X, m, nL, Y, m, nL, nL, k, nL, make_float2(1.f, 0.f), nleaf, st);
     return gemm<float>('N', 'N', nL, k, nL, one<float2>(), D0, nL, (long long)nL * nL, X, m, nL, zero<float2>(), Y, m,
                        nL, nleaf, st);

@@ -7,7 +7,9 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstdint>
 
+#include "la_tiles.cuh"
 #include "lsw_internal.cuh"
 
 namespace lsw {
@@ -202,90 +204,16 @@ k_gemm_cn_small(int m, int n, int k, const C* __restrict__ A, int lda, long long
     }
 }
 
-// The same in FP32 with 8 x 4 outputs per thread, ti + mtr a, tj + mtn b: an
-// inner step is 128 multiply-adds on 12 loads (the 4 x 4 blocks of the FP64
-// kernel, 64 on 8, are bound by shared-memory wavefronts), a warp's loads are
-// contiguous, and the next tile is fetched into registers during the products.
-// 32 x 32 outputs over 2 M rows, one GB300: 521 us with the FP64 kernel's
-// blocks, 370 us now (46 TFLOP/s).
-template <int NPRE>
+// The same in FP32 (cn_block_f32).  32 x 32 outputs over 2 M rows, one GB300:
+// 521 us with the FP64 kernel's blocks, 370 us now (46 TFLOP/s).
+template <int NPRE, int MA>
 __global__ void __launch_bounds__(256)
 k_gemm_cn_f32(int m, int n, int k, const float2* __restrict__ A, int lda, long long sA, const float2* __restrict__ B,
               int ldb, long long sB, int kchunk, float2* __restrict__ P, int batch) {
-    constexpr int TR = 32;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    const int ms = (m + 7) & ~7, ns = (n + 3) & ~3;
-    const int asd = ms + 1, bsd = ns + 1;           // odd row strides: conflict-free transposing stores
-    float2* As = reinterpret_cast<float2*>(sm_raw);
-    float2* Bs = As + TR * asd;
-    float2* Red = As;                               // G x m x n, after the products
-    const int kp = blockIdx.x, b = blockIdx.y;
-    const int k0 = kp * kchunk, k1 = min(k, k0 + kchunk);
-    const float2* Ab = A + b * sA;
-    const float2* Bb = B + b * sB;
-    const int mtr = ms / 8, mtn = ns / 4, nmt = mtr * mtn;
-    const int G = min(TR, 256 / nmt);
-    const int mt = threadIdx.x % nmt, rg = threadIdx.x / nmt;
-    const bool active = rg < G;
-    const int ti = mt % mtr, tj = mt / mtr;
-    float2 acc[8][4];
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.f, 0.f);
-    // tile entry: row rr0 of columns cc0 + 8 u
-    const int rr0 = threadIdx.x & 31, cc0 = threadIdx.x >> 5;
-    float2 pa[NPRE], pb[NPRE];
-    auto fetch = [&](int r0) {
-        const int r = r0 + rr0;
-#pragma unroll
-        for (int u = 0; u < NPRE; ++u) {
-            const int cc = cc0 + 8 * u;
-            pa[u] = r < k1 && cc < m ? Ab[(long long)cc * lda + r] : make_float2(0.f, 0.f);
-            pb[u] = r < k1 && cc < n ? Bb[(long long)cc * ldb + r] : make_float2(0.f, 0.f);
-        }
-    };
-    fetch(k0);
-    for (int r0 = k0; r0 < k1; r0 += TR) {
-#pragma unroll
-        for (int u = 0; u < NPRE; ++u) {
-            const int cc = cc0 + 8 * u;
-            if (cc < ms) As[rr0 * asd + cc] = pa[u];
-            if (cc < ns) Bs[rr0 * bsd + cc] = pb[u];
-        }
-        __syncthreads();
-        if (r0 + TR < k1) fetch(r0 + TR);
-        if (active) {
-            for (int rr = rg; rr < TR; rr += G) {
-                float2 x[8], y[4];
-#pragma unroll
-                for (int a = 0; a < 8; ++a) x[a] = As[rr * asd + ti + mtr * a];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) y[c] = Bs[rr * bsd + tj + mtn * c];
-#pragma unroll
-                for (int a = 0; a < 8; ++a)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) cfmac(acc[a][c], x[a], y[c]);
-            }
-        }
-        __syncthreads();
-    }
-    const int nout = m * n;
-    if (active) {
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int i = ti + mtr * a, j = tj + mtn * c;
-                if (i < m && j < n) Red[(long long)rg * nout + j * m + i] = acc[a][c];
-            }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nout; e += 256) {
-        float2 sacc = make_float2(0.f, 0.f);
-        for (int g = 0; g < G; ++g) sacc = cadd(sacc, Red[(long long)g * nout + e]);
-        P[((long long)kp * batch + b) * nout + e] = sacc;
-    }
+    const int kp = blockIdx.x, b = blockIdx.y, k0 = kp * kchunk;
+    cn_block_f32<NPRE, MA>(m, n, A + b * sA + k0, lda, B + b * sB + k0, ldb, min(kchunk, k - k0),
+                       reinterpret_cast<float2*>(sm_raw), P + ((long long)kp * batch + b) * m * n);
 }
 
 // C = A^H B partial sums for tiny outputs (n <= 4 columns of B): warp w of
@@ -368,6 +296,68 @@ k_gemm_nn_smallk(int m, int n, int k, C alpha, const C* __restrict__ A, int lda,
             if (beta.x != 0 || beta.y != 0) r = cadd(r, cmul(beta, *c));
             *c = r;
         }
+    }
+}
+
+// C = A B partial sums for few columns of B (n <= NN): a CTA takes 32 RPL rows
+// (RPL consecutive ones per lane) and a range of K, its warps every eighth
+// column of A (coalesced rows), and adds the warps' sums in shared memory.
+// RPL 4 (FP32 on 16-byte aligned columns, m % 128 == 0) spreads B's loads over
+// four rows.  A tile kernel computes 32 columns for n of
+// them and, for a few 1024 x 1024 leaves, on 32 CTAs: 4 leaves times 3 vectors
+// in FP64 took 1035 us and take 130 now.  Bound by FP64 issue (2 multiply-adds
+// per SM and cycle: 86 us there; up to 8 columns) or, in FP32, by reading A
+// (up to 4 columns: 32 leaves of 1024 x 1024 times 1, 2, 4 vectors inside a
+// whole H product 201, 200, 207 -> 115, 140, 145 us against the tensor cores;
+// with 5 the tensor cores are ahead).
+template <typename C, int NN, int RPL>
+__global__ void __launch_bounds__(256)
+k_gemm_nn_few(int m, int n, int k, const C* __restrict__ A, int lda, long long sA, const C* __restrict__ B, int ldb,
+              long long sB, int kchunk, C* __restrict__ P, int batch) {
+    __shared__ C red[8][NN][32 * RPL + 1];
+    const int kp = blockIdx.y, b = blockIdx.z;
+    const int k0 = kp * kchunk, k1 = min(k, k0 + kchunk);
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int i0 = blockIdx.x * 32 * RPL;
+    const C* Ab = A + b * sA + min(i0 + l * RPL, m - RPL);
+    const C* Bb = B + b * sB;
+    C acc[NN][RPL];
+#pragma unroll
+    for (int c = 0; c < NN; ++c)
+#pragma unroll
+        for (int u = 0; u < RPL; ++u) acc[c][u] = czero<C>();
+#pragma unroll 4
+    for (int t = k0 + w; t < k1; t += 8) {
+        C a[RPL];
+        if constexpr (RPL == 1) {
+            a[0] = Ab[(long long)t * lda];
+        } else {
+#pragma unroll
+            for (int u = 0; u < RPL; u += 2) {
+                const float4 v = *reinterpret_cast<const float4*>(Ab + (long long)t * lda + u);
+                a[u] = mk(v.x, v.y);
+                a[u + 1] = mk(v.z, v.w);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NN; ++c)
+            if (c < n) {
+                const C x = Bb[(long long)c * ldb + t];
+#pragma unroll
+                for (int u = 0; u < RPL; ++u) cfma(acc[c][u], a[u], x);
+            }
+    }
+#pragma unroll
+    for (int c = 0; c < NN; ++c)
+#pragma unroll
+        for (int u = 0; u < RPL; ++u) red[w][c][l * RPL + u] = acc[c][u];
+    __syncthreads();
+    for (int e = threadIdx.x; e < n * 32 * RPL; e += 256) {
+        const int c = e / (32 * RPL), q = e % (32 * RPL);
+        C s = czero<C>();
+#pragma unroll
+        for (int v = 0; v < 8; ++v) s = cadd(s, red[v][c][q]);
+        if (i0 + q < m) P[(((long long)kp * batch + b) * n + c) * m + i0 + q] = s;
     }
 }
 
@@ -1876,13 +1866,14 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
         DevBuf part;
         LSW_TRY(part.alloc(sizeof(CT) * (size_t)ksplit * batch * m * n, st));
         if constexpr (sizeof(R) == 4) {
-            const int ms = (m + 7) & ~7, ns = (n + 3) & ~3, most = std::max(ms, ns);
-            const int G = std::min(32, 256 / ((ms / 8) * (ns / 4)));
-            const size_t smem = std::max(sizeof(CT) * 32 * (size_t)(ms + ns + 2), sizeof(CT) * (size_t)G * m * n);
-            auto kern = most <= 16 ? k_gemm_cn_f32<2> : most <= 32 ? k_gemm_cn_f32<4> : k_gemm_cn_f32<8>;
+            const int ma = cn_block_ma(m, n), npre = cn_block_npre(m, n, ma);
+            const size_t smem = cn_block_smem(m, n, ma);
+            auto kern = ma == 8 ? (npre == 2 ? k_gemm_cn_f32<2, 8> : npre == 4 ? k_gemm_cn_f32<4, 8> : k_gemm_cn_f32<9, 8>)
+                                : (npre == 2 ? k_gemm_cn_f32<2, 5> : npre == 4 ? k_gemm_cn_f32<4, 5> : k_gemm_cn_f32<9, 5>);
             static std::atomic<bool> attr_cn{false};
             if (!attr_cn.load()) {
-                for (auto kk : {k_gemm_cn_f32<2>, k_gemm_cn_f32<4>, k_gemm_cn_f32<8>})
+                for (auto kk : {k_gemm_cn_f32<2, 8>, k_gemm_cn_f32<4, 8>, k_gemm_cn_f32<9, 8>, k_gemm_cn_f32<2, 5>,
+                                k_gemm_cn_f32<4, 5>, k_gemm_cn_f32<9, 5>})
                     LSW_CUDA(cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
                 attr_cn.store(true);
             }
@@ -1907,6 +1898,32 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
         const long long pairs = ((long long)m + 1) / 2;
         k_gemv_tall<CT><<<dim3((unsigned)((pairs + 255) / 256), batch), 256, 0, st>>>(m, k, alpha, A, lda, sA, B, sB,
                                                                                       beta, C, sC);
+        LSW_LAUNCH_CHECK();
+        return LSW_OK;
+    }
+    // few columns against a long inner dimension
+    if (oa == 0 && ob == 0 && k >= 128 && m >= 32 && n <= (sizeof(R) == 8 ? 8 : 4)) {
+        const bool wide = sizeof(R) == 4 && m % 128 == 0 && reinterpret_cast<uintptr_t>(A) % 16 == 0 && lda % 2 == 0 &&
+                          sA % 2 == 0;
+        const int gx = wide ? m / 128 : (m + 31) / 32;
+        // about six CTAs per SM, each with at least 64 columns of A
+        const long long want = std::max<long long>(1, 912 / ((long long)gx * batch));
+        const int kchunk = (int)std::max<long long>(64, ((k + want - 1) / want + 7) / 8 * 8);
+        const int ksplit = (k + kchunk - 1) / kchunk;
+        DevBuf part;
+        LSW_TRY(part.alloc(sizeof(CT) * (size_t)ksplit * batch * m * n, st));
+        const dim3 gr(gx, ksplit, batch);
+        auto run = [&](auto kern) { kern<<<gr, 256, 0, st>>>(m, n, k, A, lda, sA, B, ldb, sB, kchunk, part.as<CT>(), batch); };
+        if constexpr (sizeof(R) == 4) {
+            if (wide) run(n == 1 ? k_gemm_nn_few<CT, 1, 4> : n == 2 ? k_gemm_nn_few<CT, 2, 4> : k_gemm_nn_few<CT, 4, 4>);
+            else run(n == 1 ? k_gemm_nn_few<CT, 1, 1> : n == 2 ? k_gemm_nn_few<CT, 2, 1> : k_gemm_nn_few<CT, 4, 1>);
+        } else {
+            run(n == 1 ? k_gemm_nn_few<CT, 1, 1> : n == 2 ? k_gemm_nn_few<CT, 2, 1> : n <= 4 ? k_gemm_nn_few<CT, 4, 1>
+                                                                                            : k_gemm_nn_few<CT, 8, 1>);
+        }
+        LSW_LAUNCH_CHECK();
+        k_gemm_reduce<CT><<<grid_for((long long)batch * m * n), 256, 0, st>>>(m, n, batch, ksplit, part.as<CT>(), alpha,
+                                                                              beta, C, ldc, sC);
         LSW_LAUNCH_CHECK();
         return LSW_OK;
     }
