@@ -429,6 +429,37 @@ __global__ void k_gemm_reduce(int m, int n, int batch, int ksplit, const C* __re
     }
 }
 
+// The same for few outputs and many parts: 32 outputs per CTA, one warp per
+// residue of the part index, so that a sum is not one chain of loads (496
+// Gram-Schmidt coefficients of 304 parts took 22 us).
+template <typename C>
+__global__ void __launch_bounds__(1024)
+k_gemm_reduce_few(int m, int n, int batch, int ksplit, const C* __restrict__ P, C alpha, C beta, C* __restrict__ Cm,
+                  int ldc, long long sC) {
+    __shared__ C red[32][33];
+    const long long tot = (long long)batch * m * n;
+    const long long e = blockIdx.x * 32LL + threadIdx.x;
+    C s = czero<C>();
+    if (e < tot) {
+#pragma unroll 4
+        for (int kp = threadIdx.y; kp < ksplit; kp += 32) s = cadd(s, P[kp * tot + e]);
+    }
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    for (int h = 16; h > 0; h >>= 1) {
+        if (threadIdx.y < h) red[threadIdx.y][threadIdx.x] = cadd(red[threadIdx.y][threadIdx.x], red[threadIdx.y + h][threadIdx.x]);
+        __syncthreads();
+    }
+    if (threadIdx.y || e >= tot) return;
+    const int b = (int)(e / ((long long)m * n));
+    const long long r = e - (long long)b * m * n;
+    const int j = (int)(r / m), i = (int)(r - (long long)j * m);
+    C* c = Cm + b * sC + (long long)j * ldc + i;
+    C out = cmul(alpha, red[0][threadIdx.x]);
+    if (beta.x != 0 || beta.y != 0) out = cadd(out, cmul(beta, *c));
+    *c = out;
+}
+
 // ------------------------------------------------------------ FP64 Gram
 // G_b = Y_b^H Y_b, k x k (k <= 64), partial sums over row chunks; each
 // thread owns up to 16 of the k^2 entries.
@@ -1793,12 +1824,65 @@ __global__ void __launch_bounds__(256) k_norm_partial(const C* __restrict__ x, l
     }
 }
 
-__global__ void k_norm_reduce(const double* __restrict__ part, int nchunk, int batch, double* out) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= batch) return;
+// The same for complex64.  FP64 runs at 2 lanes per cycle and SM, and two
+// conversions and two multiply-adds per entry made the norms of 16 fields of
+// 512^2 cells take 46 us.  Eight entries at a time are summed in FP32
+// arithmetic without loss: scaled by a power of two to at most 2, squares
+// split exactly (p + e = x x) and added by TwoSum (Dot2 of Ogita, Rump and
+// Oishi), the pair then added in FP64: four FP64 operations instead of 64, with
+// an error of 2^-48 of the group's own sum.
+__global__ void __launch_bounds__(256) k_norm_partial_c64(const float2* __restrict__ x, long long n, int nchunk,
+                                                          double* part) {
+    const int b = blockIdx.y, ch = blockIdx.x;
+    const long long per = (n + nchunk - 1) / nchunk;
+    const long long r0 = ch * per, r1 = min(n, r0 + per);
+    const float2* xb = x + b * n;
     double s = 0;
-    for (int c = 0; c < nchunk; ++c) s += part[(long long)b * nchunk + c];
-    out[b] = s;
+    for (long long i = r0 + threadIdx.x; i < r1; i += 8 * 256) {
+        float2 v[8];
+        float top = 0.f;
+        bool fine = true;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            v[u] = i + 256 * u < r1 ? xb[i + 256 * u] : make_float2(0.f, 0.f);
+            fine = fine && isfinite(v[u].x) && isfinite(v[u].y);
+            top = fmaxf(top, fmaxf(fabsf(v[u].x), fabsf(v[u].y)));
+        }
+        if (!fine) {
+            for (int u = 0; u < 8; ++u) s += (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
+            continue;
+        }
+        const int sc = max(254 - (__float_as_int(top) >> 23), 1);      // exponent of the scale
+        const float f = __int_as_float(sc << 23);
+        float hi = 0.f, lo = 0.f;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const float a = __fmul_rn(u & 1 ? v[u >> 1].y : v[u >> 1].x, f);
+            const float p = __fmul_rn(a, a), e = __fmaf_rn(a, a, -p);
+            const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
+            lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z)), e));
+            hi = t;
+        }
+        s = fma((double)hi + (double)lo, __hiloint2double((1023 - 2 * (sc - 127)) << 20, 0), s);
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __shared__ double red[8];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        part[(long long)b * nchunk + ch] = t;
+    }
+}
+
+// a warp per field
+__global__ void k_norm_reduce(const double* __restrict__ part, int nchunk, double* out) {
+    const long long b = blockIdx.x;
+    double s = 0;
+    for (int c = threadIdx.x; c < nchunk; c += 32) s += part[b * nchunk + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) out[b] = s;
 }
 
 template <typename C>
@@ -1819,6 +1903,21 @@ size_t cn_small_smem(int m, int n) {
     const int ms = (m + 3) & ~3, ns = (n + 3) & ~3;
     const int G = std::max(1, 256 / ((ms / 4) * (ns / 4)));
     return sizeof(CT) * (32 * (size_t)(ms + ns + 2) + (size_t)G * m * n);
+}
+
+// Sum of the ksplit parts: a warp-wide sum per output from 64 parts on, while
+// the outputs alone do not fill the GPU.
+template <typename C>
+lsw_status gemm_reduce(int m, int n, int batch, int ksplit, const C* P, C alpha, C beta, C* Cm, int ldc, long long sC,
+                       cudaStream_t st) {
+    const long long tot = (long long)batch * m * n;
+    if (ksplit >= 64 && tot <= 32LL * 152 * 2)
+        k_gemm_reduce_few<C><<<(unsigned)((tot + 31) / 32), dim3(32, 32), 0, st>>>(m, n, batch, ksplit, P, alpha, beta,
+                                                                                  Cm, ldc, sC);
+    else
+        k_gemm_reduce<C><<<grid_for(tot), 256, 0, st>>>(m, n, batch, ksplit, P, alpha, beta, Cm, ldc, sC);
+    LSW_LAUNCH_CHECK();
+    return LSW_OK;
 }
 
 template <typename R>
@@ -1853,10 +1952,7 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
             default: k_gemm_cn_tiny<CT, 4><<<gr, 256, 0, st>>>(m, k, A, lda, sA, B, ldb, sB, kchunk, part.as<CT>(), batch); break;
         }
         LSW_LAUNCH_CHECK();
-        k_gemm_reduce<CT><<<grid_for((long long)batch * m * n), 256, 0, st>>>(m, n, batch, ksplit, part.as<CT>(), alpha,
-                                                                              beta, C, ldc, sC);
-        LSW_LAUNCH_CHECK();
-        return LSW_OK;
+        return gemm_reduce<CT>(m, n, batch, ksplit, part.as<CT>(), alpha, beta, C, ldc, sC, st);
     }
     // long inner products with a small result: split K, reduce in order
     if (oa == 1 && ob == 0 && m <= 64 && n <= 64 && (long long)m * n <= 4096 && k >= 128) {
@@ -1888,10 +1984,7 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
                                                                                            kchunk, part.as<CT>(), batch);
         }
         LSW_LAUNCH_CHECK();
-        k_gemm_reduce<CT><<<grid_for((long long)batch * m * n), 256, 0, st>>>(m, n, batch, ksplit, part.as<CT>(), alpha,
-                                                                              beta, C, ldc, sC);
-        LSW_LAUNCH_CHECK();
-        return LSW_OK;
+        return gemm_reduce<CT>(m, n, batch, ksplit, part.as<CT>(), alpha, beta, C, ldc, sC, st);
     }
     // tall times one column (the solvers' Krylov updates)
     if (oa == 0 && ob == 0 && k <= 64 && n == 1 && m >= 4096) {
@@ -1922,10 +2015,7 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
                                                                                             : k_gemm_nn_few<CT, 8, 1>);
         }
         LSW_LAUNCH_CHECK();
-        k_gemm_reduce<CT><<<grid_for((long long)batch * m * n), 256, 0, st>>>(m, n, batch, ksplit, part.as<CT>(), alpha,
-                                                                              beta, C, ldc, sC);
-        LSW_LAUNCH_CHECK();
-        return LSW_OK;
+        return gemm_reduce<CT>(m, n, batch, ksplit, part.as<CT>(), alpha, beta, C, ldc, sC, st);
     }
     // tall times small
     if (oa == 0 && ob == 0 && k <= 64 && n <= 64) {
@@ -1973,10 +2063,7 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
     LSW_TRY(part.alloc(sizeof(CT) * (size_t)ksplit * batch * m * n, st));
     launch(ksplit, kchunk, part.as<CT>());
     LSW_LAUNCH_CHECK();
-    k_gemm_reduce<CT><<<grid_for((long long)batch * m * n), 256, 0, st>>>(m, n, batch, ksplit, part.as<CT>(), alpha,
-                                                                          beta, C, ldc, sC);
-    LSW_LAUNCH_CHECK();
-    return LSW_OK;
+    return gemm_reduce<CT>(m, n, batch, ksplit, part.as<CT>(), alpha, beta, C, ldc, sC, st);
 }
 
 template <typename R>
@@ -2298,9 +2385,12 @@ lsw_status norms2(const typename Cx<R>::T* x, long long n, int batch, double* ou
     const int nchunk = (int)std::max<long long>(1, std::min<long long>((n + 4095) / 4096, std::max(1, 1216 / batch)));
     DevBuf part;
     LSW_TRY(part.alloc(sizeof(double) * (size_t)nchunk * batch, st));
-    k_norm_partial<typename Cx<R>::T><<<dim3(nchunk, batch), 256, 0, st>>>(x, n, nchunk, part.as<double>());
+    if constexpr (sizeof(R) == 4)
+        k_norm_partial_c64<<<dim3(nchunk, batch), 256, 0, st>>>(x, n, nchunk, part.as<double>());
+    else
+        k_norm_partial<typename Cx<R>::T><<<dim3(nchunk, batch), 256, 0, st>>>(x, n, nchunk, part.as<double>());
     LSW_LAUNCH_CHECK();
-    k_norm_reduce<<<(batch + 255) / 256, 256, 0, st>>>(part.as<double>(), nchunk, batch, out);
+    k_norm_reduce<<<batch, 32, 0, st>>>(part.as<double>(), nchunk, out);
     LSW_LAUNCH_CHECK();
     return LSW_OK;
 }

@@ -158,6 +158,43 @@ __global__ void k_gram_c64_reduce(const double2* __restrict__ part, int nchunk, 
     }
 }
 
+// The same for many chunks of few blocks: a CTA takes 32 consecutive pairs of a
+// block (contiguous in a chunk), its 32 warps every 32nd chunk (one block of
+// 1024 chunks took 24 us with one thread's chain of loads per entry).
+__global__ void __launch_bounds__(1024)
+k_gram_c64_reduce_few(const double2* __restrict__ part, int nchunk, int k, double2* __restrict__ G) {
+    __shared__ double2 red[32][33];
+    const int npair = k * (k + 1) / 2, b = blockIdx.y;
+    const int p = blockIdx.x * 32 + threadIdx.x;
+    double2 s = make_double2(0.0, 0.0);
+    if (p < npair) {
+        const double2* src = part + (long long)b * nchunk * npair + p;
+#pragma unroll 8
+        for (int c = threadIdx.y; c < nchunk; c += 32) {
+            const double2 v = src[(long long)c * npair];
+            s.x += v.x;
+            s.y += v.y;
+        }
+    }
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    for (int h = 16; h > 0; h >>= 1) {
+        if (threadIdx.y < h) {
+            const double2 v = red[threadIdx.y + h][threadIdx.x];
+            red[threadIdx.y][threadIdx.x].x += v.x;
+            red[threadIdx.y][threadIdx.x].y += v.y;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.y || p >= npair) return;
+    int i, j;
+    tri_pair(p, i, j);
+    const double2 v = red[0][threadIdx.x];
+    double2* Gb = G + (long long)b * k * k;
+    Gb[j * k + i] = v;
+    if (i != j) Gb[i * k + j] = make_double2(v.x, -v.y);    // G(j, i) = conj(G(i, j))
+}
+
 // ------------------------------------------- Cholesky and R^-1 (FP64)
 // One CTA per matrix: G + shift I = Lt D Lt^H (Lt unit lower triangular, D
 // diagonal: the square-root-free Cholesky), then Xt = Lt^-1 and
@@ -513,7 +550,11 @@ lsw_status gram64_c64(const float2* Y, int m, int k, long long sY, int batch, do
     k_gram_c64<<<dim3(nchunk, batch), 256, sizeof(float2) * (GT_ROWS + 1) * k, st>>>(Y, m, k, sY, nchunk,
                                                                                         part.as<double2>(), active);
     LSW_LAUNCH_CHECK();
-    k_gram_c64_reduce<<<grid_small((long long)batch * k * k), 256, 0, st>>>(part.as<double2>(), nchunk, k, batch, G);
+    // many chunks go with few blocks (sketch_chunks): enough CTAs either way
+    if (nchunk >= 32)
+        k_gram_c64_reduce_few<<<dim3((npair + 31) / 32, batch), dim3(32, 32), 0, st>>>(part.as<double2>(), nchunk, k, G);
+    else
+        k_gram_c64_reduce<<<grid_small((long long)batch * k * k), 256, 0, st>>>(part.as<double2>(), nchunk, k, batch, G);
     LSW_LAUNCH_CHECK();
     return LSW_OK;
 }

@@ -73,6 +73,43 @@ __global__ void k_scale_cast(const Cs* __restrict__ src, Cd* __restrict__ dst, c
     }
 }
 
+// The next Krylov vector scale_s w_s, into vj and into the basis (col: its
+// column of source 0, ldv entries between sources).  For complex64 the scale
+// is split into two FP32 parts (the product then rounds once, as in FP64,
+// whose conversions made this 50 us for 16 fields of 512^2 cells); a scale out
+// of FP32's comfortable range keeps the FP64 product.
+template <typename C>
+__global__ void __launch_bounds__(256)
+k_basis_vector(const C* __restrict__ w, const double* __restrict__ scale, C* __restrict__ vj, C* __restrict__ col,
+               long long n, long long ldv) {
+    const long long s = blockIdx.y;
+    const double a = scale[s];
+    const float ah = (float)a, al = (float)(a - (double)ah);
+    const bool split = sizeof(C) == 8 && ((fabsf(ah) > 1e-20f && fabsf(ah) < 1e20f) || a == 0.0);
+    const C* ws = w + s * n;
+    for (long long i0 = blockIdx.x * 1024LL + threadIdx.x; i0 < n; i0 += gridDim.x * 1024LL) {
+        C v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + 256 * u < n) v[u] = ws[i0 + 256 * u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long i = i0 + 256 * u;
+            if (i >= n) break;
+            C o;
+            if (split) {
+                o.x = fmaf((float)v[u].x, ah, (float)v[u].x * al);
+                o.y = fmaf((float)v[u].y, ah, (float)v[u].y * al);
+            } else {
+                o.x = (double)v[u].x * a;
+                o.y = (double)v[u].y * a;
+            }
+            vj[s * n + i] = o;
+            col[s * ldv + i] = o;
+        }
+    }
+}
+
 // u64_s += d_s (cast up) for active sources
 template <typename Cd>
 __global__ void k_add_up(double2* __restrict__ u, const Cd* __restrict__ d, const int* __restrict__ active, long long n,
@@ -298,7 +335,7 @@ lsw_status fgmres_run(const lsw_green* g, const double* chi, const lsw_hmatrix* 
     std::vector<double> scale(nb), wstart(nb);
     const C one_ = mk((R)1, (R)0), zero_ = mk((R)0, (R)0), mone = mk((R)-1, (R)0);
     int total = 0;
-    const size_t pitchV = sizeof(C) * n * (m + 1), pitchZ = sizeof(C) * n * m, row = sizeof(C) * n;
+    const size_t pitchZ = sizeof(C) * n * m, row = sizeof(C) * n;
     StepGraph sg;
     while (true) {
         // r = b - A x  (RESIDUAL gives x - G0V x - b = -r)
@@ -326,9 +363,9 @@ lsw_status fgmres_run(const lsw_green* g, const double* chi, const lsw_hmatrix* 
             conv[s] = done[s];
         }
         LSW_TRY(up(ysc, scale, st));
-        k_scale_cast<C, C><<<gridn(n * nb), 256, 0, st>>>(w.as<C>(), vj.as<C>(), ysc.as<double>(), n, nb);
+        k_basis_vector<C><<<dim3(gridn((n + 3) / 4), nb), 256, 0, st>>>(w.as<C>(), ysc.as<double>(), vj.as<C>(),
+                                                                         V.as<C>(), n, n * (m + 1));
         LSW_LAUNCH_CHECK();
-        LSW_CUDA(cudaMemcpy2DAsync(V.p, pitchV, vj.p, row, row, nb, cudaMemcpyDeviceToDevice, st));
         const bool learned = lp && lp->fno && !lp->off;
         bool stalled = false;
         int j = 0;
@@ -372,10 +409,10 @@ lsw_status fgmres_run(const lsw_green* g, const double* chi, const lsw_hmatrix* 
                 }
             for (int s = 0; s < nb; ++s) scale[s] = (!conv[s] && nr[s] > 0) ? 1.0 / std::sqrt(nr[s]) : 0.0;
             LSW_TRY(up(ysc, scale, st));
-            k_scale_cast<C, C><<<gridn(n * nb), 256, 0, st>>>(w.as<C>(), vj.as<C>(), ysc.as<double>(), n, nb);
+            k_basis_vector<C><<<dim3(gridn((n + 3) / 4), nb), 256, 0, st>>>(w.as<C>(), ysc.as<double>(), vj.as<C>(),
+                                                                             V.as<C>() + (long long)n * (j + 1), n,
+                                                                             n * (m + 1));
             LSW_LAUNCH_CHECK();
-            LSW_CUDA(cudaMemcpy2DAsync(V.as<char>() + row * (j + 1), pitchV, vj.p, row, row, nb,
-                                       cudaMemcpyDeviceToDevice, st));
             ++total;
             int still = 0;
             for (int s = 0; s < nb; ++s) {
