@@ -2067,6 +2067,12 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
 }
 
 template <typename R>
+lsw_status gemm_reduce_parts(int m, int n, int batch, int ksplit, const typename Cx<R>::T* P, typename Cx<R>::T alpha,
+                             typename Cx<R>::T beta, typename Cx<R>::T* C, int ldc, long long sC, cudaStream_t st) {
+    return gemm_reduce<typename Cx<R>::T>(m, n, batch, ksplit, P, alpha, beta, C, ldc, sC, st);
+}
+
+template <typename R>
 lsw_status qr_explicit(typename Cx<R>::T* A, int m, int k, long long sA, int batch, typename Cx<R>::T* work,
                        cudaStream_t st) {
     typedef typename Cx<R>::T CT;
@@ -2406,6 +2412,8 @@ lsw_status norms2(const typename Cx<R>::T* x, long long n, int batch, double* ou
     template lsw_status gaussian_fill<R>(Cx<R>::T*, int, int, long long, int, uint64_t, const uint32_t*,          \
                                          const uint32_t*, cudaStream_t);                                          \
     template lsw_status inverse_gj<R>(Cx<R>::T*, int, long long, int, cudaStream_t);                              \
+    template lsw_status gemm_reduce_parts<R>(int, int, int, int, const Cx<R>::T*, Cx<R>::T, Cx<R>::T, Cx<R>::T*, int, \
+                                             long long, cudaStream_t);                                            \
     template lsw_status norms2<R>(const Cx<R>::T*, long long, int, double*, cudaStream_t);
 LSW_INST(float)
 LSW_INST(double)

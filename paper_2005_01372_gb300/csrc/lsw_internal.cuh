@@ -216,6 +216,12 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
                 typename Cx<R>::T beta, typename Cx<R>::T* C, int ldc, long long sC,
                 int batch, cudaStream_t st);
 
+// C_b = alpha sum_p P_p,b + beta C_b for ksplit parts of a batched product,
+// P[part][b] an m x n matrix, column-major.
+template <typename R>
+lsw_status gemm_reduce_parts(int m, int n, int batch, int ksplit, const typename Cx<R>::T* P, typename Cx<R>::T alpha,
+                             typename Cx<R>::T beta, typename Cx<R>::T* C, int ldc, long long sC, cudaStream_t st);
+
 // Batched thin Householder QR: A_b (m x k, ld m) is replaced by Q_b with
 // orthonormal columns spanning range(A_b) (k <= 64, m >= 1).
 template <typename R>

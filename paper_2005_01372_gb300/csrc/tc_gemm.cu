@@ -18,7 +18,8 @@
 // memory in the canonical K-major layout without swizzle (8-row x 16-byte core
 // matrices, 128 B apart along K, 1024 B apart along rows); one thread issues
 // 3 x 4 tcgen05.mma of 128 x 64 x 8 and commits them to the stage's mbarrier,
-// which the producer waits on (bounded) before reusing that buffer.
+// which the producer waits on (bounded) before reusing that buffer.  With few
+// matrices K is split over blockIdx.z into parts sP apart, added afterwards.
 #include <cuda_runtime.h>
 
 #include <cuda_bf16.h>
@@ -50,16 +51,16 @@ using namespace tcx;
 
 __global__ void __launch_bounds__(128)
 k_cgemm_tc(const float2* __restrict__ A, int lda, long long sA, const float2* __restrict__ B, int ldb, long long sB,
-           float2* __restrict__ Cm, int ldc, long long sC, int N, int K, float2 alpha) {
+           float2* __restrict__ Cm, int ldc, long long sC, long long sP, int N, int Kper, float2 alpha) {
     extern __shared__ __align__(1024) unsigned char sm[];
     uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + 2 * STAGE);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + 2 * STAGE + 16);
     int* abort_flag = reinterpret_cast<int*>(sm + 2 * STAGE + 32);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int b = blockIdx.y, i0 = blockIdx.x * TC_M;
-    const float2* Ab = A + b * sA + i0;
-    const float2* Bb = B + b * sB;
-    float2* Cb = Cm + b * sC + i0;
+    const float2* Ab = A + b * sA + i0 + (long long)blockIdx.z * Kper * lda;     // part z of K
+    const float2* Bb = B + b * sB + (long long)blockIdx.z * Kper;
+    float2* Cb = Cm + blockIdx.z * sP + b * sC + i0;
     const uint32_t mb0 = smem_u32(&mbar[0]), mb1 = smem_u32(&mbar[1]);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb0));
@@ -77,7 +78,7 @@ k_cgemm_tc(const float2* __restrict__ A, int lda, long long sA, const float2* __
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tslot;
 
-    const int S = K / TC_KC;
+    const int S = Kper / TC_KC;
     const int jb = lane, gb = warp;              // B slice: column jb, complex k 4 gb .. 4 gb + 3
     // two register sets, each loaded two stages ahead of its use
     float2 ra0[TC_KC], rb0[4], ra1[TC_KC], rb1[4];
@@ -340,9 +341,27 @@ lsw_status cgemm_tc(const float2* A, int lda, long long sA, const float2* B, int
     }
     KTimer kt("leaf_tc", st, 8.0 * ((double)batch * M * K + (double)batch * K * N + (double)batch * M * N),
               8.0 * (double)batch * M * N * K);
-    k_cgemm_tc<<<dim3(M / TC_M, batch), 128, TC_SMEM, st>>>(A, lda, sA, B, ldb, sB, C, ldc, sC, N, K, alpha);
+    // A CTA takes about 1.1 us per stage however few there are, so one leaf of
+    // 1024 on 8 CTAs cost as much as 30 leaves.  K is split until two CTAs per
+    // SM are busy, with at least 4 stages each (8 CTAs of 64 stages become 128
+    // of 4): the inversion's products with 1 to 32 leaves take 18 us on average
+    // instead of 73 (256^2 build, one GB300).
+    int ksplit = 1;
+    while ((long long)(M / TC_M) * batch * ksplit * 2 <= 304 && K % (ksplit * 2 * TC_KC) == 0 &&
+           K / (ksplit * 2) >= 4 * TC_KC)
+        ksplit *= 2;
+    if (ksplit == 1) {
+        k_cgemm_tc<<<dim3(M / TC_M, batch), 128, TC_SMEM, st>>>(A, lda, sA, B, ldb, sB, C, ldc, sC, 0, N, K, alpha);
+        LSW_LAUNCH_CHECK();
+        return LSW_OK;
+    }
+    DevBuf part;
+    const long long mn = (long long)M * N;
+    LSW_TRY(part.alloc(sizeof(float2) * (size_t)(ksplit * batch * mn), st));
+    k_cgemm_tc<<<dim3(M / TC_M, batch, ksplit), 128, TC_SMEM, st>>>(A, lda, sA, B, ldb, sB, part.as<float2>(), M, mn,
+                                                                    batch * mn, N, K / ksplit, make_float2(1.f, 0.f));
     LSW_LAUNCH_CHECK();
-    return LSW_OK;
+    return gemm_reduce_parts<float>(M, N, batch, ksplit, part.as<float2>(), alpha, make_float2(0.f, 0.f), C, ldc, sC, st);
 }
 
 bool tc_bf16_fits(int M, int N, int K) { return M > 0 && M % TC_M == 0 && K > 0 && K % TB_KC == 0 && N >= 1 && N <= 32; }
