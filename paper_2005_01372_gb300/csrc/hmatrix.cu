@@ -378,7 +378,7 @@ lsw_status truncate(const typename Cx<R>::T* Q, int nb, const typename Cx<R>::T*
     LSW_TRY(G.alloc(sizeof(double2) * (size_t)nblk * rp * rp, st));
     LSW_TRY(V.alloc(sizeof(C) * (size_t)nblk * rp * rp, st));
     LSW_TRY(gram64<R>(Yt, mb, rp, (long long)mb * rp, nblk, G.as<double2>(), st));
-    if (sizeof(R) == 4) LSW_TRY(heev_c64(G.as<double2>(), reinterpret_cast<float2*>(V.p), rp, nblk, st));
+    if constexpr (sizeof(R) == 4) LSW_TRY(heev_c64(G.as<double2>(), V.as<float2>(), rp, nblk, st));
     else LSW_TRY(heev_jacobi<R>(G.as<double2>(), V.as<C>(), rp, nblk, st));
     const int rr = std::min(r, rp);
     if (rr < r) {

@@ -992,9 +992,8 @@ k_tsqr_apply(typename Cx<R>::T* __restrict__ Aall, int m, int k, long long sA, i
 // units of rounding of the working precision; a sweep that rotates nothing
 // ends the iteration (the classical threshold rule, which terminates even
 // when rounding keeps the off-diagonal norm above a fixed fraction).
-template <typename R> __device__ __forceinline__ R jacobi_skip() { return sizeof(R) == 8 ? (R)1e-14 : (R)1e-6; }
 
-// Parallel cyclic Jacobi in precision R: each round rotates k/2 disjoint
+// Parallel cyclic Jacobi in precision R (FP64; complex64 sketches take k_eig_gram): each round rotates k/2 disjoint
 // index pairs chosen by the circle method, so every pair is met once per
 // sweep.  Input: FP64 Hermitian G (k x k), scaled by its trace; output: the
 // eigenvectors as columns of V, by decreasing eigenvalue.
@@ -1006,7 +1005,7 @@ __device__ __forceinline__ R jacobi_key(R d) { return isnan(d) ? -INFINITY : d; 
 #define JACOBI_MARK_ROUND (rf[r & 1] = 1)
 template <typename R>
 __global__ void __launch_bounds__(1024)
-k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ Vall, int k, int polish) {
+k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ Vall, int k) {
     typedef typename Cx<R>::T C;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int m = (k + 1) & ~1;                 // even number of players
@@ -1043,20 +1042,10 @@ k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ 
         V[e] = mk((R)((e % k) == (e / k) ? 1 : 0), (R)0);
     }
     __syncthreads();
-    // squared off-diagonal norm relative to the total that the precision
-    // can reach (FP32 rounding stalls near 1e-13): stop there.  A polishing
-    // run (a nearly diagonal input whose small eigenvalues must be resolved
-    // relative to themselves) stops only on a sweep without rotations and
-    // uses a tighter pair threshold.
-    // polish 2 (coarse): a first pass that a polish run will finish
-    const R tol = polish == 1 ? (R)0 : polish == 2 ? (R)1e-6 : (sizeof(R) == 8 ? (R)1e-26 : (R)1e-11);
-    const R skip = polish == 1 ? (sizeof(R) == 8 ? (R)1e-15 : (R)2e-7) : jacobi_skip<R>();
-    // the trace-scaled input is known to ~1e-16 absolute (an FP64-accurate
-    // matrix): entries below that are noise and never trigger a rotation, so
-    // a polish of a matrix with (near-)zero eigenvalues still ends
-    const R floor_abs = polish == 1 ? (R)1e-15 : (R)0;
+    // squared off-diagonal norm relative to the total that FP64 can reach
+    const R tol = (R)1e-26, skip = (R)1e-14;
     __shared__ int rf[2];               // per round (alternating): some pair rotates
-    for (int sweep = 0; sweep < (polish == 1 ? 20 : 40); ++sweep) {
+    for (int sweep = 0; sweep < 40; ++sweep) {
         // both flags clear before the sweep's first round (the block sum
         // below synchronises; the previous round's reads ended at its last barrier)
         if (threadIdx.x < 2) rf[threadIdx.x] = 0;
@@ -1072,7 +1061,7 @@ k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ 
                 if (aa < b) {
                     const R app = A[aa * k + aa].x, aqq = A[b * k + b].x, ac = sqrt(v);
                     if (ac > skip * sqrt(fabs(app * aqq)) && ac > (R)1e-30 * (fabs(app) + fabs(aqq)) &&
-                        ac > floor_abs && ac > 0)
+                        ac > 0)
                         need = 1;
                 }
             }
@@ -1101,7 +1090,7 @@ k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ 
                     // rotate only while the pair is not yet negligible
                     // against its diagonal (relative threshold above rounding)
                     if (ac > skip * sqrt(fabs(app * aqq)) && ac > (R)1e-30 * (fabs(app) + fabs(aqq)) &&
-                        ac > floor_abs && ac > 0) {
+                        ac > 0) {
                         nrot = 1;
                         JACOBI_MARK_ROUND;
                         // t = tan(theta) = sign(d) 2|a_pq| / (|d| + sqrt(d^2 + 4|a_pq|^2)),
@@ -1219,8 +1208,7 @@ k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ 
 #define JACOBI_MARK_ROUND (rr = 1)
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_heev_jacobi_warp(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ Vall, int k, int batch,
-                   int polish) {
+k_heev_jacobi_warp(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ Vall, int k, int batch) {
     typedef typename Cx<R>::T C;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int m = (k + 1) & ~1;
@@ -1246,14 +1234,8 @@ k_heev_jacobi_warp(const double2* __restrict__ Gall, typename Cx<R>::T* __restri
     }
     __syncwarp();
     // the same stopping rules as the CTA version
-    // polish 2 (coarse): a first pass that a polish run will finish
-    const R tol = polish == 1 ? (R)0 : polish == 2 ? (R)1e-6 : (sizeof(R) == 8 ? (R)1e-26 : (R)1e-11);
-    const R skip = polish == 1 ? (sizeof(R) == 8 ? (R)1e-15 : (R)2e-7) : jacobi_skip<R>();
-    // the trace-scaled input is known to ~1e-16 absolute (an FP64-accurate
-    // matrix): entries below that are noise and never trigger a rotation, so
-    // a polish of a matrix with (near-)zero eigenvalues still ends
-    const R floor_abs = polish == 1 ? (R)1e-15 : (R)0;
-    for (int sweep = 0; sweep < (polish == 1 ? 20 : 40); ++sweep) {
+    const R tol = (R)1e-26, skip = (R)1e-14;
+    for (int sweep = 0; sweep < 40; ++sweep) {
         R off = 0, tot = 0;
         int need = 0;                   // some pair is above the rotation threshold
         for (int e = lane; e < k * k; e += 32) {
@@ -1266,7 +1248,7 @@ k_heev_jacobi_warp(const double2* __restrict__ Gall, typename Cx<R>::T* __restri
                 if (aa < b) {
                     const R app = A[aa * k + aa].x, aqq = A[b * k + b].x, ac = sqrt(v);
                     if (ac > skip * sqrt(fabs(app * aqq)) && ac > (R)1e-30 * (fabs(app) + fabs(aqq)) &&
-                        ac > floor_abs && ac > 0)
+                        ac > 0)
                         need = 1;
                 }
             }
@@ -1293,7 +1275,7 @@ k_heev_jacobi_warp(const double2* __restrict__ Gall, typename Cx<R>::T* __restri
                     // rotate only while the pair is not yet negligible
                     // against its diagonal (relative threshold above rounding)
                     if (ac > skip * sqrt(fabs(app * aqq)) && ac > (R)1e-30 * (fabs(app) + fabs(aqq)) &&
-                        ac > floor_abs && ac > 0) {
+                        ac > 0) {
                         JACOBI_COUNT_ROTATION;
                         JACOBI_MARK_ROUND;
                         // the same rotation as the CTA version
@@ -2155,7 +2137,7 @@ lsw_status gram64(const typename Cx<R>::T* Y, int m, int k, long long sY, int ba
 }
 
 template <typename R>
-lsw_status heev_jacobi(const double2* G, typename Cx<R>::T* V, int k, int batch, cudaStream_t st, int polish) {
+lsw_status heev_jacobi(const double2* G, typename Cx<R>::T* V, int k, int batch, cudaStream_t st) {
     typedef typename Cx<R>::T CT;
     if (batch <= 0 || k <= 0) return LSW_OK;
     if (k > 64) return LSW_ERR_INVALID_ARG;
@@ -2170,7 +2152,7 @@ lsw_status heev_jacobi(const double2* G, typename Cx<R>::T* V, int k, int batch,
     }
     if (batch >= 4 * 152) {
         // many matrices: one warp each
-        k_heev_jacobi_warp<R><<<(batch + wpc - 1) / wpc, 32 * wpc, perA * wpc, st>>>(G, V, k, batch, polish);
+        k_heev_jacobi_warp<R><<<(batch + wpc - 1) / wpc, 32 * wpc, perA * wpc, st>>>(G, V, k, batch);
         LSW_LAUNCH_CHECK();
         return LSW_OK;
     }
@@ -2182,7 +2164,7 @@ lsw_status heev_jacobi(const double2* G, typename Cx<R>::T* V, int k, int batch,
     const size_t smb = sizeof(CT) * 3 * (size_t)k * k + sizeof(R) * 4 * (m / 2) + sizeof(int2) * (m / 2);
     // few matrices: the whole CTA of 1024 threads on each (a round is a
     // handful of dependent steps; more threads make each one shorter)
-    k_heev_jacobi<R><<<batch, batch <= 2 * 152 ? 1024 : 256, smb, st>>>(G, V, k, polish);
+    k_heev_jacobi<R><<<batch, batch <= 2 * 152 ? 1024 : 256, smb, st>>>(G, V, k);
     LSW_LAUNCH_CHECK();
     return LSW_OK;
 }
@@ -2407,7 +2389,6 @@ lsw_status norms2(const typename Cx<R>::T* x, long long n, int batch, double* ou
                                 cudaStream_t);                                                                    \
     template lsw_status qr_explicit<R>(Cx<R>::T*, int, int, long long, int, Cx<R>::T*, cudaStream_t);             \
     template lsw_status gram64<R>(const Cx<R>::T*, int, int, long long, int, double2*, cudaStream_t);             \
-    template lsw_status heev_jacobi<R>(const double2*, Cx<R>::T*, int, int, cudaStream_t, int);                        \
     template lsw_status cast_from64<R>(const double2*, Cx<R>::T*, long long, cudaStream_t);                        \
     template lsw_status gaussian_fill<R>(Cx<R>::T*, int, int, long long, int, uint64_t, const uint32_t*,          \
                                          const uint32_t*, cudaStream_t);                                          \
@@ -2418,5 +2399,6 @@ lsw_status norms2(const typename Cx<R>::T* x, long long n, int batch, double* ou
 LSW_INST(float)
 LSW_INST(double)
 #undef LSW_INST
+template lsw_status heev_jacobi<double>(const double2*, double2*, int, int, cudaStream_t);
 
 }  // namespace lsw

@@ -197,8 +197,8 @@ k_gram_c64_reduce_few(const double2* __restrict__ part, int nchunk, int k, doubl
 
 // ------------------------------------------- Cholesky and R^-1 (FP64)
 // One CTA per matrix: G + shift I = Lt D Lt^H (Lt unit lower triangular, D
-// diagonal: the square-root-free Cholesky), then Xt = Lt^-1 and
-// R^-1 = Xt^H D^-1/2 (R = D^1/2 Lt^H, so R^H R = G + shift I).
+// diagonal: the square-root-free Cholesky), with Xt = Lt^-1 formed alongside,
+// and R^-1 = Xt^H D^-1/2 (R = D^1/2 Lt^H, so R^H R = G + shift I).
 // Written for the rate and latency of FP64 on this GPU (2 FP64 lanes per
 // cycle per SM): every multiply-add a thread issues is useful (the trailing
 // triangle is enumerated through a table, not masked out of a square), a
@@ -286,6 +286,10 @@ k_chol_rinv(const double2* __restrict__ Gall, int k, int batch, double shift_rel
             if (i == j) { v.x += shift; v.y = 0.0; }
             A[j * ld + i] = v;
         }
+        for (int e = tid; e < k * ld; e += CH_NT) {
+            const int c = e / ld, i = e - c * ld;
+            X[e] = make_double2(i == c ? 1.0 : 0.0, 0.0);
+        }
         if (tid == 0) {
             const double d0 = G[0].x + shift;
             fail = (d0 > 0.0 && isfinite(d0)) ? 0 : 1;
@@ -301,22 +305,42 @@ k_chol_rinv(const double2* __restrict__ Gall, int k, int batch, double shift_rel
             }
             __syncthreads();
             // trailing triangle: A(i, l) -= A(i, j) U(j, l), j < l <= i; item
-            // 0 (the next pivot) first, on thread 0, which then forms 1 / D(j+1)
-            const int nt = k - 1 - j, T = nt * (nt + 1) / 2;
-            for (int p = tid; p < T; p += CH_NT) {
-                const short2 ab = tri[T - 1 - p];
-                const int i = j + nt - ab.x, l = j + nt - ab.y;
-                const double2 a = A[j * ld + i], u = A[l * ld + j];
-                double2 v = A[l * ld + i];
-                v.x = fma(-a.x, u.x, v.x);
-                v.x = fma(a.y, u.y, v.x);
-                v.y = fma(-a.x, u.y, v.y);
-                v.y = fma(-a.y, u.x, v.y);
-                A[l * ld + i] = v;
-                if (p == 0) {
-                    const double d = v.x;
-                    if (!(d > 0.0) || !isfinite(d)) fail = 1;
-                    dinv[j + 1] = rcp64(d);
+            // 0 (the next pivot) first, on thread 0, which then forms 1 / D(j+1).
+            // In the same phase Xt = Lt^-1 in axpy form: Xt starts as I, row j
+            // is final in every column c <= j by now, and step j removes it
+            // from the rows below: Xt(i, c) -= Lt(i, j) Xt(j, c), Lt(i, j) =
+            // conj(U(j, i)).  Together a step has about k^2 / 2 items whatever j.
+            const int nt = k - 1 - j, T = nt * (nt + 1) / 2, items = T + nt * (j + 1);
+            const float rnt = 1.0f / (float)nt;
+            for (int p = tid; p < items; p += CH_NT) {
+                if (p < T) {
+                    const short2 ab = tri[T - 1 - p];
+                    const int i = j + nt - ab.x, l = j + nt - ab.y;
+                    const double2 a = A[j * ld + i], u = A[l * ld + j];
+                    double2 v = A[l * ld + i];
+                    v.x = fma(-a.x, u.x, v.x);
+                    v.x = fma(a.y, u.y, v.x);
+                    v.y = fma(-a.x, u.y, v.y);
+                    v.y = fma(-a.y, u.x, v.y);
+                    A[l * ld + i] = v;
+                    if (p == 0) {
+                        const double d = v.x;
+                        if (!(d > 0.0) || !isfinite(d)) fail = 1;
+                        dinv[j + 1] = rcp64(d);
+                    }
+                } else {
+                    // e = c * nt + (i - j - 1); the float quotient is exact here
+                    // (e < 4096, nt < 64: the fraction is at least 1 / (2 nt) from an integer)
+                    const int e = p - T;
+                    const int c = (int)(((float)e + 0.5f) * rnt), i = j + 1 + (e - c * nt);
+                    const double2 u = A[i * ld + j], xt = X[c * ld + j];
+                    double2 v = X[c * ld + i];
+                    // v -= conj(u) xt
+                    v.x = fma(-u.x, xt.x, v.x);
+                    v.x = fma(-u.y, xt.y, v.x);
+                    v.y = fma(-u.x, xt.y, v.y);
+                    v.y = fma(u.y, xt.x, v.y);
+                    X[c * ld + i] = v;
                 }
             }
             __syncthreads();
@@ -330,32 +354,6 @@ k_chol_rinv(const double2* __restrict__ Gall, int k, int batch, double shift_rel
         for (int e = tid; e < k * k; e += CH_NT) { Rout[e].x = NAN; Rout[e].y = NAN; }
         if (need2 && tid == 0) need2[mat] = 0;
         return;
-    }
-    // Xt = Lt^-1 in axpy form, every column at once: Xt starts as I; after
-    // step t - 1 row t is final in every column c <= t, and step t removes it
-    // from the rows below: Xt(i, c) -= Lt(i, t) Xt(t, c), Lt(i, t) = conj(U(t, i)).
-    for (int e = tid; e < k * ld; e += CH_NT) {
-        const int c = e / ld, i = e - c * ld;
-        X[e] = make_double2(i == c ? 1.0 : 0.0, 0.0);
-    }
-    __syncthreads();
-    for (int t = 0; t < k - 1; ++t) {
-        const int nr = k - 1 - t, n = nr * (t + 1);
-        const float rnr = 1.0f / (float)nr;
-        for (int e = tid; e < n; e += CH_NT) {
-            // e = c * nr + (i - t - 1); the float quotient is exact here
-            // (e < 4096, nr < 64: the fraction is at least 1 / (2 nr) from an integer)
-            const int c = (int)(((float)e + 0.5f) * rnr), i = t + 1 + (e - c * nr);
-            const double2 u = A[i * ld + t], xt = X[c * ld + t];
-            double2 v = X[c * ld + i];
-            // v -= conj(u) xt
-            v.x = fma(-u.x, xt.x, v.x);
-            v.x = fma(-u.y, xt.y, v.x);
-            v.y = fma(-u.x, xt.y, v.y);
-            v.y = fma(u.y, xt.x, v.y);
-            X[c * ld + i] = v;
-        }
-        __syncthreads();
     }
     // D^-1/2 for every column at once (reuses dinv)
     for (int j = tid; j < k; j += CH_NT) dinv[j] = rsqrt64(A[j * ld + j].x);
@@ -446,77 +444,220 @@ k_rmul_dot2(float2* __restrict__ Y, int m, int k, long long sY, const double2* _
     }
 }
 
-// ------------------------------- Rayleigh-Ritz projection (FP64 accuracy)
-// B = V0^H G V0 for FP32 approximate eigenvectors V0 of the FP64 Hermitian G,
-// formed with FP64 accuracy in FP32 arithmetic: G = Ghi + Glo (two FP32
-// parts), W = G V0 by Dot2 over the Ghi terms with the Glo terms added to the
-// compensation, kept as the pair Whi + Wlo; then B = V0^H (Whi + Wlo) the
-// same way.  One CTA per matrix; B is written Hermitian (upper triangle
-// computed, lower mirrored).  Small eigenvalues of G that FP32 could not
-// separate inside G (below ~1e-7 of the largest) sit on B's diagonal with
-// their own exponents, where an FP32 Jacobi resolves them.
-__global__ void __launch_bounds__(1024)
-k_rr_project(const double2* __restrict__ Gall, const float2* __restrict__ V0all, int k, double2* __restrict__ Ball) {
+// --------------------------- eigenvectors of a Gram matrix (FP64 accuracy)
+// The eigenvectors of G = Y^H Y (FP64-accurate, eigenvalues spread over up to
+// 16 decades) are the left singular vectors of its Cholesky factor L, and
+// one-sided Jacobi on L's columns finds those in FP32 however small their
+// singular values are against the largest: the factor carries the square roots
+// of the eigenvalues column by column, and a pair of columns is rotated by
+// their own inner product alone (Veselic and Hari, Numer. Math. 56, 1989).
+// One CTA per matrix.
+//   1. The trace is scaled to 1 and the indices sorted by the diagonal's
+//      thousands (2^10): a sketch's own order is nearly decreasing and saves
+//      sweeps, and a floored pivot of step 2 still comes last.
+//   2. G = Lt D Lt^H in FP64 (square-root-free, as in k_chol_rinv).  A pivot
+//      not above 1e-15, the accuracy of G itself, becomes 1e-15 with nothing
+//      below it: no restart.
+//   3. W = L, times 2^20 so that all squares are normal FP32 numbers.  Rounds of
+//      disjoint column pairs (circle method), sixteen lanes per pair: the
+//      pair's norms and inner product (four shuffles), the rotation, the update, one
+//      barrier per round.  A pair is left alone below 3e-7 of its
+//      norms (twice the rounding of a 64-term inner product); a sweep without a
+//      rotation ends.
+//   4. Columns divided by their norms, by decreasing norm, rows put back.
+// Bound by latency: for 30 x 30 about 25 us of FP64 chains in 2 and 8.5 us per
+// sweep in 3 (0.3 us a round), 5 to 6 sweeps, 78 us in all (one GB300).  A
+// coarse FP32 two-sided Jacobi, a Rayleigh-Ritz projection in split FP32 and a
+// second Jacobi that resolved the small eigenvalues took 67 + 16 + 122 us and a
+// product, and left complex64 sketches 1e-6 to 1e-5 from their FP64
+// counterparts where this leaves 3e-7 to 2e-6.
+__device__ __forceinline__ float rsqrt_newton(float a) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a));
+    return fmaf(0.5f * y, fmaf(-a * y, y, 1.f), y);
+}
+
+template <int RPL>
+__global__ void __launch_bounds__(RPL * 128)
+k_eig_gram(const double2* __restrict__ Gall, float2* __restrict__ Vall, int k) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    const int kk = k * k;
-    float2* Ghi = reinterpret_cast<float2*>(sm_raw);
-    float2* Glo = Ghi + kk;
-    float2* V = Glo + kk;
-    float2* Whi = V + kk;
-    float2* Wlo = Whi + kk;
-    const double2* G = Gall + (long long)blockIdx.x * kk;
-    const float2* V0 = V0all + (long long)blockIdx.x * kk;
-    double2* B = Ball + (long long)blockIdx.x * kk;
-    for (int e = threadIdx.x; e < kk; e += blockDim.x) {
-        const double2 g = G[e];
-        const float hx = (float)g.x, hy = (float)g.y;
-        Ghi[e] = make_float2(hx, hy);
-        Glo[e] = make_float2((float)(g.x - (double)hx), (float)(g.y - (double)hy));
-        V[e] = V0[e];
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int LW = 16 * RPL + 1;                                // rows of W, zero beyond k, and a pad
+    const int ld = k + 1;
+    double2* A = reinterpret_cast<double2*>(sm_raw);                // k x ld, then
+    double* dinv = reinterpret_cast<double*>(A + (size_t)k * ld);   // 1 / D(j), 0 for a floored pivot
+    double* dval = dinv + k;                                        // D(j)
+    const int m = (k + 1) & ~1;
+    float2* W = reinterpret_cast<float2*>(dval + k);                // m columns of LW
+    short2* tri = reinterpret_cast<short2*>(W + (size_t)m * LW);    // p -> (a, b), a <= b
+    __shared__ double trs;
+    __shared__ int order[64];
+    __shared__ float key[64];
+    __shared__ int rotated;
+    const double2* G = Gall + (long long)blockIdx.x * k * k;
+    const int ntri = k * (k - 1) / 2;
+    for (int p = tid; p < ntri; p += nt) {
+        int a, b;
+        tri_pair(p, a, b);
+        tri[p] = make_short2((short)a, (short)b);
+    }
+    if (warp == 0) {
+        double t = 0;
+        for (int i = lane; i < k; i += 32) t += fabs(G[i * k + i].x);
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) trs = t > 0 ? 1.0 / t : 0.0;
+    }
+    // position of each index by decreasing key (ties by index, NaN last)
+    auto sort_keys = [&]() {
+        for (int i = tid; i < k; i += nt) {
+            const float a = isnan(key[i]) ? -INFINITY : key[i];
+            int pos = 0;
+            for (int j = 0; j < k; ++j) {
+                const float b = isnan(key[j]) ? -INFINITY : key[j];
+                pos += (b > a || (b == a && j < i)) ? 1 : 0;
+            }
+            order[pos] = i;
+        }
+    };
+    __syncthreads();
+    for (int i = tid; i < k; i += nt) {
+        const float d = (float)(G[i * k + i].x * trs);
+        key[i] = d > 0.f ? (float)(ilogbf(d) / 10) : d == 0.f ? -100.f : d;
     }
     __syncthreads();
-    // W(i, j) = sum_t G(i, t) V(t, j)
-    for (int e = threadIdx.x; e < kk; e += blockDim.x) {
+    sort_keys();
+    __syncthreads();
+    const int row0 = lane < k ? order[lane] : 0, row1 = lane + 32 < k ? order[lane + 32] : 0;
+    for (int e = tid; e < k * k; e += nt) {
         const int j = e / k, i = e - j * k;
-        float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
-        for (int t = 0; t < k; ++t) {
-            const float2 gh = Ghi[t * k + i], gl = Glo[t * k + i], v = V[j * k + t];
-            dot2(gh.x, v.x, sr, cr);
-            dot2(-gh.y, v.y, sr, cr);
-            dot2(gh.x, v.y, si, ci);
-            dot2(gh.y, v.x, si, ci);
-            cr = fmaf(gl.x, v.x, fmaf(-gl.y, v.y, cr));
-            ci = fmaf(gl.x, v.y, fmaf(gl.y, v.x, ci));
-        }
-        // renormalise the pair so that Whi carries the leading bits
-        const float hr = __fadd_rn(sr, cr), hi = __fadd_rn(si, ci);
-        Whi[e] = make_float2(hr, hi);
-        Wlo[e] = make_float2(__fsub_rn(cr, __fsub_rn(hr, sr)), __fsub_rn(ci, __fsub_rn(hi, si)));
+        if (i < j) continue;
+        const double2 v = G[order[j] * k + order[i]];
+        A[j * ld + i] = make_double2(v.x * trs, i == j ? 0.0 : v.y * trs);
     }
     __syncthreads();
-    // B(i, j) = sum_t conj(V(t, i)) W(t, j), i <= j
-    const int npair = k * (k + 1) / 2;
-    for (int p = threadIdx.x; p < npair; p += blockDim.x) {
-        int i, j;
-        tri_pair(p, i, j);
-        float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
-        for (int t = 0; t < k; ++t) {
-            const float2 a = V[i * k + t], wh = Whi[j * k + t], wl = Wlo[j * k + t];
-            // conj(a) * w = (ax wx + ay wy) + i (ax wy - ay wx)
-            dot2(a.x, wh.x, sr, cr);
-            dot2(a.y, wh.y, sr, cr);
-            dot2(a.x, wh.y, si, ci);
-            dot2(-a.y, wh.x, si, ci);
-            cr = fmaf(a.x, wl.x, fmaf(a.y, wl.y, cr));
-            ci = fmaf(a.x, wl.y, fmaf(-a.y, wl.x, ci));
+    constexpr double tiny = 1e-15;
+    if (tid == 0) {
+        const double d = A[0].x;
+        dval[0] = d > tiny ? d : tiny;
+        dinv[0] = d > tiny ? rcp64(d) : 0.0;
+    }
+    __syncthreads();
+    for (int j = 0; j < k - 1; ++j) {
+        // column j of Lt, kept conjugated in row j: U(j, i) = conj(A(i, j)) / D(j)
+        const double dj = dinv[j];
+        for (int i = j + 1 + tid; i < k; i += nt) {
+            const double2 v = A[j * ld + i];
+            A[i * ld + j] = make_double2(v.x * dj, -v.y * dj);
         }
-        const double br = (double)sr + (double)cr, bi = (double)si + (double)ci;
-        if (i == j) {
-            B[j * k + i] = make_double2(br, 0.0);
-        } else {
-            B[j * k + i] = make_double2(br, bi);
-            B[i * k + j] = make_double2(br, -bi);
+        __syncthreads();
+        // trailing triangle: A(i, l) -= A(i, j) U(j, l); item 0, the next pivot, first
+        const int n = k - 1 - j, T = n * (n + 1) / 2;
+        for (int p = tid; p < T; p += nt) {
+            const short2 ab = tri[T - 1 - p];
+            const int i = j + n - ab.x, l = j + n - ab.y;
+            const double2 a = A[j * ld + i], u = A[l * ld + j];
+            double2 v = A[l * ld + i];
+            v.x = fma(-a.x, u.x, v.x);
+            v.x = fma(a.y, u.y, v.x);
+            v.y = fma(-a.x, u.y, v.y);
+            v.y = fma(-a.y, u.x, v.y);
+            A[l * ld + i] = v;
+            if (p == 0) {
+                dval[j + 1] = v.x > tiny ? v.x : tiny;
+                dinv[j + 1] = v.x > tiny ? rcp64(v.x) : 0.0;
+            }
         }
+        __syncthreads();
+    }
+    // W(i, j) = Lt(i, j) sqrt(D(j)) 2^20, zero above the diagonal and beyond k
+    for (int e = tid; e < m * LW; e += nt) {
+        const int j = e / LW, i = e - j * LW;
+        float2 w = make_float2(0.f, 0.f);
+        if (i >= j && i < k) {
+            const float s = sqrtf((float)dval[j]) * 1048576.f;
+            if (i == j) w.x = s;
+            else w = make_float2((float)A[i * ld + j].x * s, -(float)A[i * ld + j].y * s);
+        }
+        W[e] = w;
+    }
+    if (tid == 0) rotated = 0;
+    __syncthreads();
+    // pair i of round r: columns (m - 1, r) or (r + i, r - i) mod m - 1; an
+    // odd k's extra column is zero and never rotates
+    const int i = tid >> 4, l16 = tid & 15;
+    const bool live = i < m / 2;
+    const int lim = (m - 1) * LW;
+    for (int sweep = 0; sweep < 20; ++sweep) {
+        int po = (i == 0 ? m - 1 : i) * LW, qo = (live && i > 0 ? m - 1 - i : 0) * LW;
+        if (!live) po = 0;
+        for (int r = 0; r < m - 1; ++r) {
+            float2 *wp = W + po + l16, *wq = W + qo + l16;
+            float2 a[RPL], b[RPL];
+#pragma unroll
+            for (int u = 0; u < RPL; ++u) {
+                a[u] = wp[16 * u];
+                b[u] = wq[16 * u];
+            }
+            if (i) { po += LW; if (po == lim) po = 0; }
+            qo += LW;
+            if (qo == lim) qo = 0;
+            // norms and w_p^H w_q
+            float al = 0.f, be = 0.f;
+            float2 ga = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < RPL; ++u) {
+                al = fmaf(a[u].x, a[u].x, fmaf(a[u].y, a[u].y, al));
+                be = fmaf(b[u].x, b[u].x, fmaf(b[u].y, b[u].y, be));
+                cfmac(ga, a[u], b[u]);
+            }
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) {
+                al += __shfl_xor_sync(0xffffffffu, al, o);
+                be += __shfl_xor_sync(0xffffffffu, be, o);
+                ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
+                ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
+            }
+            const float g2 = fmaf(ga.x, ga.x, ga.y * ga.y);
+            if (live && g2 > 9e-14f * (al * be)) {
+                // the rotation that makes w_p, w_q orthogonal, by the half angle:
+                // h = sqrt(d^2 + 4 |g|^2), cos^2 = (1 + |d| / h) / 2, sin cos = |g| / h
+                const float d = be - al, rg = rsqrt_newton(g2);
+                const float rh = rsqrt_newton(fmaf(4.f, g2, d * d));
+                const float x = fmaf(0.5f * fabsf(d), rh, 0.5f), rx = rsqrt_newton(x);
+                const float cs = x * rx, sn = (d >= 0 ? g2 : -g2) * rg * rh * rx;
+                const float2 em = make_float2(ga.x * rg, -ga.y * rg);       // e^{-i phi}, g = |g| e^{i phi}
+#pragma unroll
+                for (int u = 0; u < RPL; ++u) {
+                    const float2 e = cmul(em, b[u]);
+                    wp[16 * u] = make_float2(cs * a[u].x - sn * e.x, cs * a[u].y - sn * e.y);
+                    wq[16 * u] = make_float2(sn * a[u].x + cs * e.x, sn * a[u].y + cs * e.y);
+                }
+                if (l16 == 0) rotated = sweep + 1;
+            }
+            __syncthreads();
+        }
+        if (rotated != sweep + 1) break;        // every thread reads it between the same two barriers
+        __syncthreads();
+    }
+    // norms (squared) as sort keys, columns normalised, rows back in place
+    float2* Vo = Vall + (long long)blockIdx.x * k * k;
+    for (int j = warp; j < k; j += nt >> 5) {
+        const float2 a0 = lane < k ? W[j * LW + lane] : make_float2(0.f, 0.f);
+        const float2 a1 = lane + 32 < k ? W[j * LW + lane + 32] : make_float2(0.f, 0.f);
+        float s = fmaf(a0.x, a0.x, a0.y * a0.y) + fmaf(a1.x, a1.x, a1.y * a1.y);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float f = rsqrt_newton(s);
+        if (lane < k) W[j * LW + lane] = make_float2(a0.x * f, a0.y * f);
+        if (lane + 32 < k) W[j * LW + lane + 32] = make_float2(a1.x * f, a1.y * f);
+        if (lane == 0) key[j] = s;
+    }
+    __syncthreads();
+    sort_keys();
+    __syncthreads();
+    for (int j = warp; j < k; j += nt >> 5) {
+        const float2* w = W + order[j] * LW;
+        if (lane < k) Vo[j * k + row0] = w[lane];
+        if (lane + 32 < k) Vo[j * k + row1] = w[lane + 32];
     }
 }
 
@@ -585,26 +726,20 @@ lsw_status heev_c64(const double2* G, float2* V, int k, int batch, cudaStream_t 
     // with eigenvectors, 9 k^3 real flops for real symmetric, four times that
     // for complex (reads and writes of the k x k matrices only, in bytes)
     KTimer kt("heev", st, 24.0 * (double)k * k * batch, 36.0 * (double)k * k * k * batch);
-    const size_t kk = (size_t)k * k;
-    DevBuf V0, B, Z;
-    LSW_TRY(V0.alloc(sizeof(float2) * kk * batch, st));
-    LSW_TRY(B.alloc(sizeof(double2) * kk * batch, st));
-    LSW_TRY(Z.alloc(sizeof(float2) * kk * batch, st));
-    LSW_TRY(heev_jacobi<float>(G, V0.as<float2>(), k, batch, st, 2));
+    const int rpl = k <= 32 ? 2 : 4;
+    const size_t smem = sizeof(double2) * (size_t)k * (k + 1) + 2 * sizeof(double) * k +
+                        sizeof(float2) * (size_t)((k + 1) & ~1) * (16 * rpl + 1) +
+                        sizeof(short2) * (size_t)(k * (k - 1) / 2 + 1);
     static std::atomic<bool> attr{false};
     if (!attr.load()) {
-        LSW_CUDA(cudaFuncSetAttribute(k_rr_project, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        LSW_CUDA(cudaFuncSetAttribute(k_eig_gram<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024));
+        LSW_CUDA(cudaFuncSetAttribute(k_eig_gram<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024));
         attr.store(true);
     }
-    // few matrices (the critical path of the recursive inversion): a CTA of
-    // 1024 threads on each
-    k_rr_project<<<batch, batch <= 2 * 152 ? 1024 : 128, sizeof(float2) * 5 * kk, st>>>(G, V0.as<float2>(), k,
-                                                                                       B.as<double2>());
+    if (rpl == 2) k_eig_gram<2><<<batch, 256, smem, st>>>(G, V, k);
+    else k_eig_gram<4><<<batch, 512, smem, st>>>(G, V, k);
     LSW_LAUNCH_CHECK();
-    LSW_TRY(heev_jacobi<float>(B.as<double2>(), Z.as<float2>(), k, batch, st, 1));
-    const float2 one = make_float2(1.f, 0.f), zero = make_float2(0.f, 0.f);
-    return gemm<float>('N', 'N', k, k, k, one, V0.as<float2>(), k, (long long)kk, Z.as<float2>(), k, (long long)kk,
-                       zero, V, k, (long long)kk, batch, st);
+    return LSW_OK;
 }
 
 // Thin QR of complex64 sketch blocks, Q returned in place of A (m x k, ld m,
