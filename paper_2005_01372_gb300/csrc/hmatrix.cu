@@ -170,6 +170,7 @@ struct HStoreB {
     int L = 0, r = 0, n = 0;
     int rp = 0;                       // columns per block of the tiled levels
     uint32_t* D = nullptr;
+    int dlay = 0;                     // FAC_* storage of the leaves (rank: their nL columns)
     std::vector<uint32_t*> U, W;
     std::vector<int> ulay, wlay;      // FAC_* storage of each level's U and W
     size_t bytes = 0;
@@ -1342,17 +1343,16 @@ __global__ void k_to_bf16(const float2* __restrict__ src, uint32_t* __restrict__
 
 // Y_b = D_b X_b with BF16 leaves on the CUDA cores (when the tensor-core
 // kernel does not take the shape or is switched off): thread per output.
-__global__ void k_leaf_bf16(const uint32_t* __restrict__ D, const float2* __restrict__ X, float2* __restrict__ Y,
-                            int nL, int nleaf, int k, int ld) {
+__global__ void k_leaf_bf16(const uint32_t* __restrict__ D, int dlay, const float2* __restrict__ X,
+                            float2* __restrict__ Y, int nL, int nleaf, int k, int ld) {
     const long long tot = (long long)nL * nleaf * k;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
         const int i = (int)(e % nL);
         const long long rest = e / nL;
         const int b = (int)(rest % nleaf), j = (int)(rest / nleaf);
-        const uint32_t* Db = D + (size_t)b * nL * nL;
         const float2* x = X + (size_t)j * ld + (size_t)b * nL;
         float2 acc = make_float2(0.f, 0.f);
-        for (int t = 0; t < nL; ++t) cfma(acc, ldfac(Db + (size_t)t * nL + i), x[t]);
+        for (int t = 0; t < nL; ++t) cfma(acc, ldfac(D + fac_index(dlay, nL, nL, nL, b, i, t)), x[t]);
         Y[(size_t)j * ld + (size_t)b * nL + i] = acc;
     }
 }
@@ -1367,7 +1367,10 @@ lsw_status to_bf16(const HStore<float>& H, HStoreB& B, cudaStream_t st) {
     const long long nd = (long long)H.n * nL, nf = (long long)H.n * H.r;
     LSW_TRY(pool_alloc(reinterpret_cast<void**>(&B.D), sizeof(uint32_t) * nd));
     B.bytes = sizeof(uint32_t) * nd;
-    k_to_bf16<<<gridn(nd), 256, 0, st>>>(H.D, B.D, nd);
+    // leaves of the sizes the tensor-core kernel takes are stored as its tiles
+    B.dlay = leaf_tc_tiled(nL) ? FAC_TILE_A : FAC_PLAIN;
+    if (B.dlay == FAC_TILE_A) k_to_bf16_fac<<<gridn(nd), 256, 0, st>>>(H.D, B.D, FAC_TILE_A, nL, nL, nL, 1LL << H.L);
+    else k_to_bf16<<<gridn(nd), 256, 0, st>>>(H.D, B.D, nd);
     LSW_LAUNCH_CHECK();
     B.U.assign(H.L + 1, nullptr);
     B.W.assign(H.L + 1, nullptr);
@@ -1406,12 +1409,11 @@ lsw_status hmv_bf16(const HStoreB& B, const float2* X, int k, float2* Y, cudaStr
     const int n = B.n, L = B.L, r = B.r, nL = B.nl(L), nleaf = 1 << L;
     for (int c0 = 0; c0 < k; c0 += 32) {
         const int kc = std::min(32, k - c0);
-        if (tc_gemm_enabled() && tc_bf16_fits(nL, kc, nL)) {
-            LSW_TRY(cgemm_tc_bf16(B.D, nL, (long long)nL * nL, X + (size_t)c0 * n, n, nL, Y + (size_t)c0 * n, n, nL, nL,
-                                  kc, nL, make_float2(1.f, 0.f), nleaf, st));
+        if (tc_gemm_enabled() && B.dlay == FAC_TILE_A) {
+            LSW_TRY(leaf_tc_bf16(B.D, nL, nleaf, X + (size_t)c0 * n, n, kc, Y + (size_t)c0 * n, st));
         } else {
-            k_leaf_bf16<<<gridn((long long)n * kc), 256, 0, st>>>(B.D, X + (size_t)c0 * n, Y + (size_t)c0 * n, nL,
-                                                                 nleaf, kc, n);
+            k_leaf_bf16<<<gridn((long long)n * kc), 256, 0, st>>>(B.D, B.dlay, X + (size_t)c0 * n, Y + (size_t)c0 * n,
+                                                                 nL, nleaf, kc, n);
             LSW_LAUNCH_CHECK();
         }
     }

@@ -3,6 +3,7 @@
 // Sec. 2.4 on BF16 storage):
 //     partial:  P_chunk = F_chunk^H X[rows of the sibling block]   (r x k)
 //     apply:    Y[rows] += sum over levels of G_b[rows] T_b         (rows x k)
+//     leaves:   Y[rows of a leaf] = D_leaf X[rows of the leaf]
 // with k <= 32 vectors.  Complex as real, as in the leaf products: an operand
 // row holds (re, im) pairs along K, the other operand's real columns 0..NH-1
 // carry the real parts of the result and NH..2NH-1 the imaginary parts (NH =
@@ -490,6 +491,153 @@ k_lr_apply_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2* 
     }
 }
 
+// Dense leaves: work item = 128 rows of one leaf, stages of LDK = 32 leaf
+// columns.  The leaves are stored as operand tiles (FAC_TILE_A with the leaf's
+// nL columns as its rank), so a stage is one copy of 16 KB; the vectors' 32
+// rows come raw and become B'' hi/lo (4 K-step tiles of 2 NH rows).  Bound by
+// reading the leaves: 256 leaves of 1024 x 1024 (1.07 GB) times 16 vectors took
+// 331 us when every thread loaded its rows of a column-major leaf and a block
+// barrier ended each stage; now 206 us (5.2 TB/s).
+constexpr int LDK = 32;
+constexpr int LPAD = LDK * 8 + 16;
+template <int NH>
+__global__ void __launch_bounds__(WS_THREADS)
+k_leaf_ws(const uint32_t* __restrict__ D, int nL, int nleaf, const float2* __restrict__ X, long long ld, int k,
+          float2* __restrict__ Y, int ns) {
+    constexpr int N = 2 * NH;
+    constexpr uint32_t ID = idesc(1, LM, N);
+    constexpr int KSP = LDK / 8;
+    constexpr int KB = N * 32;
+    constexpr int LBP = KSP * KB;
+    constexpr uint32_t SA = KSP * 4096u;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tiles = nL / LM, nwork = nleaf * tiles, S = nL / LDK;
+    const int XS = k * LPAD;
+    unsigned char* Abuf = sm;
+    unsigned char* Xbuf = sm + (size_t)ns * SA;
+    unsigned char* Bbuf = sm + (((size_t)ns * SA + (size_t)ns * XS + 1023) & ~(size_t)1023);
+    const WsBars bars = ws_at(Bbuf + 4 * LBP, ns);
+    const uint32_t tmem = ws_setup(bars, ns, 2 * N);
+    if (warp == WS_PROD) {
+        int g = 0;
+        bool go = true;
+        for (int w = blockIdx.x; w < nwork && go; w += gridDim.x) {
+            const int leaf = w / tiles, o = (w - leaf * tiles) * LM;
+            for (int s = 0; s < S; ++s, ++g) {
+                const int slot = g % ns;
+                if (g >= ns && !ws_wait(bars, bars.empty + slot, (uint32_t)((g / ns - 1) & 1))) { go = false; break; }
+                const uint32_t fb = smem_u32(bars.full + slot);
+                if (lane == 0) mbar_expect_tx(fb, SA + (uint32_t)k * LDK * 8u);
+                __syncwarp();
+                if (lane == 0)
+                    bulk_g2s(smem_u32(Abuf + (size_t)slot * SA),
+                             D + fac_index(FAC_TILE_A, nL, nL, nL, leaf, o, s * LDK), SA, fb);
+                if (lane < k)
+                    bulk_g2s(smem_u32(Xbuf + (size_t)slot * XS + lane * LPAD),
+                             X + (long long)leaf * nL + s * LDK + lane * ld, (uint32_t)LDK * 8u, fb);
+            }
+        }
+        if (lane == 0) bars.counts[0] = g;
+    } else if (warp == WS_MMA) {
+        if (lane == 0) {
+            int g = 0, li = 0;
+            bool go = true;
+            for (int w = blockIdx.x; w < nwork && go; w += gridDim.x, ++li) {
+                if (li >= 2 && !ws_wait(bars, bars.acce + (li & 1), (uint32_t)(((li - 2) >> 1) & 1))) break;
+                const uint32_t dt = tmem + (uint32_t)((li & 1) * N);
+                for (int s = 0; s < S; ++s, ++g) {
+                    const int slot = g % ns, bsel = g & 1;
+                    if (!ws_wait(bars, bars.bready + bsel, (uint32_t)((g >> 1) & 1))) { go = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t a = smem_u32(Abuf + (size_t)slot * SA);
+                    const uint32_t bh = smem_u32(Bbuf + (size_t)bsel * 2 * LBP), bl = bh + LBP;
+#pragma unroll
+                    for (int ks = 0; ks < KSP; ++ks) {
+                        const uint64_t da = sdesc_sbo(a + ks * 4096, 256);
+                        mma_bf16(dt, da, sdesc_sbo(bh + ks * KB, 256), ID, (s > 0 || ks > 0) ? 1u : 0u);
+                        mma_bf16(dt, da, sdesc_sbo(bl + ks * KB, 256), ID, 1u);
+                    }
+                    mma_commit(smem_u32(bars.empty + slot));
+                    mma_commit(smem_u32(bars.bfree + bsel));
+                    if (s == S - 1) mma_commit(smem_u32(bars.accf + (li & 1)));
+                    bars.counts[1] = g + 1;
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp >= WS_EPI) {
+        float d[N];
+        int li = 0;
+        for (int w = blockIdx.x; w < nwork; w += gridDim.x, ++li) {
+            if (!ws_wait(bars, bars.accf + (li & 1), (uint32_t)((li >> 1) & 1))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t taddr = tmem + (uint32_t)((li & 1) * N) + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll
+            for (int col = 0; col < N; col += 16) tmem_ld16(taddr + col, d + col);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(bars.acce + (li & 1)));
+            // items are consecutive runs of 128 rows of the whole matrix
+            const long long row = (long long)w * LM + (warp & 3) * 32 + lane;
+#pragma unroll
+            for (int jj = 0; jj < NH; ++jj)
+                if (jj < k) Y[jj * ld + row] = make_float2(d[jj], d[NH + jj]);
+        }
+    } else {
+        // builders: half-K-steps warp, warp + 6 of each stage
+        int g = 0;
+        bool go = true;
+        for (int w = blockIdx.x; w < nwork && go; w += gridDim.x) {
+            for (int s = 0; s < S; ++s, ++g) {
+                const int slot = g % ns, bsel = g & 1;
+                if (!ws_wait(bars, bars.full + slot, (uint32_t)((g / ns) & 1))) { go = false; break; }
+                if (g >= 2 && !ws_wait(bars, bars.bfree + bsel, (uint32_t)(((g - 2) >> 1) & 1))) { go = false; break; }
+                unsigned char* Bhi = Bbuf + (size_t)bsel * 2 * LBP;
+                unsigned char* Blo = Bhi + LBP;
+                if (lane < NH) {
+                    const float4* xs = reinterpret_cast<const float4*>(Xbuf + (size_t)slot * XS + lane * LPAD);
+                    for (int q = warp; q < 2 * KSP; q += WS_BUILDERS) {
+                        const int ks = q >> 1, h = q & 1;
+                        float2 x[4];
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            const float4 v = lane < k ? xs[2 * q + t] : make_float4(0.f, 0.f, 0.f, 0.f);
+                            x[2 * t] = make_float2(v.x, v.y);
+                            x[2 * t + 1] = make_float2(v.z, v.w);
+                        }
+                        uint4 rh, rl, ih, il;
+                        b_words(x, 0, rh, rl, ih, il);
+                        const int ob = ks * KB;
+                        *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane, h)) = rh;
+                        *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane, h)) = rl;
+                        *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane + NH, h)) = ih;
+                        *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane + NH, h)) = il;
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(bars.bready + bsel));
+            }
+        }
+        if (warp == 0 && lane == 0) bars.counts[2] = g;
+    }
+    if (ws_close(bars, tmem, 2 * N, ns)) {
+        for (int w = blockIdx.x; w < nwork; w += gridDim.x)
+            for (int e = threadIdx.x; e < LM * k; e += blockDim.x) {
+                const int jj = e / LM, rr = e - jj * LM;
+                Y[jj * ld + (long long)w * LM + rr] = make_float2(qnan(), qnan());
+            }
+        if (threadIdx.x == 0) atomicAdd(&g_lr_tc_timeouts, 1);
+    }
+}
+
+size_t leaf_ws_smem(int NH, int k, int ns) {
+    const size_t pre = ((size_t)ns * (LDK / 8) * 4096 + (size_t)ns * k * LPAD + 1023) & ~(size_t)1023;
+    return pre + 4 * (size_t)(LDK / 8) * (2 * NH) * 32 + ws_bar_bytes(ns);
+}
+
 size_t partial_ws_smem(int NH, int rp, int k, int ns) {
     const size_t SAS = ((size_t)rp * 4 * LKC + 1023) & ~(size_t)1023;
     const size_t pre = ((size_t)ns * SAS + (size_t)ns * k * XPAD + 1023) & ~(size_t)1023;
@@ -563,7 +711,38 @@ lsw_status apply_launch(const LrLevels<float2, uint32_t>& lv, int m, int r, int 
     return LSW_OK;
 }
 
+template <int NH>
+lsw_status leaf_launch(const uint32_t* D, int nL, int nleaf, const float2* X, long long ld, int k, float2* Y,
+                       cudaStream_t st) {
+    static std::atomic<bool> attr{false};
+    if (!attr.load()) {
+        LSW_CUDA(cudaFuncSetAttribute(k_leaf_ws<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap));
+        LSW_CUDA(cudaFuncSetAttribute(k_leaf_ws<NH>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      (int)cudaSharedmemCarveoutMaxShared));
+        attr.store(true);
+    }
+    // ring depth: 4 stages fit two CTAs to an SM (98 KB at 16 vectors), 3 at 32
+    int ns = 4;
+    if (leaf_ws_smem(NH, k, ns) > 112 * 1024) ns = 3;
+    const size_t smem = leaf_ws_smem(NH, k, ns);
+    int grid = 0;
+    LSW_TRY(persistent_grid(smem, 4 * NH, nleaf * (nL / LM), grid));
+    k_leaf_ws<NH><<<grid, WS_THREADS, smem, st>>>(D, nL, nleaf, X, ld, k, Y, ns);
+    LSW_LAUNCH_CHECK();
+    return LSW_OK;
+}
+
 }  // namespace
+
+bool leaf_tc_tiled(int nL) { return nL % LM == 0 && nL % LDK == 0; }
+
+lsw_status leaf_tc_bf16(const uint32_t* D, int nL, int nleaf, const float2* X, long long ld, int k, float2* Y,
+                        cudaStream_t st) {
+    if (!leaf_tc_tiled(nL) || k < 1 || k > 32 || nleaf < 1 || (ld & 1)) return LSW_ERR_INVALID_ARG;
+    KTimer kt("leaf_tc", st, 4.0 * (double)nleaf * nL * nL + 16.0 * (double)nleaf * nL * k,
+              8.0 * (double)nleaf * nL * nL * k);
+    return k <= 16 ? leaf_launch<16>(D, nL, nleaf, X, ld, k, Y, st) : leaf_launch<32>(D, nL, nleaf, X, ld, k, Y, st);
+}
 
 bool lr_tc_fits(const LrLevels<float2, uint32_t>& lv, int m, int r, int k) {
     if (!tc_gemm_enabled() || k < 1 || k > 32 || r < 2 || (r & 1) || lv.rp < r || lv.rp > 64 || (lv.rp & 7) ||

@@ -283,12 +283,6 @@ void tc_gemm_enable(bool on);
 bool tc_gemm_fits(int M, int N, int K);
 lsw_status cgemm_tc(const float2* A, int lda, long long sA, const float2* B, int ldb, long long sB, float2* C, int ldc,
                     long long sC, int M, int N, int K, float2 alpha, int batch, cudaStream_t st);
-// The same with A stored as BF16 (re, im) pairs, one 32-bit word per entry
-// (kind::f16 MMAs, B split into BF16 hi + lo): M % 128 == 0, K % 32 == 0.
-bool tc_bf16_fits(int M, int N, int K);
-lsw_status cgemm_tc_bf16(const uint32_t* A, int lda, long long sA, const float2* B, int ldb, long long sB, float2* C,
-                         int ldc, long long sC, int M, int N, int K, float2 alpha, int batch, cudaStream_t st);
-
 // ------------------------------------------- H-matrix level products
 // Every level of a subtree product at once: level q has blocks of nb[q] rows
 // whose factors F_j, G_j (nb x r, column-major) are consecutive; rows are cut
@@ -328,6 +322,11 @@ __host__ __device__ __forceinline__ long long fac_index(int lay, int nb, int r, 
     return base + ((long long)(o >> 7) * (rp >> 3) + (i >> 3)) * 1024 + ((o & 127) >> 3) * 64 + ((i & 7) >> 2) * 32 +
            (o & 7) * 4 + (i & 3);
 }
+// Dense leaves kept in BF16 as FAC_TILE_A tiles (rank nL; leaf_tc_tiled: the
+// sizes stored that way) times k <= 32 vectors: Y = D X, ld between vectors.
+bool leaf_tc_tiled(int nL);
+lsw_status leaf_tc_bf16(const uint32_t* D, int nL, int nleaf, const float2* X, long long ld, int k, float2* Y,
+                        cudaStream_t st);
 // tcgen05 forms for BF16 factors (lr_tc.cu): the partials P = F^H X per
 // chunk, and Y += sum over levels of G T.
 bool lr_tc_fits(const LrLevels<float2, uint32_t>& lv, int m, int r, int k);
