@@ -201,7 +201,9 @@ lsw_status lsw_point_sources(const lsw_green* g, const int32_t* positions, int n
  * Eq. 4): for each of nbatch fields computes the product named by mode
  * (lsw_op_mode).  prec: LSW_C128 or LSW_C64 for u, u0 and y.  u0 may be
  * NULL for FORWARD and RESIDUAL (read as zero) and is ignored otherwise.
- * y must not alias u or u0.  Scratch: 2 * nbatch * nz * nx complex. */
+ * y must not alias u or u0.  Scratch: 2 * nbatch * nz * nx complex; none for
+ * small fields (sides of 8 to 128, at most 8192 cells each and 32768 in all),
+ * which take one launch. */
 lsw_status lsw_apply_operator(const lsw_green* g, int prec, const double* chi,
                               const void* u, const void* u0, void* y,
                               int nbatch, int mode, void* stream);
@@ -364,7 +366,8 @@ lsw_status lsw_solve_sweep(const lsw_grid* grid, const double* velocity, const d
 
 /* Measure the operator's pass variants for this grid and precision on
  * nbatch fields -- 0: register FFT passes, 1: the same with
- * 512-thread row blocks in the x pass, 2: shared-memory Stockham passes --
+ * 512-thread row blocks in the x pass (small fields take one launch under
+ * either), 2: shared-memory Stockham passes --
  * and use the fastest for this (2nz, 2nx, precision) from now on in this
  * process.  *variant (may be NULL) receives the choice, ms3 (may be NULL)
  * the three mean times per apply in ms (-1: variant not available here).

@@ -406,12 +406,12 @@ lsw_status lsw_apply_operator(const lsw_green* g, int prec, const double* chi, c
     const long long n = (long long)g->nz * g->nx;
     OpGeom geo{g->nz, g->nx, chi, g->nz, nullptr, 1};
     DevBuf work;
+    if (!op_small(g, g->full, geo, prec == LSW_C128 ? 8 : 4, nbatch, u, y))
+        LSW_TRY(work.alloc((prec == LSW_C128 ? sizeof(double2) : sizeof(float2)) * 2 * n * nbatch, st));
     if (prec == LSW_C128) {
-        LSW_TRY(work.alloc(sizeof(double2) * 2 * n * nbatch, st));
         return op_apply<double>(g, g->full, geo, mode, (const double2*)u, (const double2*)u0, (double2*)y, nbatch,
                                 work.as<double2>(), st);
     }
-    LSW_TRY(work.alloc(sizeof(float2) * 2 * n * nbatch, st));
     return op_apply<float>(g, g->full, geo, mode, (const float2*)u, (const float2*)u0, (float2*)y, nbatch,
                            work.as<float2>(), st);
 }

@@ -18,6 +18,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "fft.cuh"
 #include "lsw_internal.cuh"
@@ -394,6 +395,45 @@ k_fb(typename Cx<R>::T* __restrict__ T_, int bz, const typename Cx<R>::T* __rest
     }
 }
 
+// The epilogue of one group's half of a column: entry a of the EH in v lies
+// at iz0 + T a of the column, which starts at col0 (chi's at ch); the fields
+// it is combined with are all loaded before the first is used.
+template <typename R, typename C, int E, int EH>
+__device__ __forceinline__ void column_out(C (&v)[E], const C* __restrict__ u, const C* __restrict__ u0,
+                                           C* __restrict__ y, const double* __restrict__ ch, long long col0, int iz0,
+                                           int T, int mode, std::integral_constant<int, EH>) {
+    const long long off = col0 + iz0;
+    if (mode == LSW_OP_RESIDUAL) {
+        C x[EH];
+#pragma unroll
+        for (int a = 0; a < EH; ++a) x[a] = __ldcs(u + off + T * a);
+#pragma unroll
+        for (int a = 0; a < EH; ++a) v[a] = csub(x[a], v[a]);
+        if (u0) {
+#pragma unroll
+            for (int a = 0; a < EH; ++a) x[a] = __ldcs(u0 + off + T * a);
+#pragma unroll
+            for (int a = 0; a < EH; ++a) v[a] = csub(v[a], x[a]);
+        }
+    } else if (mode == LSW_OP_FORWARD) {
+        if (u0) {
+            C x[EH];
+#pragma unroll
+            for (int a = 0; a < EH; ++a) x[a] = __ldcs(u0 + off + T * a);
+#pragma unroll
+            for (int a = 0; a < EH; ++a) v[a] = cadd(x[a], v[a]);
+        }
+    } else if (mode == LSW_OP_ADJOINT) {
+        R x[EH];
+#pragma unroll
+        for (int a = 0; a < EH; ++a) x[a] = (R)ch[iz0 + T * a];
+#pragma unroll
+        for (int a = 0; a < EH; ++a) v[a] = mk(v[a].x * x[a], -v[a].y * x[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < EH; ++a) __stcs(y + off + T * a, v[a]);
+}
+
 template <typename R, int LOGN>
 __global__ void __launch_bounds__(kFftThreads, (fft_ctas<R, LOGN, false>()))
 k_fc(const typename Cx<R>::T* __restrict__ T_, DevGeom geo, const typename Cx<R>::T* __restrict__ lt, int mode,
@@ -427,42 +467,200 @@ k_fc(const typename Cx<R>::T* __restrict__ T_, DevGeom geo, const typename Cx<R>
     line_fft<LOGN, true>(v, buf, t, par, lt);
     add_parities<LOGN>(v, buf, buf + (par ? -COLS * LS : COLS * LS), t, par);
     if (!valid) return;
-    // entry a of this group's half lies at off + T a; the fields it is
-    // combined with are all loaded before the first is used
     constexpr int EH = E / 2;
-    const int iz0 = par * EH * T + t;
-    const long long off = ((long long)b * geo.bx + ix) * N + iz0;
-    if (mode == LSW_OP_RESIDUAL) {
-        C x[EH];
-#pragma unroll
-        for (int a = 0; a < EH; ++a) x[a] = __ldcs(u + off + T * a);
-#pragma unroll
-        for (int a = 0; a < EH; ++a) v[a] = csub(x[a], v[a]);
-        if (u0) {
-#pragma unroll
-            for (int a = 0; a < EH; ++a) x[a] = __ldcs(u0 + off + T * a);
-#pragma unroll
-            for (int a = 0; a < EH; ++a) v[a] = csub(v[a], x[a]);
-        }
-    } else if (mode == LSW_OP_FORWARD) {
-        if (u0) {
-            C x[EH];
-#pragma unroll
-            for (int a = 0; a < EH; ++a) x[a] = __ldcs(u0 + off + T * a);
-#pragma unroll
-            for (int a = 0; a < EH; ++a) v[a] = cadd(x[a], v[a]);
-        }
-    } else if (mode == LSW_OP_ADJOINT) {
-        const int2 org = box_origin(geo, b);
-        const double* ch = geo.chi + (long long)(org.y + ix) * geo.chi_ld + org.x + iz0;
-        R x[EH];
-#pragma unroll
-        for (int a = 0; a < EH; ++a) x[a] = (R)ch[T * a];
-#pragma unroll
-        for (int a = 0; a < EH; ++a) v[a] = mk(v[a].x * x[a], -v[a].y * x[a]);
+    const int2 org = box_origin(geo, b);
+    column_out<R>(v, u, u0, y, geo.chi + (long long)(org.y + ix) * geo.chi_ld + org.x,
+                  ((long long)b * geo.bx + ix) * N, par * EH * T + t, T, mode, std::integral_constant<int, EH>());
+}
+
+// --------------------------------------------- small fields: one launch
+// Boxes of few cells finish in one launch: a cluster of CL thread blocks takes
+// a field through all three passes, the intermediate T lying in the blocks'
+// shared memory, each holding 2 bz / CL of its rows.  Pass A writes its
+// columns into the owners' rows (distributed shared memory), pass B works on
+// a block's own rows, pass C reads its columns back.  The line transforms and
+// the epilogues are those of the three-pass kernels, so the results are the same
+// bit for bit.  Bound by its chain of latencies (three line transforms, two
+// cluster barriers): one 64 x 64 c64 field takes 8.2 us on the GPU (three
+// launches: 7.6, overlapping their starts), but a call costs the host 13.9 us
+// instead of 19.5, with one launch and no work array.
+constexpr int kSmallThreads = 256;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// the address of this block's shared variable at p in block `rank`
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, float2 v) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, double2 v) {
+    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ void cluster_load(uint32_t a, float2& v) {
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cluster_load(uint32_t a, double2& v) {
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
+}
+
+// The block's share of a field: columns ix0 .. ix0 + cols, rows of T
+// rank * rows ..; row r of T at rows + r * ls in shared memory.
+template <typename C> struct SmallField {
+    int cl, logrows, cols, ix0, ls;
+    C* rows;
+    C* bufs;                                 // transpose buffers of the block's lines
+    __device__ __forceinline__ uint32_t remote(int kz, int ix) const {
+        return cluster_addr(rows + (kz & ((1 << logrows) - 1)) * ls + ix, (uint32_t)(kz >> logrows));
     }
+};
+
+template <typename R, int LOGN, typename C>
+__device__ __forceinline__ void small_a(const SmallField<C>& f, const C* __restrict__ ub, const double* __restrict__ chb,
+                                        int chi_ld, int adjoint, const C* __restrict__ lt) {
+    typedef LineCfg<LOGN> L;
+    constexpr int N = L::N, E = L::E, T = L::T, LINES = kSmallThreads / T, LS = line_stride<C, LOGN, kblk<C>()>();
+    const int t = threadIdx.x % T;
+    C* buf = f.bufs + (threadIdx.x / T) * LS;
+    for (int l0 = 0; l0 < 2 * f.cols; l0 += LINES) {
+        const int line = l0 + threadIdx.x / T;
+        const bool valid = line < 2 * f.cols;
+        const int par = valid && line >= f.cols, ix = f.ix0 + (valid ? line - par * f.cols : 0);
+        const C* uc = ub + (long long)ix * N;
+        const double* ch = chb + (long long)ix * chi_ld;
+        C v[E];
 #pragma unroll
-    for (int a = 0; a < EH; ++a) __stcs(y + off + T * a, v[a]);
+        for (int a = 0; a < E; ++a) v[a] = uc[T * a + t];
+        if (adjoint) {
+#pragma unroll
+            for (int a = 0; a < E; ++a) v[a].y = -v[a].y;
+        } else {
+            double c[E];
+#pragma unroll
+            for (int a = 0; a < E; ++a) c[a] = ch[T * a + t];
+#pragma unroll
+            for (int a = 0; a < E; ++a) v[a] = cscale(v[a], (R)c[a]);
+        }
+        line_fft<LOGN, false>(v, buf, t, par, lt);
+        if (l0 == 0) cluster_wait();         // every block of the cluster has started
+        if (valid) {
+#pragma unroll
+            for (int a = 0; a < E; ++a) cluster_store(f.remote(par * N + T * a + t, ix), v[a]);
+        }
+    }
+}
+
+// spec: the spectra of the block's rows, N + 1 entries each
+template <int LOGN, typename C>
+__device__ __forceinline__ void small_b(const SmallField<C>& f, const C* spec, const C* __restrict__ lt) {
+    typedef LineCfg<LOGN> L;
+    constexpr int N = L::N, E = L::E, T = L::T, HALF = kSmallThreads / T / 2, LS = line_stride<C, LOGN, kblk<C>()>();
+    const int t = threadIdx.x % T, line = threadIdx.x / T, par = line / HALF, nrows = 1 << f.logrows;
+    C* buf = f.bufs + line * LS;
+    for (int r0 = 0; r0 < nrows; r0 += HALF) {
+        const int row = r0 + line - par * HALF;
+        const bool valid = row < nrows;
+        C* rowp = f.rows + (valid ? row : 0) * f.ls;
+        if (r0) __syncthreads();
+        C v[E];
+#pragma unroll
+        for (int a = 0; a < E; ++a) v[a] = rowp[T * a + t];
+        line_fft<LOGN, false>(v, buf, t, par, lt);
+        const C* sp = spec + (valid ? row : 0) * (N + 1) + par * (N / 2 + 1);
+#pragma unroll
+        for (int a = 0; a < E; ++a) v[a] = cmul(v[a], sp[min(T * a + t, N - par - (T * a + t))]);
+        line_fft<LOGN, true>(v, buf, t, par, lt);
+        add_parities<LOGN>(v, buf, buf + (par ? -HALF * LS : HALF * LS), t, par);
+        constexpr int EH = E / 2;
+        if (valid) {
+#pragma unroll
+            for (int a = 0; a < EH; ++a) rowp[T * (par * EH + a) + t] = v[a];
+        }
+    }
+}
+
+template <typename R, int LOGN, typename C>
+__device__ __forceinline__ void small_c(const SmallField<C>& f, const C* __restrict__ ub, const C* __restrict__ u0b,
+                                        C* __restrict__ yb, const double* __restrict__ chb, int chi_ld, int mode,
+                                        const C* __restrict__ lt) {
+    typedef LineCfg<LOGN> L;
+    constexpr int N = L::N, E = L::E, T = L::T, HALF = kSmallThreads / T / 2, LS = line_stride<C, LOGN, kblk<C>()>();
+    const int t = threadIdx.x % T, line = threadIdx.x / T, par = line / HALF;
+    C* buf = f.bufs + line * LS;
+    for (int c0 = 0; c0 < f.cols; c0 += HALF) {
+        const int col = c0 + line - par * HALF;
+        const bool valid = col < f.cols;
+        const int ix = f.ix0 + (valid ? col : 0);
+        if (c0) __syncthreads();
+        C v[E];
+#pragma unroll
+        for (int a = 0; a < E; ++a) cluster_load(f.remote(par * N + T * a + t, ix), v[a]);
+        if (c0 + HALF >= f.cols) cluster_arrive();
+        line_fft<LOGN, true>(v, buf, t, par, lt);
+        add_parities<LOGN>(v, buf, buf + (par ? -HALF * LS : HALF * LS), t, par);
+        if (valid) {
+            constexpr int EH = E / 2;
+            column_out<R>(v, ub, u0b, yb, chb + (long long)ix * chi_ld, (long long)ix * N, par * EH * T + t, T, mode,
+                          std::integral_constant<int, EH>());
+        }
+    }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kSmallThreads, sizeof(R) == 8 ? 1 : 2)
+k_small(const typename Cx<R>::T* __restrict__ u, DevGeom geo, int logrows, const typename Cx<R>::T* __restrict__ spt,
+        const typename Cx<R>::T* __restrict__ tab, int mode, const typename Cx<R>::T* __restrict__ u0,
+        typename Cx<R>::T* __restrict__ y, int cl) {
+    typedef typename Cx<R>::T C;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    const int b = blockIdx.x / cl, rank = (int)cluster_rank(), nrows = 1 << logrows, bz = geo.bz, bx = geo.bx;
+    SmallField<C> f;
+    f.cl = cl;
+    f.logrows = logrows;
+    f.cols = bx / cl;
+    f.ix0 = rank * f.cols;
+    f.ls = bx + 1;
+    f.rows = reinterpret_cast<C*>(sm_raw);
+    cluster_arrive();
+    C* spec = f.rows + nrows * f.ls;
+    f.bufs = spec + nrows * f.ls;
+    for (int r = threadIdx.x >> 5; r < nrows; r += kSmallThreads / 32) {
+        const int kr = rank * nrows + r, kz = kr < bz ? 2 * kr : 2 * (kr - bz) + 1;
+        const C* sp = spt + (long long)min(kz, 2 * bz - kz) * (bx + 1);
+        for (int e = threadIdx.x & 31; e <= bx; e += 32) cp_async<sizeof(C)>(spec + r * (bx + 1) + e, sp + e);
+    }
+    const int2 org = box_origin(geo, b);
+    const double* chb = geo.chi + (long long)org.y * geo.chi_ld + org.x;
+    const long long off = (long long)b * bz * bx;
+    const C* ub = u + off;
+    const C* u0b = u0 ? u0 + off : nullptr;
+    const C* ltz = tab + line_table(bz);
+#define LSW_SMALL_SWITCH(n, ...)                                  \
+    switch (n) {                                                  \
+        case 8: { constexpr int L_ = 3; __VA_ARGS__; break; }     \
+        case 16: { constexpr int L_ = 4; __VA_ARGS__; break; }    \
+        case 32: { constexpr int L_ = 5; __VA_ARGS__; break; }    \
+        case 64: { constexpr int L_ = 6; __VA_ARGS__; break; }    \
+        default: { constexpr int L_ = 7; __VA_ARGS__; break; }    \
+    }
+    LSW_SMALL_SWITCH(bz, small_a<R, L_>(f, ub, chb, geo.chi_ld, mode == LSW_OP_ADJOINT, ltz))
+    cp_async_wait_all();
+    cluster_arrive();
+    cluster_wait();
+    LSW_SMALL_SWITCH(bx, small_b<L_>(f, spec, tab + line_table(bx)))
+    cluster_arrive();
+    cluster_wait();
+    LSW_SMALL_SWITCH(bz, small_c<R, L_>(f, ub, u0b, y + off, chb, geo.chi_ld, mode, ltz))
+#undef LSW_SMALL_SWITCH
+    cluster_wait();                          // no block leaves while its rows may be read
 }
 
 // line twiddles and half-sample shifts of every line length (line_table)
@@ -704,6 +902,28 @@ lsw_status launch_fc(int lz, int nbatch, cudaStream_t st, const typename Cx<R>::
     return LSW_OK;
 }
 
+// The one-launch kernel's cluster: blocks per field, as many (at most 8) as
+// give every block a full set of row lines in pass B, and its shared memory.
+template <typename R>
+size_t small_cfg(int bz, int bx, int& cl) {
+    typedef typename Cx<R>::T C;
+    auto line_t = [](int n) { return n >= 512 ? n / 32 : n >= 128 ? n / 16 : n >= 32 ? n / 8 : n / 4; };   // LineCfg::T
+    cl = 1;
+    while (cl < 8 && 4 * bz * line_t(bx) > kSmallThreads * cl && bx / cl > 1) cl *= 2;
+    size_t bufs = 0;
+    auto lines = [&](auto lg) {
+        constexpr int L = decltype(lg)::value;
+        if (bz == 1 << L || bx == 1 << L)
+            bufs = std::max(bufs, (size_t)(kSmallThreads / LineCfg<L>::T) * line_stride<C, L, kblk<C>()>());
+    };
+    lines(std::integral_constant<int, 3>());
+    lines(std::integral_constant<int, 4>());
+    lines(std::integral_constant<int, 5>());
+    lines(std::integral_constant<int, 6>());
+    lines(std::integral_constant<int, 7>());
+    return sizeof(C) * (2 * (size_t)(2 * bz / cl) * (bx + 1) + bufs);
+}
+
 // ---------------------------------------------------------- pass tuning
 // Variant of the operator passes per (2bz, 2bx, precision): 0 register FFT
 // with 256-thread row CTAs in pass B, 1 the same with 512-thread row CTAs,
@@ -728,6 +948,24 @@ void op_set_variant(int pz, int px, int rsize, int v) {
     g_tune[std::make_tuple(pz, px, rsize)] = v;
 }
 
+// One launch (k_small) for this product?  Where the GPU finishes before the
+// host has launched three kernels and fetched a work array (19.5 us a call
+// against 13.9).  GPU time of one launch against three, c64: 64 x 64 cells, 1
+// field 8.2 / 7.6 us, 8 fields 8.3 / 7.7, 16 fields 11.6 / 8.0; 64 x 128, 1
+// field 10.2 / 9.5; 128 x 128, 1 field 17.4 / 11.9.  c128: 32 x 32 46.6 / 47.2,
+// 64 x 64, 8 fields 53.5 / 54.2, 16 fields 103 / 54.5.  So fields of up to 8192
+// cells, 32768 cells in all.  u and y must not overlap: one field's blocks may
+// write y before another's read u.
+bool op_small(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, int rsize, int nbatch, const void* u,
+              const void* y) {
+    const int bz = geo.bz, bx = geo.bx;
+    if (!is_pow2(bz) || !is_pow2(bx) || bz < 8 || bx < 8 || bz > 128 || bx > 128 || bz * bx > 8192) return false;
+    const long long cells = (long long)bz * bx * nbatch;
+    if (cells > (1 << 15) || !sp.t32 || !sp.t64 || op_variant(2 * bz, 2 * bx, rsize) == 2) return false;
+    const char *pu = static_cast<const char*>(u), *py = static_cast<const char*>(y);
+    return py + 2 * rsize * cells <= pu || pu + 2 * rsize * cells <= py;
+}
+
 // ------------------------------------------------------------ op_apply
 template <typename R>
 lsw_status op_apply(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, int mode,
@@ -746,6 +984,33 @@ lsw_status op_apply(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, i
     DevGeom dg{bz, bx, ilog2(bz), geo.chi, geo.chi_ld, geo.origin, geo.vpb > 0 ? geo.vpb : 1};
     const int logpz = ilog2(pz), logpx = ilog2(px);
     const int variant = op_variant(pz, px, (int)sizeof(R));
+    // no work array: the caller has asked op_small (the variant may change meanwhile)
+    if (!work || op_small(g, sp, geo, (int)sizeof(R), nbatch, u, y)) {
+        int cl = 1;
+        const size_t smem = small_cfg<R>(bz, bx, cl);
+        static std::atomic<bool> done{false};
+        LSW_TRY(set_smem(k_small<R>, done));
+        KTimer kt(sizeof(R) == 8 ? "operator_c128" : "operator_c64", st,
+                  op_bytes(sizeof(C), bz, bx, nbatch, u0 != nullptr, mode), op_flops(bz, bx, nbatch));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(cl * nbatch);
+        cfg.blockDim = dim3(kSmallThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = cl;
+        at.val.clusterDim.y = 1;
+        at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        LSW_CUDA(cudaLaunchKernelEx(&cfg, k_small<R>, u, dg, ilog2(2 * bz / cl),
+                                    reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)sp.t64 : (const void*)sp.t32),
+                                    reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)g->lt64 : (const void*)g->lt32),
+                                    mode, u0, y, cl));
+        LSW_LAUNCH_CHECK();
+        return LSW_OK;
+    }
     if (variant != 2 && bz >= 8 && bx >= 8 && bz <= 1024 && bx <= 1024 && sp.t32 && sp.t64) {
         const C* spt = reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)sp.t64 : (const void*)sp.t32);
         const C* tab = reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)g->lt64 : (const void*)g->lt32);

@@ -203,6 +203,11 @@ lsw_status op_apply(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, i
                     const typename Cx<R>::T* u, const typename Cx<R>::T* u0, typename Cx<R>::T* y,
                     int nbatch, typename Cx<R>::T* work, cudaStream_t st);
 
+// Products of small fields that take one launch and no work array (work may
+// be null for them).  rsize: bytes of the real type.
+bool op_small(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, int rsize, int nbatch, const void* u,
+              const void* y);
+
 lsw_status build_spectrum(const lsw_green* g, int bz, int bx, Spectrum* out, cudaStream_t st);
 void free_spectrum(Spectrum* s);
 
