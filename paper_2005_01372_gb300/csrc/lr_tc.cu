@@ -45,30 +45,43 @@ __device__ __forceinline__ float qnan() { return __int_as_float(0x7fc00000); }
 
 // The hi/lo BF16 words of four complex values x for the two B'' rows of one
 // vector column: conj = 1 builds the operand of F^H x, rows (xr, xi) and
-// (xi, -xr); conj = 0 that of G t, rows (tr, -ti) and (ti, tr).
+// (xi, -xr); conj = 0 that of G t, rows (tr, -ti) and (ti, tr).  Conversions
+// run at a quarter of the ALU's rate or less, so each value is rounded twice
+// (hi and lo, two values to an instruction) and the rest is shifts, swaps and
+// sign flips of those words.
 __device__ __forceinline__ void b_words(const float2 (&x)[4], int conj, uint4& rh, uint4& rl, uint4& ih, uint4& il) {
     uint32_t a[4], b[4], c[4], d[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-        float xh, xl, yh, yl;
-        split_bf16(x[t].x, xh, xl);
-        split_bf16(x[t].y, yh, yl);
-        if (conj) {
-            a[t] = pack_bf16(xh, yh);
-            b[t] = pack_bf16(xl, yl);
-            c[t] = pack_bf16(yh, -xh);
-            d[t] = pack_bf16(yl, -xl);
-        } else {
-            a[t] = pack_bf16(xh, -yh);
-            b[t] = pack_bf16(xl, -yl);
-            c[t] = pack_bf16(yh, xh);
-            d[t] = pack_bf16(yl, xl);
-        }
+        const uint32_t h = pack_bf16(x[t].x, x[t].y);
+        const uint32_t l = pack_bf16(x[t].x - __uint_as_float(h << 16), x[t].y - __uint_as_float(h & 0xffff0000u));
+        const uint32_t hs = __funnelshift_l(h, h, 16), lsw = __funnelshift_l(l, l, 16);
+        const uint32_t NEG = 0x80000000u;          // the second entry of a word
+        a[t] = conj ? h : h ^ NEG;
+        b[t] = conj ? l : l ^ NEG;
+        c[t] = conj ? hs ^ NEG : hs;
+        d[t] = conj ? lsw ^ NEG : lsw;
     }
     rh = make_uint4(a[0], a[1], a[2], a[3]);
     rl = make_uint4(b[0], b[1], b[2], b[3]);
     ih = make_uint4(c[0], c[1], c[2], c[3]);
     il = make_uint4(d[0], d[1], d[2], d[3]);
+}
+
+// The share of a builder warp: half K-steps (4 complex) of a stage, 32 / NH of
+// them side by side in a warp, so that every lane has a column.
+template <int NH>
+__device__ __forceinline__ int half_step(int q, int lane) { return q * (32 / NH) + lane / NH; }
+template <int NH, int KB>
+__device__ __forceinline__ void store_b(unsigned char* Bhi, unsigned char* Blo, int hk, int col, const float2 (&x)[4],
+                                        int conj) {
+    uint4 rh, rl, ih, il;
+    b_words(x, conj, rh, rl, ih, il);
+    const int o = (hk >> 1) * KB, h = hk & 1;
+    *reinterpret_cast<uint4*>(Bhi + o + kstep_off(col, h)) = rh;
+    *reinterpret_cast<uint4*>(Blo + o + kstep_off(col, h)) = rl;
+    *reinterpret_cast<uint4*>(Bhi + o + kstep_off(col + NH, h)) = ih;
+    *reinterpret_cast<uint4*>(Blo + o + kstep_off(col + NH, h)) = il;
 }
 
 // ------------------------------------------------ warp-specialised forms
@@ -190,7 +203,7 @@ __device__ __forceinline__ bool ws_close(const WsBars& b, uint32_t tmem, uint32_
 // X's 64 rows of each of the k columns are copied raw (512 B each) and become
 // B'' hi/lo in K-step tiles of 2 NH rows.
 template <int NH>
-__global__ void __launch_bounds__(WS_THREADS)
+__global__ void __launch_bounds__(WS_THREADS, 2)
 k_lr_partial_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2* __restrict__ X, int swapA,
                 float2* __restrict__ P, int ns) {
     constexpr int N = 2 * NH;
@@ -295,7 +308,7 @@ k_lr_partial_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2
             }
         }
     } else {
-        // builders: warp (0..5) takes K-steps warp, warp + 6 of each stage
+        // builders: warp (0..5) takes every sixth share (half_step) of each stage
         int g = 0;
         bool go = true;
         for (int w = blockIdx.x; w < nwork && go; w += gridDim.x) {
@@ -306,27 +319,18 @@ k_lr_partial_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2
                 if (g >= 2 && !ws_wait(bars, bars.bfree + bsel, (uint32_t)(((g - 2) >> 1) & 1))) { go = false; break; }
                 unsigned char* Bhi = Bbuf + (size_t)bsel * 2 * LBP;
                 unsigned char* Blo = Bhi + LBP;
-                if (lane < NH) {
-                    const float4* xs = reinterpret_cast<const float4*>(Xbuf + (size_t)slot * XS + lane * XPAD);
-                    for (int ks = warp; ks < KSP; ks += WS_BUILDERS) {
+                const int col = lane % NH;
+                const float4* xs = reinterpret_cast<const float4*>(Xbuf + (size_t)slot * XS + (col < k ? col : 0) * XPAD);
+                for (int q = warp; q < 2 * KSP * NH / 32; q += WS_BUILDERS) {
+                    const int hk = half_step<NH>(q, lane);
+                    float2 x[4];
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            float2 x[4];
-#pragma unroll
-                            for (int t = 0; t < 2; ++t) {
-                                const float4 v = lane < k ? xs[4 * ks + 2 * h + t] : make_float4(0.f, 0.f, 0.f, 0.f);
-                                x[2 * t] = make_float2(v.x, v.y);
-                                x[2 * t + 1] = make_float2(v.z, v.w);
-                            }
-                            uint4 rh, rl, ih, il;
-                            b_words(x, 1, rh, rl, ih, il);
-                            const int ob = ks * KB;
-                            *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane, h)) = rh;
-                            *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane, h)) = rl;
-                            *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane + NH, h)) = ih;
-                            *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane + NH, h)) = il;
-                        }
+                    for (int t = 0; t < 2; ++t) {
+                        const float4 v = col < k ? xs[2 * hk + t] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        x[2 * t] = make_float2(v.x, v.y);
+                        x[2 * t + 1] = make_float2(v.z, v.w);
                     }
+                    store_b<NH, KB>(Bhi, Blo, hk, col, x, 1);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -349,7 +353,7 @@ k_lr_partial_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2
 // and becomes B'' hi/lo (rp / 8 K-step tiles of 2 NH rows).  All levels
 // accumulate in one TMEM accumulator, which the epilogue adds to Y.
 template <int NH>
-__global__ void __launch_bounds__(WS_THREADS)
+__global__ void __launch_bounds__(WS_THREADS, 2)
 k_lr_apply_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2* __restrict__ T, int swapC,
               float2* __restrict__ Y, int ns) {
     constexpr int N = 2 * NH;
@@ -442,7 +446,7 @@ k_lr_apply_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2* 
             }
         }
     } else {
-        // builders: warp (0..5) takes K-steps warp, warp + 6 of each level
+        // builders: warp (0..5) takes every sixth share (half_step) of each level
         int g = 0;
         bool go = true;
         for (int w = blockIdx.x; w < nwork && go; w += gridDim.x) {
@@ -452,27 +456,18 @@ k_lr_apply_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2* 
                 if (g >= 2 && !ws_wait(bars, bars.bfree + bsel, (uint32_t)(((g - 2) >> 1) & 1))) { go = false; break; }
                 unsigned char* Bhi = Bbuf + (size_t)bsel * 2 * BB;
                 unsigned char* Blo = Bhi + BB;
-                if (lane < NH) {
-                    const unsigned char* tcol = Tbuf + (size_t)slot * TS + lane * TP;
-                    for (int ks = warp; ks < nks; ks += WS_BUILDERS) {
+                const int col = lane % NH;
+                const unsigned char* tcol = Tbuf + (size_t)slot * TS + (col < k ? col : 0) * TP;
+                for (int q = warp; q < 2 * nks * NH / 32; q += WS_BUILDERS) {
+                    const int hk = half_step<NH>(q, lane);
+                    float2 x[4];
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            float2 x[4];
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                const int kk = 8 * ks + 4 * h + t;
-                                x[t] = (lane < k && kk < r) ? *reinterpret_cast<const float2*>(tcol + kk * 8)
-                                                            : make_float2(0.f, 0.f);
-                            }
-                            uint4 rh, rl, ih, il;
-                            b_words(x, 0, rh, rl, ih, il);
-                            const int ob = ks * KB;
-                            *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane, h)) = rh;
-                            *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane, h)) = rl;
-                            *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane + NH, h)) = ih;
-                            *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane + NH, h)) = il;
-                        }
+                    for (int t = 0; t < 4; ++t) {
+                        const int kk = 4 * hk + t;
+                        x[t] = (col < k && kk < r) ? *reinterpret_cast<const float2*>(tcol + kk * 8)
+                                                   : make_float2(0.f, 0.f);
                     }
+                    store_b<NH, KB>(Bhi, Blo, hk, col, x, 0);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -501,7 +496,7 @@ k_lr_apply_ws(LrLevels<float2, uint32_t> lv, int m, int r, int k, const float2* 
 constexpr int LDK = 32;
 constexpr int LPAD = LDK * 8 + 16;
 template <int NH>
-__global__ void __launch_bounds__(WS_THREADS)
+__global__ void __launch_bounds__(WS_THREADS, 2)
 k_leaf_ws(const uint32_t* __restrict__ D, int nL, int nleaf, const float2* __restrict__ X, long long ld, int k,
           float2* __restrict__ Y, int ns) {
     constexpr int N = 2 * NH;
@@ -586,7 +581,7 @@ k_leaf_ws(const uint32_t* __restrict__ D, int nL, int nleaf, const float2* __res
                 if (jj < k) Y[jj * ld + row] = make_float2(d[jj], d[NH + jj]);
         }
     } else {
-        // builders: half-K-steps warp, warp + 6 of each stage
+        // builders: warp (0..5) takes every sixth share (half_step) of each stage
         int g = 0;
         bool go = true;
         for (int w = blockIdx.x; w < nwork && go; w += gridDim.x) {
@@ -596,25 +591,18 @@ k_leaf_ws(const uint32_t* __restrict__ D, int nL, int nleaf, const float2* __res
                 if (g >= 2 && !ws_wait(bars, bars.bfree + bsel, (uint32_t)(((g - 2) >> 1) & 1))) { go = false; break; }
                 unsigned char* Bhi = Bbuf + (size_t)bsel * 2 * LBP;
                 unsigned char* Blo = Bhi + LBP;
-                if (lane < NH) {
-                    const float4* xs = reinterpret_cast<const float4*>(Xbuf + (size_t)slot * XS + lane * LPAD);
-                    for (int q = warp; q < 2 * KSP; q += WS_BUILDERS) {
-                        const int ks = q >> 1, h = q & 1;
-                        float2 x[4];
+                const int col = lane % NH;
+                const float4* xs = reinterpret_cast<const float4*>(Xbuf + (size_t)slot * XS + (col < k ? col : 0) * LPAD);
+                for (int q = warp; q < 2 * KSP * NH / 32; q += WS_BUILDERS) {
+                    const int hk = half_step<NH>(q, lane);
+                    float2 x[4];
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {
-                            const float4 v = lane < k ? xs[2 * q + t] : make_float4(0.f, 0.f, 0.f, 0.f);
-                            x[2 * t] = make_float2(v.x, v.y);
-                            x[2 * t + 1] = make_float2(v.z, v.w);
-                        }
-                        uint4 rh, rl, ih, il;
-                        b_words(x, 0, rh, rl, ih, il);
-                        const int ob = ks * KB;
-                        *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane, h)) = rh;
-                        *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane, h)) = rl;
-                        *reinterpret_cast<uint4*>(Bhi + ob + kstep_off(lane + NH, h)) = ih;
-                        *reinterpret_cast<uint4*>(Blo + ob + kstep_off(lane + NH, h)) = il;
+                    for (int t = 0; t < 2; ++t) {
+                        const float4 v = col < k ? xs[2 * hk + t] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        x[2 * t] = make_float2(v.x, v.y);
+                        x[2 * t + 1] = make_float2(v.z, v.w);
                     }
+                    store_b<NH, KB>(Bhi, Blo, hk, col, x, 0);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
