@@ -15,20 +15,9 @@ constexpr int WAIT_LIMIT = 1 << 22;   // mbarrier polls before giving up
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// byte offset of core-matrix row (row, kgroup) in a K-major tile of 8 kgroups
-// (8 rows x 16 bytes per core matrix; 128 B to the next kgroup, 1024 B to the
-// next 8 rows)
-__device__ __forceinline__ int kmaj(int row, int kg) { return (((row >> 3) << 3) + kg) * 128 + (row & 7) * 16; }
-
-// shared-memory matrix descriptor: start >> 4, LBO = 128 B (next core matrix
-// along K), SBO = 1024 B (next 8 rows), descriptor version 1, no swizzle
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           (1ull << 46);
-}
-
-// the same with the 8-row stride given: tiles of one 16-element K-step
-// (two core matrices 128 B apart along K, 8-row groups sbo bytes apart)
+// shared-memory matrix descriptor of a K-major tile without swizzle: start >> 4,
+// LBO = 128 B (next 8-row x 16-byte core matrix along K), SBO = sbo bytes (next 8
+// rows), descriptor version 1
 __device__ __forceinline__ uint64_t sdesc_sbo(uint32_t saddr, uint32_t sbo) {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
            (1ull << 46);
@@ -69,6 +58,16 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db
         : "memory");
 }
 
+// the same with A in tensor memory (row = lane, 8 consecutive columns per MMA)
+__device__ __forceinline__ void mma_tf32_ta(uint32_t tmem, uint32_t ta, uint64_t db, uint32_t id, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
+        :
+        : "r"(tmem), "r"(ta), "l"(db), "r"(id), "r"(acc)
+        : "memory");
+}
+
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t id, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
@@ -106,6 +105,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
         : "r"(taddr));
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+        "%14, %15};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]),
+        "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "r"(taddr)
+        : "memory");
 }
 
 __device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
