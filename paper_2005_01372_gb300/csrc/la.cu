@@ -1482,216 +1482,208 @@ k_gj_panel(C* __restrict__ Aall, int n, long long sA, int k0, int nb, int* __res
     }
 }
 
-// Register-resident panel step for n <= NT: thread i holds row i of the
-// nb (<= 16) panel columns.  Each pivot step is an argmax over the rows at
-// or below the pivot, a row exchange between two threads, and an update of
-// every row by the scaled pivot row -- four barriers per column.
+// Pivot choice: each row's |entry|^2 as an unsigned key (non-negative floats
+// order like their bits), plus one so that rows out of the running are 0.
+// redux_first: the largest key of a warp and its lowest lane.
+__device__ __forceinline__ unsigned pivot_key(float v) { return __float_as_uint(v) + 1u; }
+__device__ __forceinline__ unsigned long long pivot_key(double v) { return (unsigned long long)__double_as_longlong(v) + 1ull; }
+__device__ __forceinline__ unsigned redux_first(unsigned key, int& lane) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, key);
+    lane = __ffs(__ballot_sync(0xffffffffu, key == m)) - 1;
+    return m;
+}
+__device__ __forceinline__ unsigned long long redux_first(unsigned long long key, int& lane) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32));
+    const bool in = (unsigned)(key >> 32) == hi;
+    const unsigned lo = __reduce_max_sync(0xffffffffu, in ? (unsigned)key : 0u);
+    lane = __ffs(__ballot_sync(0xffffffffu, in && (unsigned)key == lo)) - 1;
+    return (unsigned long long)hi << 32 | lo;
+}
+
+// Panel step for n <= NT <= 1024: columns c0 .. c0 + nb (nb <= NB) of the n-row
+// array S, pivot rows r0 .. r0 + nb; thread i holds row i of them in registers.
+// Two barriers per column: the warps' pivot candidates (every warp then picks
+// the winner for itself), and the pivot row together with the row it changes
+// places with.  The pivot column is kept in entry 0: a step shifts the row by
+// one, so no entry is addressed by the loop counter.  Bound by this one
+// block's issue and the latency of a column's chain; 16 panels of 1024 x 16 (c64)
+// took 66 us with four barriers and selected entries, now 22 us.
+// map: where the panel's row i came from, map + n: the same since the first
+// panel of the strip (`first`: this is it).
 template <typename C, int NT, int NB>
 __global__ void __launch_bounds__(NT)
-k_gj_panel_reg(C* __restrict__ Aall, int n, long long sA, int k0, int nb, int* __restrict__ pivall,
-               int* __restrict__ swlall) {
-    typedef decltype(Aall->x) R;
-    __shared__ R wbest[NT / 32];
-    __shared__ int widx[NT / 32];
-    __shared__ int pivrow;
-    __shared__ int pvs[NB];
-    __shared__ C rowc[NB];
-    __shared__ C xbuf[2][NB];
-    C* A = Aall + blockIdx.x * sA;
+k_gj_panel_reg(C* __restrict__ Sall, int n, long long sS, int c0, int r0, int nb, int* __restrict__ pivall,
+               int* __restrict__ mapall, int first) {
+    typedef decltype(Sall->x) R;
+    typedef decltype(pivot_key(R(0))) K;
+    constexpr int W = NT / 32;
+    __shared__ K wkey[2][W];
+    __shared__ int wrow[2][W];
+    __shared__ __align__(16) C xrow[2][2][NB];   // by parity of the step: the pivot row, the row it replaces
+    __shared__ int xorg[2][2][2];
+    C* S = Sall + blockIdx.x * sS + (long long)c0 * n;
     int* piv = pivall + (long long)blockIdx.x * n;
-    const int i = threadIdx.x;
+    int* map = mapall + (long long)blockIdx.x * 2 * n;
+    const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
     const bool own = i < n;
     C prow[NB];
 #pragma unroll
-    for (int t = 0; t < NB; ++t) prow[t] = (own && t < nb) ? A[(long long)(k0 + t) * n + i] : czero<C>();
+    for (int t = 0; t < NB; ++t) prow[t] = (own && t < nb) ? S[(long long)t * n + i] : czero<C>();
+    int org = i, cum = own && !first ? map[n + i] : i;
+#pragma unroll 1
     for (int j = 0; j < nb; ++j) {
-        const int c = k0 + j;
-        C pj = czero<C>();
-#pragma unroll
-        for (int t = 0; t < NB; ++t) if (t == j) pj = prow[t];
-        R best = (own && i >= c) ? pj.x * pj.x + pj.y * pj.y : (R)-1;
-        int bi = (own && i >= c) ? i : n;
-        for (int o = 16; o > 0; o >>= 1) {
-            const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if ((i & 31) == 0) { wbest[i >> 5] = best; widx[i >> 5] = bi; }
-        __syncthreads();
-        if (i < 32) {
-            R b2 = i < NT / 32 ? wbest[i] : (R)-1;
-            int i2 = i < NT / 32 ? widx[i] : n;
-            for (int o = 16; o > 0; o >>= 1) {
-                const R ob = __shfl_xor_sync(0xffffffffu, b2, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, i2, o);
-                if (ob > b2 || (ob == b2 && oi < i2)) { b2 = ob; i2 = oi; }
-            }
-            if (i == 0) {
-                pivrow = i2 < n ? i2 : c;
-                piv[c] = pivrow;
-                pvs[j] = pivrow;
-            }
+        const int c = r0 + j, h = j & 1;
+        int wl;
+        const K wk = redux_first(own && i >= c ? pivot_key(prow[0].x * prow[0].x + prow[0].y * prow[0].y) : K(0), wl);
+        if (lane == 0) {
+            wkey[h][warp] = wk;
+            wrow[h][warp] = (i & ~31) + wl;
         }
         __syncthreads();
-        const int p = pivrow;
-        if (p != c) {
-            if (i == c) {
+        redux_first(lane < W ? wkey[h][lane] : K(0), wl);
+        const int p = wrow[h][wl];                 // row c is in the running: p is one of the rows c .. n - 1
+        if (i == p) {
 #pragma unroll
-                for (int t = 0; t < NB; ++t) xbuf[0][t] = prow[t];
-            }
-            if (i == p) {
-#pragma unroll
-                for (int t = 0; t < NB; ++t) xbuf[1][t] = prow[t];
-            }
-            __syncthreads();
-            if (i == c) {
-#pragma unroll
-                for (int t = 0; t < NB; ++t) prow[t] = xbuf[1][t];
-            }
-            if (i == p) {
-#pragma unroll
-                for (int t = 0; t < NB; ++t) prow[t] = xbuf[0][t];
-            }
+            for (int t = 0; t < NB; ++t) xrow[h][0][t] = prow[t];
+            xorg[h][0][0] = org;
+            xorg[h][0][1] = cum;
+            piv[c] = p;
         }
         if (i == c) {
-            C d = czero<C>();
 #pragma unroll
-            for (int t = 0; t < NB; ++t) if (t == j) d = prow[t];
-            const R den = d.x * d.x + d.y * d.y;
-            const C inv = den > 0 ? mk(d.x / den, -d.y / den) : czero<C>();
-#pragma unroll
-            for (int t = 0; t < NB; ++t) {
-                prow[t] = t == j ? inv : cmul(prow[t], inv);
-                rowc[t] = prow[t];
-            }
+            for (int t = 0; t < NB; ++t) xrow[h][1][t] = prow[t];
+            xorg[h][1][0] = org;
+            xorg[h][1][1] = cum;
         }
         __syncthreads();
-        if (own && i != c) {
-            const C inv = rowc[j];
-            C f = czero<C>();
+        const C d = xrow[h][0][0];
+        const R den = d.x * d.x + d.y * d.y;
+        const C inv = den > 0 ? mk(d.x / den, -d.y / den) : czero<C>();
+        if (i == c) {
+            org = xorg[h][0][0];
+            cum = xorg[h][0][1];
 #pragma unroll
-            for (int t = 0; t < NB; ++t) if (t == j) f = prow[t];
+            for (int t = 1; t < NB; ++t) prow[t - 1] = cmul(xrow[h][0][t], inv);
+            prow[NB - 1] = inv;
+        } else {
+            if (i == p) {
+                org = xorg[h][1][0];
+                cum = xorg[h][1][1];
 #pragma unroll
-            for (int t = 0; t < NB; ++t) {
-                if (t == j) prow[t] = mk(-(f.x * inv.x - f.y * inv.y), -(f.x * inv.y + f.y * inv.x));
-                else if (t < nb) prow[t] = csub(prow[t], cmul(f, rowc[t]));
+                for (int t = 0; t < NB; ++t) prow[t] = xrow[h][1][t];
             }
+            const C f = cmul(prow[0], inv);
+            const C m = mk(-f.x, -f.y);
+#pragma unroll
+            for (int t = 1; t < NB; ++t) {
+                C v = prow[t];
+                cfma(v, m, xrow[h][0][t]);
+                prow[t - 1] = v;
+            }
+            prow[NB - 1] = m;
         }
     }
-    if (own) {
+    if (!own) return;
+    // nb steps have turned the rows by nb entries
 #pragma unroll
-        for (int t = 0; t < NB; ++t)
-            if (t < nb) A[(long long)(k0 + t) * n + i] = prow[t];
-    }
-    // the panel's interchanges composed into one permutation sigma of the
-    // positions they touch (count, then position/value pairs), for the update
-    if (i == 0) {
-        int* swl = swlall + (long long)blockIdx.x * (4 * NB + 1);
-        int cnt = 0;
-        for (int j = 0; j < nb; ++j) {
-            const int c = k0 + j, p = pvs[j];
-            if (p == c) continue;
-            int ic = -1, ip = -1;
-            for (int q = 0; q < cnt; ++q) {
-                if (swl[1 + 2 * q] == c) ic = q;
-                if (swl[1 + 2 * q] == p) ip = q;
-            }
-            if (ic < 0) { swl[1 + 2 * cnt] = c; swl[2 + 2 * cnt] = c; ic = cnt++; }
-            if (ip < 0) { swl[1 + 2 * cnt] = p; swl[2 + 2 * cnt] = p; ip = cnt++; }
-            const int t = swl[2 + 2 * ic]; swl[2 + 2 * ic] = swl[2 + 2 * ip]; swl[2 + 2 * ip] = t;
-        }
-        swl[0] = cnt;
-    }
+    for (int t = 0; t < NB; ++t)
+        if (t >= NB - nb) S[(long long)(t - (NB - nb)) * n + i] = prow[t];
+    map[i] = org;
+    map[n + i] = cum;
 }
 
-// Out-of-place block step for every column outside the panel, with the
-// panel's row swaps folded into the reads:  row i of the result is
-//   (i outside P) X[sigma(i)] + sum_t Pan[i][t] X[sigma(k0 + t)],
-// sigma the composition of the swaps; panel columns are copied.
-template <typename C>
-__global__ void __launch_bounds__(256)
-k_gj_update_oop(const C* __restrict__ Ain, C* __restrict__ Aout, int n, long long sA, int k0, int nb,
-                const int* __restrict__ swlall, int swstride) {
-    __shared__ C Ps[64][17];
-    __shared__ C Xs[16][65];
+// Block step of the n x ncol array A for every column outside the nb <= 64
+// panel columns c0 .. c0 + nb (pivot rows P = r0 .. r0 + nb), out of place, with
+// the panel's row swaps folded into the reads:  row i of the result is
+//   (i outside P) A[map(i)] + sum_t Pan[i][t] A[map(r0 + t)];
+// the panel's columns are copied from Pan.  64 x 64 outputs per CTA, KC panel
+// columns at a time.  Bound by the FP32 (c128: FP64) pipe: with 64 panel columns
+// an entry is read and written once for 64 multiply-adds, where steps of 16
+// moved 16 leaves of 1024 x 1024 through memory four times for them: 111 us a
+// step of 16, now about 215 us a strip of 64 and 13 us a panel inside it.  The
+// inverses of 64 such leaves took 45 ms, panels included, now 23 ms.
+template <typename C, int KC>
+__global__ void __launch_bounds__(256, sizeof(C) == 8 ? 2 : 1)
+k_gj_update_oop(const C* __restrict__ Ain, long long sIn, C* __restrict__ Aout, long long sOut, int n, int ncol, int c0,
+                int r0, int nb, const C* __restrict__ Pall, long long sP, const int* __restrict__ mapall) {
+    __shared__ C Ps[64][KC + 1];
+    __shared__ C Xs[KC][65];
     __shared__ int rmap[64];
-    __shared__ int pmap[16];
-    __shared__ int sw_pos[32], sw_val[32];
-    __shared__ int nsw;
-    const int b = blockIdx.z;
-    const C* A = Ain + b * sA;
-    C* O = Aout + b * sA;
+    __shared__ int pmap[64];
+    constexpr int PER = 64 * KC / 256;
+    const int b = blockIdx.z, tid = threadIdx.x;
+    const C* A = Ain + b * sIn;
+    C* O = Aout + b * sOut;
+    const C* Pan = Pall + b * sP;
+    const int* map = mapall + (long long)b * 2 * n;
     const int i0 = blockIdx.x * 64, j0 = blockIdx.y * 64;
-    {
-        // sigma on the positions the panel's swaps touch, composed by the panel kernel
-        const int* swl = swlall + (long long)b * swstride;
-        const int cnt = swl[0];
-        if (threadIdx.x == 0) nsw = cnt;
-        if (threadIdx.x < cnt) {
-            sw_pos[threadIdx.x] = swl[1 + 2 * threadIdx.x];
-            sw_val[threadIdx.x] = swl[2 + 2 * threadIdx.x];
-        }
-    }
+    if (tid < 64) rmap[tid] = i0 + tid < n ? map[i0 + tid] : 0;
+    else if (tid < 128) pmap[tid - 64] = tid - 64 < nb ? map[r0 + tid - 64] : 0;
     __syncthreads();
-    auto sigma = [&](int pos) {
-        for (int q = 0; q < nsw; ++q) if (sw_pos[q] == pos) return sw_val[q];
-        return pos;
+    const int ty = tid & 15, tx = tid >> 4;        // consecutive lanes: consecutive rows
+    C pr[PER], xr[PER];
+    auto fetch = [&](int t0) {
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int e = tid + 256 * u;
+            const int ii = e & 63, tp = t0 + (e >> 6), tt = t0 + e % KC, jj = e / KC;
+            pr[u] = (i0 + ii < n && tp < nb) ? Pan[(long long)tp * n + i0 + ii] : czero<C>();
+            xr[u] = (j0 + jj < ncol && tt < nb) ? A[(long long)(j0 + jj) * n + pmap[tt]] : czero<C>();
+        }
     };
-    if (threadIdx.x < 64) rmap[threadIdx.x] = i0 + threadIdx.x < n ? sigma(i0 + threadIdx.x) : 0;
-    if (threadIdx.x < 16) pmap[threadIdx.x] = threadIdx.x < nb ? sigma(k0 + threadIdx.x) : 0;
-    __syncthreads();
-    const int ty = threadIdx.x & 15, tx = threadIdx.x >> 4;   // consecutive lanes: consecutive rows
-    // the old entries this thread's outputs add to, requested before the
-    // panel product so that their latency overlaps it
-    C aold[4][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int li = ty + 16 * p;
-            const int gi = i0 + li, gj = j0 + tx + 16 * q;
-            C v = czero<C>();
-            if (gi < n && gj < n) {
-                if (gj >= k0 && gj < k0 + nb) v = A[(long long)gj * n + gi];
-                else if (!(gi >= k0 && gi < k0 + nb)) v = A[(long long)gj * n + rmap[li]];
-            }
-            aold[p][q] = v;
-        }
-    C acc[4][4];
+    C acc[4][4], old[4][4];
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[p][q] = czero<C>();
-    for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-        const int ii = e % 64, t = e / 64;
-        const int gi = i0 + ii;
-        Ps[ii][t] = (gi < n && t < nb) ? A[(long long)(k0 + t) * n + gi] : czero<C>();
-        const int jj = e % 64;
-        const int gj = j0 + jj;
-        Xs[t][jj] = (gj < n && t < nb) ? A[(long long)gj * n + pmap[t]] : czero<C>();
-    }
-    __syncthreads();
+    fetch(0);
+    for (int t0 = 0; t0 < nb; t0 += KC) {
 #pragma unroll
-    for (int t = 0; t < 16; ++t) {
-        C a[4], bb[4];
+        for (int u = 0; u < PER; ++u) {
+            const int e = tid + 256 * u;
+            Ps[e & 63][e >> 6] = pr[u];
+            Xs[e % KC][e / KC] = xr[u];
+        }
+        __syncthreads();
+        if (t0 + KC < nb) {
+            fetch(t0 + KC);
+        } else {
+            // the old entries, or the panel's columns
 #pragma unroll
-        for (int q = 0; q < 4; ++q) { a[q] = Ps[ty + 16 * q][t]; bb[q] = Xs[t][tx + 16 * q]; }
+            for (int p = 0; p < 4; ++p)
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
+                for (int q = 0; q < 4; ++q) {
+                    const int li = ty + 16 * p, gi = i0 + li, gj = j0 + tx + 16 * q;
+                    C v = czero<C>();
+                    if (gi < n && gj < ncol) {
+                        if (gj >= c0 && gj < c0 + nb) v = Pan[(long long)(gj - c0) * n + gi];
+                        else if (!(gi >= r0 && gi < r0 + nb)) v = A[(long long)gj * n + rmap[li]];
+                    }
+                    old[p][q] = v;
+                }
+        }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) cfma(acc[p][q], a[p], bb[q]);
+        for (int t = 0; t < KC; ++t) {
+            C a[4], x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                a[q] = Ps[ty + 16 * q][t];
+                x[q] = Xs[t][tx + 16 * q];
+            }
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cfma(acc[p][q], a[p], x[q]);
+        }
+        __syncthreads();
     }
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int li = ty + 16 * p;
-            const int gi = i0 + li, gj = j0 + tx + 16 * q;
-            if (gi >= n || gj >= n) continue;
-            C* o = O + (long long)gj * n + gi;
-            if (gj >= k0 && gj < k0 + nb) *o = aold[p][q];
-            else if (gi >= k0 && gi < k0 + nb) *o = acc[p][q];
-            else *o = cadd(aold[p][q], acc[p][q]);
+            const int gi = i0 + ty + 16 * p, gj = j0 + tx + 16 * q;
+            if (gi >= n || gj >= ncol) continue;
+            O[(long long)gj * n + gi] = gj >= c0 && gj < c0 + nb ? old[p][q] : cadd(old[p][q], acc[p][q]);
         }
 }
 
@@ -2308,28 +2300,48 @@ lsw_status inverse_gj(typename Cx<R>::T* A, int n, long long sA, int batch, cuda
         }
     }
     if (n <= NT) {
-        // register panels + out-of-place updates, ping-pong between A and B
-        constexpr int NB = sizeof(R) == 8 ? 8 : 16;
-        const int nb = NB;
-        DevBuf piv, B, swl;
+        // Strips of up to 64 columns, out of place between A and B.  Within a
+        // strip, panels of NB columns update the strip alone (between the
+        // buffers S); its 64 columns then update the whole matrix at once.
+        // In-place Gauss-Jordan leaves in a strip's columns exactly what its
+        // row operations multiply the strip's (exchanged) rows by, whatever
+        // the panels inside.
+        constexpr int NB = sizeof(R) == 8 ? 8 : 16, WS = 64;
+        DevBuf piv, B, map, S;
         LSW_TRY(piv.alloc(sizeof(int) * (size_t)n * batch, st));
         LSW_TRY(B.alloc(sizeof(CT) * (size_t)sA * batch, st));
-        const int swstride = 4 * NB + 1;
-        LSW_TRY(swl.alloc(sizeof(int) * (size_t)swstride * batch, st));
+        LSW_TRY(map.alloc(sizeof(int) * 2 * (size_t)n * batch, st));
+        const long long sS = (long long)n * WS;
+        LSW_TRY(S.alloc(sizeof(CT) * 2 * (size_t)sS * batch, st));
         CT* cur = A;
         CT* nxt = B.as<CT>();
-        for (int k0 = 0; k0 < n; k0 += nb) {
-            const int w = std::min(nb, n - k0);
-            k_gj_panel_reg<CT, NT, NB><<<batch, NT, 0, st>>>(cur, n, sA, k0, w, piv.as<int>(), swl.as<int>());
-            LSW_LAUNCH_CHECK();
-            if (w == n) continue;
-            {
-                // reads and writes every matrix once; 8 n^2 w real flops each
-                KTimer kt("gj_update", st, 2.0 * sizeof(CT) * (double)n * n * batch, 8.0 * (double)n * n * w * batch);
-                k_gj_update_oop<CT><<<dim3((n + 63) / 64, (n + 63) / 64, batch), 256, 0, st>>>(cur, nxt, n, sA, k0, w,
-                                                                                              swl.as<int>(), swstride);
+        const dim3 blk(256);
+        for (int k0 = 0; k0 < n; k0 += WS) {
+            const int ws = std::min(WS, n - k0);
+            CT* strip = cur + (long long)k0 * n;
+            long long ss = sA;
+            for (int c = 0; c < ws; c += NB) {
+                const int w = std::min(NB, ws - c), first = c == 0;
+                if (n <= 256)
+                    k_gj_panel_reg<CT, 256, NB><<<batch, 256, 0, st>>>(strip, n, ss, c, k0 + c, w, piv.as<int>(), map.as<int>(), first);
+                else if (n <= 512)
+                    k_gj_panel_reg<CT, 512, NB><<<batch, 512, 0, st>>>(strip, n, ss, c, k0 + c, w, piv.as<int>(), map.as<int>(), first);
+                else
+                    k_gj_panel_reg<CT, NT, NB><<<batch, NT, 0, st>>>(strip, n, ss, c, k0 + c, w, piv.as<int>(), map.as<int>(), first);
                 LSW_LAUNCH_CHECK();
+                if (w == ws) break;
+                CT* to = S.as<CT>() + ((c / NB) & 1) * sS * batch;
+                k_gj_update_oop<CT, NB><<<dim3((n + 63) / 64, 1, batch), blk, 0, st>>>(
+                    strip, ss, to, sS, n, ws, c, k0 + c, w, strip + (long long)c * n, ss, map.as<int>());
+                LSW_LAUNCH_CHECK();
+                strip = to;
+                ss = sS;
             }
+            // reads and writes every matrix once; 8 n^2 ws real flops each
+            KTimer kt("gj_update", st, 2.0 * sizeof(CT) * (double)n * n * batch, 8.0 * (double)n * n * ws * batch);
+            k_gj_update_oop<CT, 16><<<dim3((n + 63) / 64, (n + 63) / 64, batch), blk, 0, st>>>(
+                cur, sA, nxt, sA, n, n, k0, k0, ws, strip, ss, map.as<int>() + n);
+            LSW_LAUNCH_CHECK();
             std::swap(cur, nxt);
         }
         if (cur != A) {
