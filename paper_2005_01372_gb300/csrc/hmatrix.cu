@@ -265,17 +265,31 @@ __global__ void k_gather_map(const C* __restrict__ src, int m, int k, const int*
     }
 }
 
-// x_tree[s][i] = x_grid[s][perm[i]]   (dir = 0)   or the inverse (dir = 1)
+// x_tree[s][i] = x_grid[s][perm[i]]   (dir = 0)   or the inverse (dir = 1).
+// Thread per cell and PERM_V vectors, all read before the first is written:
+// bound by memory (perm runs over a box's columns, so accesses are runs of the
+// box's height).  A thread per entry, with its 64-bit divisions, took 17.3 us
+// for 16 vectors of 512 x 512, now 10.3 us.
+constexpr int PERM_V = 8;
 template <typename C>
-__global__ void k_permute(const C* __restrict__ src, C* __restrict__ dst, const int* __restrict__ perm, int n, int nb,
-                          int dir) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)n * nb; e += (long long)gridDim.x * blockDim.x) {
-        const int s = (int)(e / n), i = (int)(e - (long long)s * n);
-        const long long g = (long long)s * n + perm[i];
-        if (dir == 0) dst[e] = src[g];
-        else dst[g] = src[e];
+__global__ void __launch_bounds__(256)
+k_permute(const C* __restrict__ src, C* __restrict__ dst, const int* __restrict__ perm, int n, int nb, int dir) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const int g = perm[i];
+    for (int s0 = blockIdx.y * PERM_V; s0 < nb; s0 += gridDim.y * PERM_V) {
+        const C* from = src + (long long)s0 * n + (dir ? i : g);
+        C* to = dst + (long long)s0 * n + (dir ? g : i);
+        C v[PERM_V];
+#pragma unroll
+        for (int u = 0; u < PERM_V; ++u)
+            if (s0 + u < nb) v[u] = from[(long long)u * n];
+#pragma unroll
+        for (int u = 0; u < PERM_V; ++u)
+            if (s0 + u < nb) to[(long long)u * n] = v[u];
     }
 }
+dim3 perm_grid(int n, int nb) { return dim3((n + 255) / 256, std::min((nb + PERM_V - 1) / PERM_V, 65535)); }
 
 // Dense leaf of I - Gt diag(chi): entry (i, j) of leaf c, tree order.
 template <typename C>
@@ -1474,10 +1488,10 @@ lsw_status apply_h(const lsw_hmatrix* h, const typename Cx<R>::T* x, typename Cx
         DevBuf xt, yt;
         LSW_TRY(xt.alloc(sizeof(C) * (size_t)n * nb, st));
         LSW_TRY(yt.alloc(sizeof(C) * (size_t)n * nb, st));
-        k_permute<C><<<gridn((long long)n * nb), 256, 0, st>>>(x, xt.as<C>(), h->perm_d, n, nb, 0);
+        k_permute<C><<<perm_grid(n, nb), 256, 0, st>>>(x, xt.as<C>(), h->perm_d, n, nb, 0);
         LSW_LAUNCH_CHECK();
         LSW_TRY(hmv_bf16(h->hb, reinterpret_cast<const float2*>(xt.p), nb, reinterpret_cast<float2*>(yt.p), st));
-        k_permute<C><<<gridn((long long)n * nb), 256, 0, st>>>(yt.as<C>(), y, h->perm_d, n, nb, 1);
+        k_permute<C><<<perm_grid(n, nb), 256, 0, st>>>(yt.as<C>(), y, h->perm_d, n, nb, 1);
         LSW_LAUNCH_CHECK();
         return LSW_OK;
     }
@@ -1486,10 +1500,10 @@ lsw_status apply_h(const lsw_hmatrix* h, const typename Cx<R>::T* x, typename Cx
     LSW_TRY(xt.alloc(sizeof(C) * (size_t)n * nb, st));
     LSW_TRY(yt.alloc(sizeof(C) * (size_t)n * nb, st));
     LSW_TRY(T.alloc(sizeof(C) * ((size_t)1 << h->L) * r * nb, st));
-    k_permute<C><<<gridn((long long)n * nb), 256, 0, st>>>(x, xt.as<C>(), h->perm_d, n, nb, 0);
+    k_permute<C><<<perm_grid(n, nb), 256, 0, st>>>(x, xt.as<C>(), h->perm_d, n, nb, 0);
     LSW_LAUNCH_CHECK();
     LSW_TRY(hmv<R>(H, 0, 0, xt.as<C>(), nb, yt.as<C>(), T.as<C>(), st));
-    k_permute<C><<<gridn((long long)n * nb), 256, 0, st>>>(yt.as<C>(), y, h->perm_d, n, nb, 1);
+    k_permute<C><<<perm_grid(n, nb), 256, 0, st>>>(yt.as<C>(), y, h->perm_d, n, nb, 1);
     LSW_LAUNCH_CHECK();
     return LSW_OK;
 }
