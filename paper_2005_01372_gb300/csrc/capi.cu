@@ -126,7 +126,7 @@ void timer_release(std::vector<TimedSpan>& spans) {
 }
 
 namespace {
-constexpr int kPool = 8, kSlots = 8;
+constexpr int kPool = Fork::kStreams, kSlots = 8;
 std::mutex g_pool_mu;
 cudaStream_t g_pool[64][kSlots][kPool] = {};
 thread_local int g_slot = 0;     // which pool this host thread forks onto
@@ -135,16 +135,6 @@ thread_local int g_slot = 0;     // which pool this host thread forks onto
 void set_worker_slot(int slot) { g_slot = slot >= 0 && slot < kSlots ? slot : 0; }
 
 Fork::Fork(cudaStream_t parent) : parent_(parent) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    {
-        std::lock_guard<std::mutex> lk(g_pool_mu);
-        for (int i = 0; i < kPool; ++i) {
-            cudaStream_t* slot = (dev >= 0 && dev < 64) ? &g_pool[dev][g_slot][i] : nullptr;
-            if (slot && !*slot) cudaStreamCreateWithFlags(slot, cudaStreamNonBlocking);
-            streams_[i] = slot ? *slot : parent;
-        }
-    }
     cudaEventCreateWithFlags(&start_, cudaEventDisableTiming);
     cudaEventRecord(start_, parent_);
 }
@@ -157,6 +147,12 @@ Fork::~Fork() {
 cudaStream_t Fork::child(int i) {
     const int k = i % kPool;
     if (!(used_ & (1u << k))) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        cudaStream_t* slot = (dev >= 0 && dev < 64) ? &g_pool[dev][g_slot][k] : nullptr;
+        if (slot && !*slot) cudaStreamCreateWithFlags(slot, cudaStreamNonBlocking);
+        streams_[k] = slot ? *slot : parent_;
         cudaStreamWaitEvent(streams_[k], start_, 0);
         used_ |= 1u << k;
     }

@@ -1009,6 +1009,10 @@ lsw_status add_lowrank(HStore<R>& M, int l, int c, const typename Cx<R>::T* X, c
     const int m = M.nl(l), L = M.L, r = M.r, nL = M.nl(L);
     const int rp = r + oversample;
     const int nleaf = 1 << (L - l);
+    // The leaves' update runs on st beside the levels' recompressions: they
+    // touch different arrays of M, and either is a chain of small launches
+    // (with the subtree products side by side: 128 x 256 build 37 -> 34 ms)
+    Fork fk(st0);
     if (lu) {
         // the leaves hold inverses: each leaf j of the node gets
         // D_j^-1 <- (D_j + U_j V_j^H)^-1 with U_j, V_j its rows of X, Y, by
@@ -1041,7 +1045,6 @@ lsw_status add_lowrank(HStore<R>& M, int l, int c, const typename Cx<R>::T* X, c
         LSW_TRY(gemm<R>('N', 'C', nL, nL, r, one<C>(), X, m, nL, Y, m, nL, one<C>(), D0, nL, (long long)nL * nL, nleaf,
                         st));
     }
-    Fork fk(st0);
     for (int lp = l + 1; lp <= L; ++lp) {
         // the levels' recompressions are independent of each other
         cudaStream_t st = fk.child(lp);
@@ -1083,6 +1086,8 @@ lsw_status add_lowrank(HStore<R>& M, int l, int c, const typename Cx<R>::T* X, c
     return fk.join();
 }
 
+constexpr int kSubtreeChild = Fork::kStreams - 1;     // apart from the leaf inverses' (0) and the levels'
+
 // Inverse of node (l, c) of X written into the same node of Hi (recursive
 // block inversion).  X's node c+1 subtree is overwritten by the Schur
 // complement S = D - C A^-1 B.
@@ -1112,7 +1117,7 @@ lsw_status invert_node(HStore<R>& X, int l, int c, HStore<R>& Hi, int oversample
     // the first use of level l + 1's blocks (deeper levels were waited for
     // inside the subtree just inverted, which holds a node of every level)
     LSW_TRY(lu.wait_level(l + 1, st));
-    DevBuf P, Rm, T1, T2, K, XK, T;
+    DevBuf P, Rm, T1, T2, K, XK, T, Ta;
     const size_t vb = sizeof(C) * (size_t)m1 * r;
     LSW_TRY(P.alloc(vb, st));
     LSW_TRY(Rm.alloc(vb, st));
@@ -1121,21 +1126,22 @@ lsw_status invert_node(HStore<R>& X, int l, int c, HStore<R>& Hi, int oversample
     LSW_TRY(XK.alloc(vb, st));
     LSW_TRY(K.alloc(sizeof(C) * r * r, st));
     LSW_TRY(T.alloc(sizeof(C) * ((size_t)1 << (L - l)) * r * r, st));
-    {
+    LSW_TRY(Ta.alloc(sizeof(C) * ((size_t)1 << (L - l)) * r * r, st));
+    // a subtree's product and adjoint product are independent: side by side
+    auto subtree_products = [&](int node, const C* x, C* y, const C* xa, C* ya) -> lsw_status {
         KTimer kt_sub("hodlr_subtree_products", st, 0, 0);
-        LSW_TRY(hmv<R>(Hi, l + 1, a, UB, r, P.as<C>(), T.as<C>(), st));        // P = A^-1 UB
-        LSW_TRY(hmv_adj<R>(Hi, l + 1, a, WC, r, Rm.as<C>(), T.as<C>(), st));   // R = A^-H WC
-    }
+        Fork fk(st);
+        LSW_TRY(hmv_adj<R>(Hi, l + 1, node, xa, r, ya, Ta.as<C>(), fk.child(kSubtreeChild)));
+        LSW_TRY(hmv<R>(Hi, l + 1, node, x, r, y, T.as<C>(), st));
+        return fk.join();
+    };
+    LSW_TRY(subtree_products(a, UB, P.as<C>(), WC, Rm.as<C>()));               // P = A^-1 UB, R = A^-H WC
     LSW_TRY(gemm<R>('C', 'N', r, r, m1, one<C>(), WC, m1, 0, P.as<C>(), m1, 0, zero<C>(), K.as<C>(), r, 0, 1, st));
     // S = D - UC K WB^H  (in place on X's node b)
     LSW_TRY(gemm<R>('N', 'N', m1, r, r, minus_one<C>(), UC, m1, 0, K.as<C>(), r, 0, zero<C>(), XK.as<C>(), m1, 0, 1, st));
     LSW_TRY(add_lowrank<R>(X, l + 1, b, XK.as<C>(), WB, 0, l, c, oversample, seed, st, &lu));
     LSW_TRY(invert_node<R>(X, l + 1, b, Hi, oversample, seed, st, lu));     // S^-1 into Hi
-    {
-        KTimer kt_sub("hodlr_subtree_products", st, 0, 0);
-        LSW_TRY(hmv<R>(Hi, l + 1, b, UC, r, T1.as<C>(), T.as<C>(), st));       // T1 = S^-1 UC
-        LSW_TRY(hmv_adj<R>(Hi, l + 1, b, WB, r, T2.as<C>(), T.as<C>(), st));   // T2 = S^-H WB
-    }
+    LSW_TRY(subtree_products(b, UC, T1.as<C>(), WB, T2.as<C>()));              // T1 = S^-1 UC, T2 = S^-H WB
     LSW_TRY(gemm<R>('C', 'N', r, r, m1, one<C>(), WB, m1, 0, T1.as<C>(), m1, 0, zero<C>(), K.as<C>(), r, 0, 1, st));
     // top-left: A^-1 + P K2 R^H
     LSW_TRY(gemm<R>('N', 'N', m1, r, r, one<C>(), P.as<C>(), m1, 0, K.as<C>(), r, 0, zero<C>(), XK.as<C>(), m1, 0, 1, st));

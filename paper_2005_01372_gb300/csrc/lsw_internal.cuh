@@ -145,6 +145,9 @@ void set_worker_slot(int slot);
 
 class Fork {
   public:
+    // streams of a pool: more than the levels of a tree, so that a level's
+    // child never queues behind another's (or behind child 0, the leaf inverses)
+    static constexpr int kStreams = 16;
     explicit Fork(cudaStream_t parent);
     ~Fork();
     cudaStream_t child(int i);
@@ -154,7 +157,7 @@ class Fork {
     cudaStream_t parent_;
     cudaEvent_t start_ = nullptr;
     unsigned used_ = 0;
-    cudaStream_t streams_[8] = {};
+    cudaStream_t streams_[kStreams] = {};
 };
 
 // ------------------------------------------------------------ FFT geometry
