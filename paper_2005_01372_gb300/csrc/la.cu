@@ -2005,12 +2005,18 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
         LSW_LAUNCH_CHECK();
         return LSW_OK;
     }
-    const bool narrow = n <= 32;
-    const int BMv = narrow ? 128 : 64, BNv = narrow ? 32 : 64;
+    // tiles of 64 x 64 outputs, or 32 on a side that has no more: 20 rows of the
+    // leaf updates' V^H D^-1 filled a third of a 64-row tile (25 us on average
+    // in a 256^2 build, 17 with 32 rows)
+    const bool narrow = n <= 32, low = !narrow && m <= 32;
+    const int BMv = narrow ? 128 : low ? 32 : 64, BNv = narrow ? 32 : low ? 128 : 64;
     const int gx = (m + BMv - 1) / BMv, gy = (n + BNv - 1) / BNv;
     auto launch = [&](int ks, int kc, CT* P) {
         if (narrow)
             k_gemm<CT, 128, 32><<<dim3(gx, gy, batch * ks), 256, 0, st>>>(oa, ob, m, n, k, alpha, A, lda, sA, B, ldb, sB,
+                                                                           beta, C, ldc, sC, ks, kc, P);
+        else if (low)
+            k_gemm<CT, 32, 128><<<dim3(gx, gy, batch * ks), 256, 0, st>>>(oa, ob, m, n, k, alpha, A, lda, sA, B, ldb, sB,
                                                                            beta, C, ldc, sC, ks, kc, P);
         else
             k_gemm<CT, 64, 64><<<dim3(gx, gy, batch * ks), 256, 0, st>>>(oa, ob, m, n, k, alpha, A, lda, sA, B, ldb, sB,
