@@ -357,8 +357,6 @@ lsw_status lsw_destroy_green(lsw_green* g) {
     if (g->table) cudaFree(g->table);
     if (g->tw64) cudaFree(g->tw64);
     if (g->tw32) cudaFree(g->tw32);
-    if (g->lt64) cudaFree(g->lt64);
-    if (g->lt32) cudaFree(g->lt32);
     free_spectrum(&g->full);
     delete g;
     return LSW_OK;

@@ -1089,11 +1089,13 @@ lsw_status build_spectrum(const lsw_green* g, int bz, int bx, Spectrum* out, cud
     s.bz = bz;
     s.bx = bx;
     const size_t nq = (size_t)(bz + 1) * (bx + 1);
-    if (cudaMalloc(&s.q64, nq * sizeof(double2)) != cudaSuccess || cudaMalloc(&s.q32, nq * sizeof(float2)) != cudaSuccess ||
-        cudaMalloc(&s.t64, nq * sizeof(double2)) != cudaSuccess || cudaMalloc(&s.t32, nq * sizeof(float2)) != cudaSuccess) {
+    if (cudaMalloc(&s.q64, 2 * nq * sizeof(double2)) != cudaSuccess ||
+        cudaMalloc(&s.q32, 2 * nq * sizeof(float2)) != cudaSuccess) {
         free_spectrum(&s);
         return LSW_ERR_OOM;
     }
+    s.t64 = s.q64 + nq;
+    s.t32 = s.q32 + nq;
     k_quarter<<<grid_for((long long)nq), 256, 0, st>>>(E, bz, bx, s.q64, s.q32, s.t64, s.t32);
     LSW_LAUNCH_CHECK();
     *out = s;
@@ -1103,8 +1105,6 @@ lsw_status build_spectrum(const lsw_green* g, int bz, int bx, Spectrum* out, cud
 void free_spectrum(Spectrum* s) {
     if (s->q64) cudaFree(s->q64);
     if (s->q32) cudaFree(s->q32);
-    if (s->t64) cudaFree(s->t64);
-    if (s->t32) cudaFree(s->t32);
     s->q64 = nullptr;
     s->q32 = nullptr;
     s->t64 = nullptr;
@@ -1117,12 +1117,12 @@ lsw_status green_init(lsw_green* g, cudaStream_t st) {
     k_green_table<<<grid_for((long long)nt), 256, 0, st>>>(g->table, g->nz, g->nx, g->h, g->k);
     LSW_LAUNCH_CHECK();
     g->twP = 2 * std::max(g->nz, g->nx);
-    LSW_CUDA(cudaMalloc(&g->tw64, g->twP * sizeof(double2)));
-    LSW_CUDA(cudaMalloc(&g->tw32, g->twP * sizeof(float2)));
+    LSW_CUDA(cudaMalloc(&g->tw64, (g->twP + kLineTables) * sizeof(double2)));
+    LSW_CUDA(cudaMalloc(&g->tw32, (g->twP + kLineTables) * sizeof(float2)));
+    g->lt64 = g->tw64 + g->twP;
+    g->lt32 = g->tw32 + g->twP;
     k_twiddles<<<grid_for(g->twP), 256, 0, st>>>(g->tw64, g->tw32, g->twP);
     LSW_LAUNCH_CHECK();
-    LSW_CUDA(cudaMalloc(&g->lt64, kLineTables * sizeof(double2)));
-    LSW_CUDA(cudaMalloc(&g->lt32, kLineTables * sizeof(float2)));
     k_line_tables<<<grid_for(kLineTables), 256, 0, st>>>(g->lt64, g->lt32);
     LSW_LAUNCH_CHECK();
     LSW_TRY(build_spectrum(g, g->nz, g->nx, &g->full, st));

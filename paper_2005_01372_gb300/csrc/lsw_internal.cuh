@@ -168,7 +168,7 @@ struct Spectrum {
     int bz = 0, bx = 0;
     double2* q64 = nullptr;
     float2* q32 = nullptr;
-    double2* t64 = nullptr;   // the same quarter, kz-major: (bz + 1) rows of the even kx, then the odd ones
+    double2* t64 = nullptr;   // (behind q64, q32) the same quarter, kz-major: (bz + 1) rows of the even kx, then the odd ones
     float2* t32 = nullptr;
 };
 
@@ -183,7 +183,7 @@ struct lsw_green {
     int twP = 0;                         // twiddle table length (max FFT size)
     double2* tw64 = nullptr;             // tw[m] = exp(-2 pi i m / twP)
     float2* tw32 = nullptr;
-    double2* lt64 = nullptr;             // line FFT tables (fft.cuh, line_table)
+    double2* lt64 = nullptr;             // (behind tw64, tw32) line FFT tables (fft.cuh, line_table)
     float2* lt32 = nullptr;
 };
 

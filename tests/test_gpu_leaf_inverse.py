@@ -1,4 +1,5 @@
-"""The batched Gauss-Jordan inverses of H's leaves by leaf size: one or more
+"""The batched Gauss-Jordan inverses of H's leaves by leaf size: up to 160
+rows in shared memory; beyond, one or more
 strips of 64 columns, panels by blocks of 256, 512 and 1024 threads.
 
 The contrast is confined to one leaf's cells.  The blocks that couple into that
@@ -25,7 +26,7 @@ def lsw():
     return L
 
 
-@pytest.mark.parametrize("nz,nx", [(16, 16), (8, 32), (16, 32), (32, 32), (32, 64)])
+@pytest.mark.parametrize("nz,nx", [(4, 8), (8, 8), (8, 16), (16, 16), (8, 32), (16, 32), (32, 32), (32, 64)])
 @pytest.mark.parametrize("prec", ["C128", "C64"])
 def test_leaf_sizes(lsw, nz, nx, prec):
     rng = np.random.default_rng(nz + nx)
