@@ -107,12 +107,12 @@ class ClockSampler:
 
 # The kernel family with the largest share of the step's serialised launch
 # list (an ncu capture of one step, gpu__time_duration per launch): the truncation's
-# eigen-decompositions (FP32 Jacobi kernels, Rayleigh-Ritz projection),
+# eigen-decompositions (FP64 Cholesky factor, one-sided FP32 Jacobi),
 # latency-bound; timed live with CUDA events on their launching streams over
 # the timed steps, against the algorithmic 36 k^3 real flops per matrix.
 DOMINANT = "heev"
-DOMINANT_KERNEL = ("heev: eigen-decompositions of the sketches' k x k Gram matrices for the truncation (FP32 "
-                   "Jacobi, FP64-accurate Rayleigh-Ritz projection, FP32 Jacobi polish; k = 50), 36 k^3 flops each")
+DOMINANT_KERNEL = ("heev: eigen-decompositions of the sketches' k x k Gram matrices for the truncation "
+                   "(one-sided FP32 Jacobi on the FP64 Cholesky factor; k = 50), 36 k^3 flops each")
 # DRAM bytes (read + write) per launch of the dominant family from one ncu
 # capture of this workload's step, or None when not captured for this build.
 DOMINANT_TRAFFIC_PER_LAUNCH = None
@@ -122,8 +122,8 @@ DOMINANT_TRAFFIC_PER_LAUNCH = None
 SOLVE_KERNEL = ("k_lr_partial_ws: every level's W^H x partials of the BF16 HODLR apply (tcgen05, warp-specialised "
                 "bulk-copy ring), 16 vectors at 1024^2")
 # DRAM bytes of one 16-field 1024^2 FP32 RESIDUAL apply (passes k_fa, k_fb,
-# k_fc: 369 + 489 + 516 MB), from one ncu capture of three applies.
-OPERATOR_TRAFFIC = 1.3735e9
+# k_fc: 381 + 488 + 639 MB), from one ncu capture of a cold apply.
+OPERATOR_TRAFFIC = 1.5083e9
 
 
 def fp32_alu_peak_tflops(sms: int = 152, sm_mhz: float = 2070.0) -> float:

@@ -144,7 +144,7 @@ lsw_status lsw_mempool_usage(uint64_t* used_current, uint64_t* used_high, int re
 
 /* Diagnostic timing of one kernel family inside any call (not part of the
  * method).  lsw_kernel_timer_start(family) resets and enables it for
- * "operator_c64" / "operator_c128" (the three FFT passes of one operator
+ * "operator_c64" / "operator_c128" (the FFT passes of one operator
  * apply in that precision), "qr" (the thin QR of complex64 sketch blocks),
  * "gram", "chol", "heev" (the truncation's eigen-decompositions),
  * "gj_update" (the Gauss-Jordan block updates), "leaf_tc" (the tensor-core
