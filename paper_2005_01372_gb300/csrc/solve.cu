@@ -171,6 +171,7 @@ lsw_status zero_residual(const lsw_green* g, const double* chi, const typename C
                          const typename Cx<R>::T* u0, typename Cx<R>::T* a, int nb, DevBuf& work, cudaStream_t st) {
     typedef typename Cx<R>::T C;
     const long long n = (long long)g->nz * g->nx;
+    if (nb == 1) return op_full<R>(g, chi, LSW_OP_RESIDUAL, u, u0, a, 1, work, st);     // one launch less
     if (!work.p) LSW_TRY(work.alloc(sizeof(C) * 2 * n * nb, st));
     LSW_TRY(op_full<R>(g, chi, LSW_OP_PLAIN, u, nullptr, a, 1, work, st));
     k_zero_residual<C><<<gridn(n), 256, 0, st>>>(a, u0, n, nb);
