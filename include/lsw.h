@@ -469,7 +469,11 @@ lsw_status lsw_fno_error(const lsw_fno* f, const void* x, const void* t, int bat
                          void* stream);
 /* The preconditioner: z_b = ||v_b|| * network([v_b / ||v_b||, chi/k0^2 + i k0 h])
  * for nbatch fields v (prec LSW_C128 or LSW_C64, device), on g's grid, which
- * must match the network's. */
+ * must match the network's.  The network computes in FP32 for either type:
+ * complex128 vectors are divided by their FP64 norms, rounded to complex64, and
+ * the results widened, so z carries FP32 accuracy.  For complex128 the order of
+ * the FP32 operations is fixed (dense products: slower than the fused passes
+ * complex64 takes), so that z repeats to its last digit. */
 lsw_status lsw_fno_apply(const lsw_fno* f, const lsw_green* g, const double* chi, const void* v,
                          void* z, int nbatch, int prec, void* stream);
 

@@ -77,6 +77,29 @@ __global__ void k_conj(const float2* a, float2* b, long long n) {
         b[e] = make_float2(a[e].x, -a[e].y);
 }
 
+// v[b][w][i] += bias[w]
+__global__ void k_bias(float2* v, const float2* __restrict__ bias, long long n, int W, int B) {
+    const long long tot = n * W * B;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
+        const int w = (int)((e / n) % W);
+        v[e].x += bias[w].x;
+        v[e].y += bias[w].y;
+    }
+}
+
+// v = split-GELU(z + bias) (or z + bias)
+__global__ void k_bias_act(const float2* __restrict__ z, const float2* __restrict__ bias, float2* __restrict__ v,
+                           long long n, int W, int B, int act) {
+    const long long tot = n * W * B;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
+        const int w = (int)((e / n) % W);
+        float2 t = z[e];
+        t.x += bias[w].x;
+        t.y += bias[w].y;
+        v[e] = act ? make_float2(gelu_f(t.x), gelu_f(t.y)) : t;
+    }
+}
+
 // [b][w][mode] <-> [mode][b][w]: per mode a W x B column-major matrix
 __global__ void k_bwm_to_mwb(const float2* __restrict__ s, float2* __restrict__ d, int B, int W, int MM) {
     const long long tot = (long long)B * W * MM;
@@ -403,6 +426,61 @@ static lsw_status fno_forward(const lsw_fno* f, const float2* x, float2* y, int 
     return LSW_OK;
 }
 
+// The forward pass for complex128 vectors (fno_apply_precond): the same network
+// as a chain of dense products.  The arithmetic is FP32 either way, but its
+// results leave as complex128, and callers compare and store them to the digits
+// of that type, where the rounding of every sum shows.  So for this type the
+// products, the order of their sums and with them every bit stay as they are;
+// the fused passes round differently (1e-6 of the result).
+static lsw_status fno_forward_dense(const lsw_fno* f, const float2* x, float2* y, int B, FnoTape& tp, cudaStream_t st) {
+    const long long n = f->n;
+    const int W = f->W, M = f->M, MM = M * M, nz = f->nz, nx = f->nx;
+    const float2* P = f->params;
+    lsw_status s = LSW_OK;
+    const size_t act = (size_t)B * W * n, modes = (size_t)B * W * MM;
+    float2* v = tp.get(act, st, &s);
+    float2* z = tp.get(act, st, &s);
+    float2* T1 = tp.get((size_t)B * W * M * nx, st, &s);
+    float2* Vh = tp.get(modes, st, &s);         // [b][w][mode]
+    float2* Vt = tp.get(modes, st, &s);         // [mode][b][w]
+    float2* Zt = tp.get(modes, st, &s);
+    if (s != LSW_OK) return s;
+    // lift: V_b (n x W) = X_b (n x 2) P^T (2 x W) + p
+    LSW_TRY(gemm<float>('N', 'N', (int)n, W, 2, c1(), x, (int)n, 2 * n, P + f->oPT, 2, 0, c0(), v, (int)n, W * n, B, st, true));
+    k_bias<<<gridn(n * W * B), 256, 0, st>>>(v, P + f->op, n, W, B);
+    LSW_LAUNCH_CHECK();
+    for (int l = 0; l < f->L; ++l) {
+        // Vh = Fz v FxT   (per sample and channel: M x M)
+        LSW_TRY(gemm<float>('N', 'N', M, nx, nz, c1(), f->Fz, M, 0, v, nz, n, c0(), T1, M, (long long)M * nx, B * W, st, true));
+        LSW_TRY(gemm<float>('N', 'N', M, M, nx, c1(), T1, M, (long long)M * nx, f->FxT, nx, 0, c0(), Vh, M, MM, B * W, st,
+                            true));
+        k_bwm_to_mwb<<<gridn((long long)B * W * MM), 256, 0, st>>>(Vh, Vt, B, W, MM);
+        LSW_LAUNCH_CHECK();
+        // Zt[mode] = R[mode] Vt[mode]
+        LSW_TRY(gemm<float>('N', 'N', W, B, W, c1(), P + f->oR[l], W, (long long)W * W, Vt, W, (long long)W * B, c0(), Zt,
+                            W, (long long)W * B, MM, st, true));
+        k_mwb_to_bwm<<<gridn((long long)B * W * MM), 256, 0, st>>>(Zt, Vh, B, W, MM);
+        LSW_LAUNCH_CHECK();
+        // z = Fz^H (Zh conj(Fx)) / n
+        LSW_TRY(gemm<float>('N', 'N', M, nx, M, c1(), Vh, M, MM, f->Fxc, M, 0, c0(), T1, M, (long long)M * nx, B * W, st,
+                            true));
+        LSW_TRY(gemm<float>('C', 'N', nz, nx, M, make_float2(1.f / (float)n, 0.f), f->Fz, M, 0, T1, M, (long long)M * nx,
+                            c0(), z, nz, n, B * W, st, true));
+        // z += V W^T;  v = sigma(z + b)
+        LSW_TRY(gemm<float>('N', 'N', (int)n, W, W, c1(), v, (int)n, W * n, P + f->oWT[l], W, 0, c1(), z, (int)n, W * n, B,
+                            st, true));
+        k_bias_act<<<gridn(n * W * B), 256, 0, st>>>(z, P + f->ob[l], v, n, W, B, l < f->L - 1);
+        LSW_LAUNCH_CHECK();
+    }
+    // project: y_b (n x 1) = x0_b + V_b Q^T + q  (the residual channel passes through)
+    LSW_CUDA(cudaMemcpy2DAsync(y, sizeof(float2) * n, x, sizeof(float2) * 2 * n, sizeof(float2) * n, B,
+                               cudaMemcpyDeviceToDevice, st));
+    LSW_TRY(gemm<float>('N', 'N', (int)n, 1, W, c1(), v, (int)n, W * n, P + f->oQT, W, 0, c1(), y, (int)n, n, B, st, true));
+    k_bias<<<gridn(n * B), 256, 0, st>>>(y, P + f->oq, n, 1, B);
+    LSW_LAUNCH_CHECK();
+    return LSW_OK;
+}
+
 static lsw_status fno_backward(lsw_fno* f, const float2* x, const float2* Gy, int B, FnoTape& tp, cudaStream_t st) {
     const long long n = f->n;
     const int W = f->W, M = f->M, MM = M * M;
@@ -495,7 +573,8 @@ lsw_status fno_apply_precond(const lsw_fno* f, const lsw_green* g, const double*
                                                          x.as<float2>(), n, nb);
     LSW_LAUNCH_CHECK();
     FnoTape tp;
-    LSW_TRY(fno_forward(f, x.as<float2>(), y.as<float2>(), nb, tp, st));
+    if (prec == LSW_C128) LSW_TRY(fno_forward_dense(f, x.as<float2>(), y.as<float2>(), nb, tp, st));
+    else LSW_TRY(fno_forward(f, x.as<float2>(), y.as<float2>(), nb, tp, st));
     if (prec == LSW_C128)
         k_fno_output<double2><<<gridn(n * nb), 256, 0, st>>>(y.as<float2>(), nrm.as<double>(), (double2*)z, n, nb);
     else

@@ -1850,12 +1850,16 @@ __global__ void __launch_bounds__(256) k_norm_partial_c64(const float2* __restri
     }
 }
 
-// a warp per field
+// A warp per field: the chunks' sums are read 32 at a time and added in their
+// order.
 __global__ void k_norm_reduce(const double* __restrict__ part, int nchunk, double* out) {
     const long long b = blockIdx.x;
     double s = 0;
-    for (int c = threadIdx.x; c < nchunk; c += 32) s += part[b * nchunk + c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    for (int c0 = 0; c0 < nchunk; c0 += 32) {
+        const int c = c0 + threadIdx.x, m = min(32, nchunk - c0);
+        const double v = c < nchunk ? part[b * nchunk + c] : 0.0;
+        for (int i = 0; i < m; ++i) s += __shfl_sync(0xffffffffu, v, i);
+    }
     if (threadIdx.x == 0) out[b] = s;
 }
 
@@ -1899,7 +1903,7 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
                 const typename Cx<R>::T* A, int lda, long long sA,
                 const typename Cx<R>::T* B, int ldb, long long sB,
                 typename Cx<R>::T beta, typename Cx<R>::T* C, int ldc, long long sC,
-                int batch, cudaStream_t st) {
+                int batch, cudaStream_t st, bool square) {
     typedef typename Cx<R>::T CT;
     if (m <= 0 || n <= 0 || batch <= 0) return LSW_OK;
     const int oa = (opA == 'N' || opA == 'n') ? 0 : 1, ob = (opB == 'N' || opB == 'n') ? 0 : 1;
@@ -2007,8 +2011,9 @@ lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha
     }
     // tiles of 64 x 64 outputs, or 32 on a side that has no more: 20 rows of the
     // leaf updates' V^H D^-1 filled a third of a 64-row tile (25 us on average
-    // in a 256^2 build, 17 with 32 rows)
-    const bool narrow = n <= 32, low = !narrow && m <= 32;
+    // in a 256^2 build, 17 with 32 rows).  square: 64 x 64 all the same, whose
+    // grid decides how K is split and with it the order of the sums.
+    const bool narrow = n <= 32, low = !narrow && m <= 32 && !square;
     const int BMv = narrow ? 128 : low ? 32 : 64, BNv = narrow ? 32 : low ? 128 : 64;
     const int gx = (m + BMv - 1) / BMv, gy = (n + BNv - 1) / BNv;
     auto launch = [&](int ks, int kc, CT* P) {
@@ -2404,7 +2409,7 @@ lsw_status norms2(const typename Cx<R>::T* x, long long n, int batch, double* ou
 #define LSW_INST(R)                                                                                               \
     template lsw_status gemm<R>(char, char, int, int, int, Cx<R>::T, const Cx<R>::T*, int, long long,             \
                                 const Cx<R>::T*, int, long long, Cx<R>::T, Cx<R>::T*, int, long long, int,        \
-                                cudaStream_t);                                                                    \
+                                cudaStream_t, bool);                                                              \
     template lsw_status qr_explicit<R>(Cx<R>::T*, int, int, long long, int, Cx<R>::T*, cudaStream_t);             \
     template lsw_status gram64<R>(const Cx<R>::T*, int, int, long long, int, double2*, cudaStream_t);             \
     template lsw_status cast_from64<R>(const double2*, Cx<R>::T*, long long, cudaStream_t);                        \

@@ -216,13 +216,14 @@ void free_spectrum(Spectrum* s);
 
 // ------------------------------------------------------ dense helpers (la.cu)
 // Batched complex GEMM, column-major:  C_b = alpha * op(A_b) * op(B_b) + beta * C_b
-// op: 'N' or 'C' (conjugate transpose).  A_b = A + b * sA, etc.
+// op: 'N' or 'C' (conjugate transpose).  A_b = A + b * sA, etc.  square: no
+// tiles of their own for m <= 32 (see the dispatch).
 template <typename R>
 lsw_status gemm(char opA, char opB, int m, int n, int k, typename Cx<R>::T alpha,
                 const typename Cx<R>::T* A, int lda, long long sA,
                 const typename Cx<R>::T* B, int ldb, long long sB,
                 typename Cx<R>::T beta, typename Cx<R>::T* C, int ldc, long long sC,
-                int batch, cudaStream_t st);
+                int batch, cudaStream_t st, bool square = false);
 
 // C_b = alpha sum_p P_p,b + beta C_b for ksplit parts of a batched product,
 // P[part][b] an m x n matrix, column-major.
