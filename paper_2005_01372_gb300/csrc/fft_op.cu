@@ -336,7 +336,10 @@ k_fb(typename Cx<R>::T* __restrict__ T_, int bz, const typename Cx<R>::T* __rest
         r = blk * KB + rp * PK;
         return Tb + ((long long)(row0 / KB + blk) * N + ix) * KB + (row0 % KB) + rp * PK;
     };
-    // the spectra arrive asynchronously behind the rows
+    pdl_start_next();
+    pdl_wait();
+    // the spectra arrive asynchronously behind the rows (after the wait: the
+    // kernel that made them may be the one before pass A)
     for (int r = threadIdx.x >> 5; r < ROWS; r += NTB / 32) {
         // kz = 2k + (kz parity) of row kz'; the spectrum's row holds the even
         // qx (N / 2 + 1 entries) and then the odd ones
@@ -345,8 +348,6 @@ k_fb(typename Cx<R>::T* __restrict__ T_, int bz, const typename Cx<R>::T* __rest
         const C* sp = spt + (long long)min(kz, pz - kz) * (N + 1);
         for (int e = threadIdx.x & 31; e <= N; e += 32) cp_async<sizeof(C)>(spec + r * (N + 1) + e, sp + e);
     }
-    pdl_start_next();
-    pdl_wait();
 #pragma unroll 8
     for (int e = threadIdx.x; e < nrun; e += NTB) {
         int r, ix;
