@@ -1798,13 +1798,23 @@ __global__ void __launch_bounds__(256) k_norm_partial(const C* __restrict__ x, l
     }
 }
 
-// The same for complex64.  FP64 runs at 2 lanes per cycle and SM, and two
-// conversions and two multiply-adds per entry made the norms of 16 fields of
-// 512^2 cells take 46 us.  Eight entries at a time are summed in FP32
-// arithmetic without loss: scaled by a power of two to at most 2, squares
-// split exactly (p + e = x x) and added by TwoSum (Dot2 of Ogita, Rump and
-// Oishi), the pair then added in FP64: four FP64 operations instead of 64, with
-// an error of 2^-48 of the group's own sum.
+// s <- fl(s + x); the rounding error, exactly (Knuth's TwoSum)
+__device__ __forceinline__ float two_sum(float& s, float x) {
+    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z));
+    s = t;
+    return e;
+}
+
+// The same for complex64, to FP64's own accuracy.  FP64 runs at 2 lanes per
+// cycle and SM, and two conversions and two multiply-adds per entry made the
+// norms of 16 fields of 512^2 cells take 46 us.  Eight entries at a time are
+// summed in FP32 arithmetic: scaled by a power of two to at most 2, squares
+// split exactly (p + e = x x) and added in threefold FP32 (Sum3 of Ogita, Rump
+// and Oishi: the rounding errors of the sum are summed with their own rounding
+// errors), an error of at most 2^-64 of the group's sum; its three parts then
+// join the FP64 sum: six FP64 operations for a group instead of 32.  Those
+// norms take 15 us (14 in two parts, which some groups put 8e-14 off).
 __global__ void __launch_bounds__(256) k_norm_partial_c64(const float2* __restrict__ x, long long n, int nchunk,
                                                           double* part) {
     const int b = blockIdx.y, ch = blockIdx.x;
@@ -1828,16 +1838,15 @@ __global__ void __launch_bounds__(256) k_norm_partial_c64(const float2* __restri
         }
         const int sc = max(254 - (__float_as_int(top) >> 23), 1);      // exponent of the scale
         const float f = __int_as_float(sc << 23);
-        float hi = 0.f, lo = 0.f;
+        float hi = 0.f, mid = 0.f, lo = 0.f;
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
             const float a = __fmul_rn(u & 1 ? v[u >> 1].y : v[u >> 1].x, f);
             const float p = __fmul_rn(a, a), e = __fmaf_rn(a, a, -p);
-            const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
-            lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z)), e));
-            hi = t;
+            const float r = two_sum(mid, two_sum(hi, p));
+            lo = __fadd_rn(lo, __fadd_rn(r, two_sum(mid, e)));
         }
-        s = fma((double)hi + (double)lo, __hiloint2double((1023 - 2 * (sc - 127)) << 20, 0), s);
+        s = fma((double)hi + ((double)mid + (double)lo), __hiloint2double((1023 - 2 * (sc - 127)) << 20, 0), s);
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     __shared__ double red[8];
