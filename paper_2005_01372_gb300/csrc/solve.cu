@@ -73,11 +73,22 @@ __global__ void k_scale_cast(const Cs* __restrict__ src, Cd* __restrict__ dst, c
     }
 }
 
+// v a rounded as the FP64 product is, with a = ah + al (to 2^-48): the FP32
+// arithmetic below is off by less than 2^-46 of the result, so where moving it by
+// 2^-44 either way leaves the same float, that float is the product's (Ziv's
+// test).  sure is cleared for the other entries, one in 2^18 and those too small
+// or too large for the argument: they need the FP64 product itself.
+__device__ __forceinline__ float scaled(float v, float ah, float al, bool& sure) {
+    const float p = v * al, t = fmaf(v, ah, p), e = fabsf(t) * 0x1p-44f;
+    const float lo = fmaf(v, ah, p - e), hi = fmaf(v, ah, p + e);
+    sure = sure && lo == hi && e > 1e-32f;
+    return lo;
+}
+
 // The next Krylov vector scale_s w_s, into vj and into the basis (col: its
-// column of source 0, ldv entries between sources).  For complex64 the scale
-// is split into two FP32 parts (the product then rounds once, as in FP64,
-// whose conversions made this 50 us for 16 fields of 512^2 cells); a scale out
-// of FP32's comfortable range keeps the FP64 product.
+// column of source 0, ldv entries between sources).  For complex64 most entries
+// stay off the FP64 pipe, whose conversions made this 50 us for 16 fields of
+// 512^2 cells (14 now); the results are the FP64 products all the same.
 template <typename C>
 __global__ void __launch_bounds__(256)
 k_basis_vector(const C* __restrict__ w, const double* __restrict__ scale, C* __restrict__ vj, C* __restrict__ col,
@@ -85,27 +96,35 @@ k_basis_vector(const C* __restrict__ w, const double* __restrict__ scale, C* __r
     const long long s = blockIdx.y;
     const double a = scale[s];
     const float ah = (float)a, al = (float)(a - (double)ah);
-    const bool split = sizeof(C) == 8 && ((fabsf(ah) > 1e-20f && fabsf(ah) < 1e20f) || a == 0.0);
+    const bool zero = a == 0.0, split = sizeof(C) == 8 && fabsf(ah) > 1e-20f && fabsf(ah) < 1e20f;
     const C* ws = w + s * n;
     for (long long i0 = blockIdx.x * 1024LL + threadIdx.x; i0 < n; i0 += gridDim.x * 1024LL) {
-        C v[4];
+        C v[4], o[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (i0 + 256 * u < n) v[u] = ws[i0 + 256 * u];
+        for (int u = 0; u < 4; ++u) v[u] = i0 + 256 * u < n ? ws[i0 + 256 * u] : czero<C>();
+        bool sure = zero || split;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (sizeof(C) == 8) {
+                // a zero scale keeps the signs of the FP64 products, and their NaNs
+                o[u].x = zero ? v[u].x * 0 : scaled((float)v[u].x, ah, al, sure);
+                o[u].y = zero ? v[u].y * 0 : scaled((float)v[u].y, ah, al, sure);
+            }
+        }
+        if (sizeof(C) == 16 || !(zero || sure)) {
+            // one branch for the eight: with one each, every product was computed (57 us)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                o[u].x = (double)v[u].x * a;
+                o[u].y = (double)v[u].y * a;
+            }
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const long long i = i0 + 256 * u;
             if (i >= n) break;
-            C o;
-            if (split) {
-                o.x = fmaf((float)v[u].x, ah, (float)v[u].x * al);
-                o.y = fmaf((float)v[u].y, ah, (float)v[u].y * al);
-            } else {
-                o.x = (double)v[u].x * a;
-                o.y = (double)v[u].y * a;
-            }
-            vj[s * n + i] = o;
-            col[s * ldv + i] = o;
+            vj[s * n + i] = o[u];
+            col[s * ldv + i] = o[u];
         }
     }
 }
