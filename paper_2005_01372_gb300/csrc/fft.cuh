@@ -55,15 +55,18 @@ __device__ __forceinline__ void dft8(C* v, bool inv) {
     dft4(o0, o1, o2, o3, inv);
     typedef decltype(o0.x) R;
     const R s = (R)0.70710678118654752440;
-    // w8^1 = (1 -+ i)/sqrt2, w8^2 = -+ i, w8^3 = (-1 -+ i)/sqrt2
-    const C w1o1 = inv ? mk((o1.x - o1.y) * s, (o1.x + o1.y) * s) : mk((o1.x + o1.y) * s, (o1.y - o1.x) * s);
-    const C w3o3 = inv ? mk((-o3.x - o3.y) * s, (o3.x - o3.y) * s) : mk((o3.y - o3.x) * s, (-o3.x - o3.y) * s);
+    // w8^1 = (1 -+ i)/sqrt2, w8^2 = -+ i, w8^3 = (-1 -+ i)/sqrt2; the factor
+    // 1/sqrt2 goes into the sums (one rounding less than a product and a sum)
+    const C q1 = inv ? mk(o1.x - o1.y, o1.x + o1.y) : mk(o1.x + o1.y, o1.y - o1.x);
+    const C q3 = inv ? mk(-o3.x - o3.y, o3.x - o3.y) : mk(o3.y - o3.x, -o3.x - o3.y);
     v[0] = vadd(e0, o0); v[4] = vsub(e0, o0);
-    v[1] = vadd(e1, w1o1); v[5] = vsub(e1, w1o1);
+    v[1] = mk(fma(s, q1.x, e1.x), fma(s, q1.y, e1.y));
+    v[5] = mk(fma(-s, q1.x, e1.x), fma(-s, q1.y, e1.y));
     const C a = mk(e2.x + o2.y, e2.y - o2.x), b = mk(e2.x - o2.y, e2.y + o2.x);
     v[2] = inv ? b : a;
     v[6] = inv ? a : b;
-    v[3] = vadd(e3, w3o3); v[7] = vsub(e3, w3o3);
+    v[3] = mk(fma(s, q3.x, e3.x), fma(s, q3.y, e3.y));
+    v[7] = mk(fma(-s, q3.x, e3.x), fma(-s, q3.y, e3.y));
 }
 
 // One radix-R stage over nlines lines of length P (line l at s + l*lstride).
@@ -143,43 +146,36 @@ template <int LOGN> struct LineCfg {
     static_assert(T <= E && T <= 32 && E % T == 0, "one transpose");
 };
 
-// cos(pi k / 16), 0 <= k <= 8
-__host__ __device__ constexpr double cos16(int k) {
-    return k == 0 ? 1.0 : k == 1 ? 0.98078528040323044913 : k == 2 ? 0.92387953251128675613
-         : k == 3 ? 0.83146961230254523708 : k == 4 ? 0.70710678118654752440 : k == 5 ? 0.55557023301960222474
-         : k == 6 ? 0.38268343236508977173 : k == 7 ? 0.19509032201612826785 : 0.0;
+// tan(pi r / 64) and sin(pi r / 32), 1 <= r <= 8
+__host__ __device__ constexpr double tan64(int r) {
+    return r == 1 ? 0.04912684976946725411 : r == 2 ? 0.09849140335716425308 : r == 3 ? 0.14833598753834742875
+         : r == 4 ? 0.19891236737965800691 : r == 5 ? 0.25048696019130546160 : r == 6 ? 0.30334668360734239168
+         : r == 7 ? 0.35780572131452410467 : 0.41421356237309504880;
 }
-__host__ __device__ constexpr double cos32(int k) {      // cos(2 pi k / 32), 0 <= k < 32
-    return k <= 8 ? cos16(k) : k <= 16 ? -cos16(16 - k) : k <= 24 ? -cos16(k - 16) : cos16(32 - k);
-}
-
-// cos(2 pi k / 64) for odd k, 0 < k < 64 (even k: cos32)
-__host__ __device__ constexpr double cos64(int k) {
-    return k % 2 == 0 ? cos32((k / 2) % 32) : k > 32 ? cos64(64 - k) : k > 16 ? -cos64(32 - k)
-         : k == 1 ? 0.99518472667219688624 : k == 3 ? 0.95694033573220886494 : k == 5 ? 0.88192126434835502971
-         : k == 7 ? 0.77301045336273696081 : k == 9 ? 0.63439328416364549822 : k == 11 ? 0.47139673682599764856
-         : k == 13 ? 0.29028467725446236764 : 0.09801714032956060199;
+__host__ __device__ constexpr double sin32(int r) {
+    return r == 1 ? 0.09801714032956060199 : r == 2 ? 0.19509032201612826785 : r == 3 ? 0.29028467725446236764
+         : r == 4 ? 0.38268343236508977172 : r == 5 ? 0.47139673682599764856 : r == 6 ? 0.55557023301960222474
+         : r == 7 ? 0.63439328416364549822 : 0.70710678118654752440;
 }
 
-// v times exp(-2 pi i K / 32) (forward) or its conjugate (inverse)
+// v times exp(-2 pi i K / 64) (forward) or its conjugate (inverse): an exact
+// quarter turn and a turn of at most 45 degrees by three shears,
+//   x += t y,  y -= s x,  x += t y,   t = tan(phi / 2), s = sin(phi).
+// Three multiply-adds instead of the four operations of a product with
+// (cos, sin), and a smaller error: the rounding of a cosine near one (3e-8 at
+// cos(pi / 16)), which all entries share, was the largest part of a transform's.
 template <int K, bool INV, typename C>
-__device__ __forceinline__ C rot32(C v) {
+__device__ __forceinline__ C rot64(C v) {
     typedef decltype(v.x) R;
-    constexpr int k = (INV ? 32 - (K % 32) : K) % 32;
-    if constexpr (k == 0) return v;
-    else if constexpr (k == 8) return mk(v.y, -v.x);
-    else if constexpr (k == 16) return mk(-v.x, -v.y);
-    else if constexpr (k == 24) return mk(-v.y, v.x);
-    else if constexpr (k % 8 == 4) {
-        constexpr R s = (R)0.70710678118654752440;
-        if constexpr (k == 4) return mk((v.x + v.y) * s, (v.y - v.x) * s);
-        else if constexpr (k == 12) return mk((v.y - v.x) * s, -(v.x + v.y) * s);
-        else if constexpr (k == 20) return mk(-(v.x + v.y) * s, (v.x - v.y) * s);
-        else return mk((v.x - v.y) * s, (v.x + v.y) * s);
+    constexpr int k = (INV ? 64 - (K % 64) : K) % 64;
+    constexpr int quarter = (k + 8) / 16 % 4, r = k - (k + 8) / 16 * 16;       // -8 <= r < 8
+    const C u = quarter == 0 ? v : quarter == 1 ? mk(v.y, -v.x) : quarter == 2 ? mk(-v.x, -v.y) : mk(-v.y, v.x);
+    if constexpr (r == 0) {
+        return u;
     } else {
-        constexpr R c = (R)cos32(k), s = (R)cos32((k + 24) % 32);     // cos(x - pi/2) = sin x
-        // (x + iy)(c - is)
-        return mk(v.x * c + v.y * s, v.y * c - v.x * s);
+        constexpr R t = (R)(r > 0 ? tan64(r) : -tan64(-r)), sn = (R)(r > 0 ? sin32(r) : -sin32(-r));
+        const R x = fma(t, u.y, u.x), y = fma(-sn, x, u.y);
+        return mk(fma(t, y, x), y);
     }
 }
 
@@ -187,10 +183,10 @@ __device__ __forceinline__ C rot32(C v) {
 template <int M, bool INV, int LEFT, typename C>
 __device__ __forceinline__ void rot_rows(C* y1, C* y2, C* y3) {
     if constexpr (LEFT > 1) {
-        constexpr int c = LEFT - 1, S = 32 / M;
-        y1[c] = rot32<S * c, INV>(y1[c]);
-        y2[c] = rot32<S * 2 * c, INV>(y2[c]);
-        y3[c] = rot32<S * 3 * c, INV>(y3[c]);
+        constexpr int c = LEFT - 1, S = 64 / M;
+        y1[c] = rot64<S * c, INV>(y1[c]);
+        y2[c] = rot64<S * 2 * c, INV>(y2[c]);
+        y3[c] = rot64<S * 3 * c, INV>(y3[c]);
         rot_rows<M, INV, LEFT - 1>(y1, y2, y3);
     }
 }
@@ -238,14 +234,7 @@ template <int M, bool INV, int LEFT = M, typename C>
 __device__ __forceinline__ void half_shift(C* v) {
     if constexpr (LEFT > 1) {
         constexpr int a = LEFT - 1;
-        if constexpr (M <= 16) {
-            v[a] = rot32<a * (16 / M), INV>(v[a]);
-        } else {
-            typedef decltype(v->x) R;
-            constexpr R c = (R)cos64(a), s = (R)cos64((a + 48) % 64);
-            v[a] = INV ? mk(v[a].x * c - v[a].y * s, v[a].y * c + v[a].x * s)
-                       : mk(v[a].x * c + v[a].y * s, v[a].y * c - v[a].x * s);
-        }
+        v[a] = rot64<a * (32 / M), INV>(v[a]);
         half_shift<M, INV, LEFT - 1>(v);
     }
 }

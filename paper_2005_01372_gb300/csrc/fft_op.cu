@@ -195,9 +195,10 @@ k_pass_c(const typename Cx<R>::T* __restrict__ T, DevGeom geo, int pz, int logpz
 // (85% busy).  A line's transform moves every entry twice through shared
 // memory (one transpose, inside a warp) where the radix-8 passes these
 // replaced moved it six times with two block barriers each.  RESIDUAL on one
-// GB300, before -> now: 256^2, 32 fields 95 -> 55 us; 1024^2, 16 fields 1098 ->
-// 539 us; ADJOINT 256 x 1024, 30 fields 487 -> 216 us; FP64 256^2, 32 fields
-// 1401 -> 1352 us.
+// GB300, before -> now: 256^2, 32 fields 95 -> 56 us; 1024^2, 16 fields 1098 ->
+// 536 us; ADJOINT 256 x 1024, 30 fields 487 -> 216 us; FP64 256^2, 32 fields
+// 1401 -> 1320 us.  The complex64 results are nearer to FP64's at every size
+// (256^2: 1.97e-7 -> 1.63e-7, 1024^2: 2.20e-7 -> 1.85e-7; rot64).
 template <typename C> __host__ __device__ constexpr int kblk() { return 64 / (int)sizeof(C); }
 template <typename C> __device__ __forceinline__ long long tile_index(int kz, int ix, int bx) {
     constexpr int KB = kblk<C>();
