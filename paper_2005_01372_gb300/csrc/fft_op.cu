@@ -950,14 +950,18 @@ void op_set_variant(int pz, int px, int rsize, int v) {
     g_tune[std::make_tuple(pz, px, rsize)] = v;
 }
 
-// One launch (k_small) for this product?  Where the GPU finishes before the
-// host has launched three kernels and fetched a work array (19.5 us a call
-// against 13.9).  GPU time of one launch against three, c64: 64 x 64 cells, 1
+// One launch (k_small) for this product?  Where a call's time is the host's,
+// which takes longer to launch three kernels and fetch a work array (19.5 us a
+// call of one 64 x 64 field) than to launch one (13.9).  The GPU alone is a little
+// slower with it.  One launch against three, c64: 64 x 64 cells, 1
 // field 8.2 / 7.6 us, 8 fields 8.3 / 7.7, 16 fields 11.6 / 8.0; 64 x 128, 1
 // field 10.2 / 9.5; 128 x 128, 1 field 17.4 / 11.9.  c128: 32 x 32 46.6 / 47.2,
 // 64 x 64, 8 fields 53.5 / 54.2, 16 fields 103 / 54.5.  So fields of up to 8192
-// cells, 32768 cells in all.  u and y must not overlap: one field's blocks may
-// write y before another's read u.
+// cells, 32768 cells in all.  Solvers keep a work array and replay their steps as
+// graphs; there the two are even: FGMRES in c64, 4 sources, 32 x 32 1.96 / 1.99 ms,
+// 64 x 64 5.34 / 5.29, 64 x 128 7.20 / 7.10; mixed with H 1.74 / 1.78, 2.85 / 2.87,
+// 2.74 / 2.69.  u and y must not overlap: one field's blocks may write y before
+// another's read u.
 bool op_small(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, int rsize, int nbatch, const void* u,
               const void* y) {
     const int bz = geo.bz, bx = geo.bx;
