@@ -285,6 +285,17 @@ __device__ __forceinline__ void line_fft(C (&v)[LineCfg<LOGN>::E], C* buf, int t
         for (int d = 0; d < T; ++d) v[j + J * d] = x[j * T + d];
 }
 
+// Lines of both parities of `cols` columns (a power of two) over groups of T
+// threads: group `line` takes column col of parity par, or none (false).  The
+// odd ones start on a whole warp, as line_fft wants it.
+__host__ __device__ constexpr int parity_lines(int cols, int T) { return 2 * (cols > 32 / T ? cols : 32 / T); }
+__host__ __device__ inline bool parity_line(int line, int cols, int T, int& par, int& col) {
+    const int half = parity_lines(cols, T) / 2;
+    par = line >= half;
+    col = line - par * half;
+    return col < cols;
+}
+
 // Tables of the line transforms, N = 8 .. 1024: three of N entries each.
 __host__ __device__ constexpr int line_table(int N) { return 3 * N - 24; }   // first entry of N's tables
 constexpr int kLineTables = line_table(2048);                                // entries in all

@@ -532,10 +532,10 @@ __device__ __forceinline__ void small_a(const SmallField<C>& f, const C* __restr
     constexpr int N = L::N, E = L::E, T = L::T, LINES = kSmallThreads / T, LS = line_stride<C, LOGN, kblk<C>()>();
     const int t = threadIdx.x % T;
     C* buf = f.bufs + (threadIdx.x / T) * LS;
-    for (int l0 = 0; l0 < 2 * f.cols; l0 += LINES) {
-        const int line = l0 + threadIdx.x / T;
-        const bool valid = line < 2 * f.cols;
-        const int par = valid && line >= f.cols, ix = f.ix0 + (valid ? line - par * f.cols : 0);
+    for (int l0 = 0; l0 < parity_lines(f.cols, T); l0 += LINES) {
+        int par, col;
+        const bool valid = parity_line(l0 + threadIdx.x / T, f.cols, T, par, col);
+        const int ix = f.ix0 + (valid ? col : 0);
         const C* uc = ub + (long long)ix * N;
         const double* ch = chb + (long long)ix * chi_ld;
         C v[E];
