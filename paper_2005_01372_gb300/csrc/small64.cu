@@ -454,10 +454,16 @@ k_rmul_dot2(float2* __restrict__ Y, int m, int k, long long sY, const double2* _
 // One CTA per matrix.
 //   1. The trace is scaled to 1 and the indices sorted by the diagonal's
 //      thousands (2^10): a sketch's own order is nearly decreasing and saves
-//      sweeps, and a floored pivot of step 2 still comes last.
-//   2. G = Lt D Lt^H in FP64 (square-root-free, as in k_chol_rinv).  A pivot
-//      not above 1e-15, the accuracy of G itself, becomes 1e-15 with nothing
-//      below it: no restart.
+//      sweeps, and a block's empty columns come last.
+//   2. G = Lt D Lt^H in FP64 (square-root-free, as in k_chol_rinv), without
+//      further pivoting.  A pivot not above 1e-15, the accuracy of G itself,
+//      becomes 1e-15 with nothing below it: no restart.  What is dropped below it
+//      can be as large as 3e-8 (columns nearly equal to earlier ones ahead of
+//      independent ones), but it couples directions of no weight: for the matrix
+//      G' that is factored, v^H G v <= (p + 1) v^H G' v after p such pivots
+//      (||v||_S <= ||v_j||_d + ||rest||_R for a positive S with diagonal
+//      blocks d and R), so directions that the truncation leaves out for their
+//      small eigenvalues in G' carry no more than p + 1 times as much of G.
 //   3. W = L, times 2^20 so that all squares are normal FP32 numbers.  Rounds of
 //      disjoint column pairs (circle method), sixteen lanes per pair: the
 //      pair's norms and inner product (four shuffles), the rotation, the update, one
