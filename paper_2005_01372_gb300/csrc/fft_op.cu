@@ -517,7 +517,7 @@ __device__ __forceinline__ void cluster_load(uint32_t a, double2& v) {
 // The block's share of a field: columns ix0 .. ix0 + cols, rows of T
 // rank * rows ..; row r of T at rows + r * ls in shared memory.
 template <typename C> struct SmallField {
-    int cl, logrows, cols, ix0, ls;
+    int logrows, cols, ix0, ls;
     C* rows;
     C* bufs;                                 // transpose buffers of the block's lines
     __device__ __forceinline__ uint32_t remote(int kz, int ix) const {
@@ -625,7 +625,6 @@ k_small(const typename Cx<R>::T* __restrict__ u, DevGeom geo, int logrows, const
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int b = blockIdx.x / cl, rank = (int)cluster_rank(), nrows = 1 << logrows, bz = geo.bz, bx = geo.bx;
     SmallField<C> f;
-    f.cl = cl;
     f.logrows = logrows;
     f.cols = bx / cl;
     f.ix0 = rank * f.cols;

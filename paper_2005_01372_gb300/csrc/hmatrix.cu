@@ -351,11 +351,6 @@ __global__ void k_eye_minus(C* M, int r) {
     }
 }
 
-template <typename C>
-__global__ void k_copy(const C* __restrict__ s, C* __restrict__ d, long long n) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) d[e] = s[e];
-}
-
 template <typename C, typename R>
 __global__ void k_scale_copy(const C* __restrict__ s, C* __restrict__ d, long long n, R a) {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
@@ -394,7 +389,7 @@ lsw_status truncate(const typename Cx<R>::T* Q, int nb, const typename Cx<R>::T*
     LSW_TRY(V.alloc(sizeof(C) * (size_t)nblk * rp * rp, st));
     LSW_TRY(gram64<R>(Yt, mb, rp, (long long)mb * rp, nblk, G.as<double2>(), st));
     if constexpr (sizeof(R) == 4) LSW_TRY(heev_c64(G.as<double2>(), V.as<float2>(), rp, nblk, st));
-    else LSW_TRY(heev_jacobi<R>(G.as<double2>(), V.as<C>(), rp, nblk, st));
+    else LSW_TRY(heev_jacobi(G.as<double2>(), V.as<double2>(), rp, nblk, st));
     const int rr = std::min(r, rp);
     if (rr < r) {
         LSW_CUDA(cudaMemsetAsync(Uout, 0, sizeof(C) * (size_t)sU * nblk, st));

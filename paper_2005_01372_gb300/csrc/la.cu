@@ -993,20 +993,19 @@ k_tsqr_apply(typename Cx<R>::T* __restrict__ Aall, int m, int k, long long sA, i
 // ends the iteration (the classical threshold rule, which terminates even
 // when rounding keeps the off-diagonal norm above a fixed fraction).
 
-// Parallel cyclic Jacobi in precision R (FP64; complex64 sketches take k_eig_gram): each round rotates k/2 disjoint
-// index pairs chosen by the circle method, so every pair is met once per
-// sweep.  Input: FP64 Hermitian G (k x k), scaled by its trace; output: the
+// Parallel cyclic Jacobi in FP64 (complex64 sketches take k_eig_gram): each
+// round rotates k/2 disjoint index pairs chosen by the circle method, so every
+// pair is met once per sweep.  Input: FP64 Hermitian G (k x k), scaled by its trace; output: the
 // eigenvectors as columns of V, by decreasing eigenvalue.
 // sort key of an eigenvalue: a NaN sorts last, so that the ranks of any k
 // values (ties broken by index) are a permutation of 0 .. k-1
-template <typename R>
-__device__ __forceinline__ R jacobi_key(R d) { return isnan(d) ? -INFINITY : d; }
+__device__ __forceinline__ double jacobi_key(double d) { return isnan(d) ? -INFINITY : d; }
 
 #define JACOBI_MARK_ROUND (rf[r & 1] = 1)
-template <typename R>
 __global__ void __launch_bounds__(1024)
-k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ Vall, int k) {
-    typedef typename Cx<R>::T C;
+k_heev_jacobi(const double2* __restrict__ Gall, double2* __restrict__ Vall, int k) {
+    typedef double R;
+    typedef double2 C;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int m = (k + 1) & ~1;                 // even number of players
     C* A = reinterpret_cast<C*>(sm_raw);        // k x k, column-major
@@ -1206,10 +1205,10 @@ k_heev_jacobi(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ 
 #undef JACOBI_MARK_ROUND
 #define JACOBI_COUNT_ROTATION ++nrw
 #define JACOBI_MARK_ROUND (rr = 1)
-template <typename R>
 __global__ void __launch_bounds__(256)
-k_heev_jacobi_warp(const double2* __restrict__ Gall, typename Cx<R>::T* __restrict__ Vall, int k, int batch) {
-    typedef typename Cx<R>::T C;
+k_heev_jacobi_warp(const double2* __restrict__ Gall, double2* __restrict__ Vall, int k, int batch) {
+    typedef double R;
+    typedef double2 C;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int m = (k + 1) & ~1;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2148,35 +2147,33 @@ lsw_status gram64(const typename Cx<R>::T* Y, int m, int k, long long sY, int ba
     return LSW_OK;
 }
 
-template <typename R>
-lsw_status heev_jacobi(const double2* G, typename Cx<R>::T* V, int k, int batch, cudaStream_t st) {
-    typedef typename Cx<R>::T CT;
+lsw_status heev_jacobi(const double2* G, double2* V, int k, int batch, cudaStream_t st) {
     if (batch <= 0 || k <= 0) return LSW_OK;
     if (k > 64) return LSW_ERR_INVALID_ARG;
     const int m = (k + 1) & ~1;
-    const size_t per = sizeof(CT) * 2 * k * k + sizeof(R) * 4 * (m / 2) + sizeof(int2) * (m / 2) + sizeof(int) * 64;
+    const size_t per = sizeof(double2) * 2 * k * k + sizeof(double) * 4 * (m / 2) + sizeof(int2) * (m / 2) + sizeof(int) * 64;
     const size_t perA = (per + 15) & ~size_t(15);
     const int wpc = (int)std::max<size_t>(1, std::min<size_t>(8, (200 * 1024) / perA));
-    static std::atomic<bool> attr[2];
-    if (!attr[sizeof(R) == 8]) {
-        LSW_CUDA(cudaFuncSetAttribute(k_heev_jacobi_warp<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        attr[sizeof(R) == 8] = true;
+    static std::atomic<bool> attr{false};
+    if (!attr) {
+        LSW_CUDA(cudaFuncSetAttribute(k_heev_jacobi_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        attr = true;
     }
     if (batch >= 4 * 152) {
         // many matrices: one warp each
-        k_heev_jacobi_warp<R><<<(batch + wpc - 1) / wpc, 32 * wpc, perA * wpc, st>>>(G, V, k, batch);
+        k_heev_jacobi_warp<<<(batch + wpc - 1) / wpc, 32 * wpc, perA * wpc, st>>>(G, V, k, batch);
         LSW_LAUNCH_CHECK();
         return LSW_OK;
     }
-    static std::atomic<bool> attrb[2];
-    if (!attrb[sizeof(R) == 8]) {
-        LSW_CUDA(cudaFuncSetAttribute(k_heev_jacobi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-        attrb[sizeof(R) == 8] = true;
+    static std::atomic<bool> attrb{false};
+    if (!attrb) {
+        LSW_CUDA(cudaFuncSetAttribute(k_heev_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        attrb = true;
     }
-    const size_t smb = sizeof(CT) * 3 * (size_t)k * k + sizeof(R) * 4 * (m / 2) + sizeof(int2) * (m / 2);
+    const size_t smb = sizeof(double2) * 3 * (size_t)k * k + sizeof(double) * 4 * (m / 2) + sizeof(int2) * (m / 2);
     // few matrices: the whole CTA of 1024 threads on each (a round is a
     // handful of dependent steps; more threads make each one shorter)
-    k_heev_jacobi<R><<<batch, batch <= 2 * 152 ? 1024 : 256, smb, st>>>(G, V, k);
+    k_heev_jacobi<<<batch, batch <= 2 * 152 ? 1024 : 256, smb, st>>>(G, V, k);
     LSW_LAUNCH_CHECK();
     return LSW_OK;
 }
@@ -2431,6 +2428,5 @@ lsw_status norms2(const typename Cx<R>::T* x, long long n, int batch, double* ou
 LSW_INST(float)
 LSW_INST(double)
 #undef LSW_INST
-template lsw_status heev_jacobi<double>(const double2*, double2*, int, int, cudaStream_t);
 
 }  // namespace lsw

@@ -242,11 +242,9 @@ template <typename R>
 lsw_status gram64(const typename Cx<R>::T* Y, int m, int k, long long sY, int batch,
                   double2* G, cudaStream_t st);
 
-// Batched Hermitian eigenvectors by cyclic Jacobi in precision R (FP64): V_b
-// (k x k) receives the eigenvectors of the FP64 matrix G_b as columns, sorted
-// by decreasing eigenvalue.
-template <typename R>
-lsw_status heev_jacobi(const double2* G, typename Cx<R>::T* V, int k, int batch, cudaStream_t st);
+// Batched Hermitian eigenvectors by cyclic Jacobi in FP64: V_b (k x k)
+// receives the eigenvectors of G_b as columns, sorted by decreasing eigenvalue.
+lsw_status heev_jacobi(const double2* G, double2* V, int k, int batch, cudaStream_t st);
 
 // FP64 small-matrix arithmetic of the sketches (small64.cu).
 // Gram matrices of complex64 blocks with error-free products (Dot2), FP64 result.

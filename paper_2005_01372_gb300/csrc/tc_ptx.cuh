@@ -1,7 +1,7 @@
 // Inline-PTX helpers of the library's tcgen05 kernels (tc_gemm.cu, lr_tc.cu):
 // shared-memory matrix descriptors of the canonical K-major layout without
-// swizzle, MMA issue and commit, bounded mbarrier waits, TMEM loads, and the
-// BF16 / TF32 splits of FP32 values.
+// swizzle, MMA issue and commit, bounded mbarrier waits, TMEM loads and stores,
+// the TF32 split of FP32 values and BF16 pairs.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -49,16 +49,7 @@ __host__ __device__ constexpr uint32_t idesc(uint32_t ab, int M, int N) {
     return (1u << 4) | (ab << 7) | (ab << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db, uint32_t id, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        :
-        : "r"(tmem), "l"(da), "l"(db), "r"(id), "r"(acc)
-        : "memory");
-}
-
-// the same with A in tensor memory (row = lane, 8 consecutive columns per MMA)
+// A in tensor memory (row = lane, 8 consecutive columns per MMA)
 __device__ __forceinline__ void mma_tf32_ta(uint32_t tmem, uint32_t ta, uint64_t db, uint32_t id, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
@@ -125,11 +116,6 @@ __device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
-}
-
-__device__ __forceinline__ void split_bf16(float x, float& hi, float& lo) {
-    hi = __bfloat162float(__float2bfloat16_rn(x));
-    lo = x - hi;
 }
 
 }  // namespace tcx
