@@ -197,7 +197,7 @@ k_pass_c(const typename Cx<R>::T* __restrict__ T, DevGeom geo, int pz, int logpz
 // replaced moved it six times with two block barriers each.  RESIDUAL on one
 // GB300, before -> now: 256^2, 32 fields 95 -> 56 us; 1024^2, 16 fields 1098 ->
 // 536 us; ADJOINT 256 x 1024, 30 fields 487 -> 216 us; FP64 256^2, 32 fields
-// 1401 -> 1320 us.  The complex64 results are nearer to FP64's at every size
+// 1401 -> 1272 us.  The complex64 results are nearer to FP64's at every size
 // (256^2: 1.97e-7 -> 1.63e-7, 1024^2: 2.20e-7 -> 1.85e-7; rot64).
 template <typename C> __host__ __device__ constexpr int kblk() { return 64 / (int)sizeof(C); }
 template <typename C> __device__ __forceinline__ long long tile_index(int kz, int ix, int bx) {
@@ -236,11 +236,15 @@ __device__ __forceinline__ void add_parities(C (&v)[LineCfg<LOGN>::E], C* buf, c
 }
 // T is read and written past L1 (every sector is used once per pass; L1 is
 // left to the twiddles), u0 and y evict first from L2, where T is to stay.
-constexpr int kFftThreads = 256;
+// Threads of a CTA.  FP64 128: its pipe is the bound (2 lanes per SM and cycle),
+// so that few fields want their lines on many SMs, and many fields gain by the
+// finer tail (with 256: one field of 256 x 256 137 us instead of 78, 8 fields of 1024 x
+// 256 1.49 ms instead of 1.37).
+template <typename R> constexpr int fft_threads() { return sizeof(R) == 8 ? 128 : 256; }
 // launch bounds: CTAs per SM the registers are to allow (E complex entries
 // and about as many temporaries per thread, more in pass B)
 template <typename R, int LOGN, bool PASS_B> constexpr int fft_ctas() {
-    return sizeof(R) == 8 ? (LineCfg<LOGN>::E == 32 ? 1 : 2)
+    return sizeof(R) == 8 ? (LineCfg<LOGN>::E == 32 ? 2 : 4)
                           : (LineCfg<LOGN>::E == 32 ? 2 : LineCfg<LOGN>::E == 16 && PASS_B ? 3 : 4);
 }
 
@@ -257,12 +261,12 @@ __device__ __forceinline__ void pdl_start_next() { asm volatile("griddepcontrol.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename R, int LOGN>
-__global__ void __launch_bounds__(kFftThreads, (fft_ctas<R, LOGN, false>()))
+__global__ void __launch_bounds__(fft_threads<R>(), (fft_ctas<R, LOGN, false>()))
 k_fa(const typename Cx<R>::T* __restrict__ u, DevGeom geo, const typename Cx<R>::T* __restrict__ lt, int adjoint,
      typename Cx<R>::T* __restrict__ T_, int nbatch, int per) {
     typedef typename Cx<R>::T C;
     typedef LineCfg<LOGN> L;
-    constexpr int N = L::N, E = L::E, T = L::T, COLS = kFftThreads / (2 * T);
+    constexpr int N = L::N, E = L::E, T = L::T, NT = fft_threads<R>(), COLS = NT / (2 * T);
     constexpr int LS = line_stride<C, LOGN, kblk<C>()>();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int t = threadIdx.x % T, line = threadIdx.x / T;
@@ -281,7 +285,7 @@ k_fa(const typename Cx<R>::T* __restrict__ u, DevGeom geo, const typename Cx<R>:
             const int2 org = box_origin(geo, b);
             if (b != b0) __syncthreads();
 #pragma unroll 4
-            for (int e = threadIdx.x; e < COLS * N; e += kFftThreads) {
+            for (int e = threadIdx.x; e < COLS * N; e += NT) {
                 const int c = e / N, iz = e % N;
                 if (ix0 + c < geo.bx) chs[e] = (R)geo.chi[(long long)(org.y + ix0 + c) * geo.chi_ld + org.x + iz];
             }
@@ -314,7 +318,7 @@ k_fa(const typename Cx<R>::T* __restrict__ u, DevGeom geo, const typename Cx<R>:
 // row itself, once both groups have read it.  Rows past the field's end are
 // transformed as they lie in shared memory and not stored.
 template <typename R, int LOGN, int NTB>
-__global__ void __launch_bounds__(NTB, (NTB == 256 ? fft_ctas<R, LOGN, true>() : 1))
+__global__ void __launch_bounds__(NTB, (NTB == fft_threads<R>() ? fft_ctas<R, LOGN, true>() : 1))
 k_fb(typename Cx<R>::T* __restrict__ T_, int bz, const typename Cx<R>::T* __restrict__ spt,
      const typename Cx<R>::T* __restrict__ lt) {
     typedef typename Cx<R>::T C;
@@ -437,13 +441,13 @@ __device__ __forceinline__ void column_out(C (&v)[E], const C* __restrict__ u, c
 }
 
 template <typename R, int LOGN>
-__global__ void __launch_bounds__(kFftThreads, (fft_ctas<R, LOGN, false>()))
+__global__ void __launch_bounds__(fft_threads<R>(), (fft_ctas<R, LOGN, false>()))
 k_fc(const typename Cx<R>::T* __restrict__ T_, DevGeom geo, const typename Cx<R>::T* __restrict__ lt, int mode,
      const typename Cx<R>::T* __restrict__ u, const typename Cx<R>::T* __restrict__ u0,
      typename Cx<R>::T* __restrict__ y) {
     typedef typename Cx<R>::T C;
     typedef LineCfg<LOGN> L;
-    constexpr int N = L::N, E = L::E, T = L::T, COLS = kFftThreads / (2 * T);
+    constexpr int N = L::N, E = L::E, T = L::T, NT = fft_threads<R>(), COLS = NT / (2 * T);
     constexpr int LS = line_stride<C, LOGN, kblk<C>()>();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int t = threadIdx.x % T, line = threadIdx.x / T;
@@ -833,8 +837,9 @@ lsw_status set_smem(K k, std::atomic<bool>& done) {
         default: return LSW_ERR_UNSUPPORTED_SIZE;        \
     }
 
+// pdl: let the kernel start while its predecessor runs (pdl_wait)
 template <typename K, typename... A>
-lsw_status launch_pdl(K k, dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+lsw_status launch_pass(K k, bool pdl, dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -844,7 +849,7 @@ lsw_status launch_pdl(K k, dim3 grid, int threads, size_t smem, cudaStream_t st,
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl ? 1 : 0;
     LSW_CUDA(cudaLaunchKernelEx(&cfg, k, args...));
     LSW_LAUNCH_CHECK();
     return LSW_OK;
@@ -852,55 +857,74 @@ lsw_status launch_pdl(K k, dim3 grid, int threads, size_t smem, cudaStream_t st,
 
 // log2 box sides lz, lx: 3 .. 10
 template <typename R>
-lsw_status launch_fa(int lz, int nbatch, cudaStream_t st, const typename Cx<R>::T* u, const DevGeom& dg,
+lsw_status launch_fa(int lz, bool pdl, int nbatch, cudaStream_t st, const typename Cx<R>::T* u, const DevGeom& dg,
                      const typename Cx<R>::T* tab, int adj, typename Cx<R>::T* work) {
     typedef typename Cx<R>::T C;
     static std::atomic<bool> done[11];
     LSW_LOG_SWITCH(lz, {
-        constexpr int lines = kFftThreads / LineCfg<L_>::T, cols = lines / 2;
+        constexpr int NT = fft_threads<R>(), lines = NT / LineCfg<L_>::T, cols = lines / 2;
         LSW_TRY(set_smem(k_fa<R, L_>, done[L_]));
-        // fields per CTA: up to 4 while about four CTAs per SM slot remain
+        // fields per CTA: up to 4 while 2048 threads per SM remain
         const int gx = (dg.bx + cols - 1) / cols;
-        const int per = std::max(1, std::min(4, (int)((long long)gx * nbatch / (152 * 8))));
-        LSW_TRY(launch_pdl(k_fa<R, L_>, dim3(gx, (nbatch + per - 1) / per), kFftThreads,
-                           sizeof(C) * lines * line_stride<C, L_, kblk<C>()>() + sizeof(R) * cols * LineCfg<L_>::N, st,
-                           u, dg, tab + line_table(1 << L_), adj, work, nbatch, per));
+        const int per = std::max(1, std::min(4, (int)((long long)gx * nbatch * NT / (152 * 2048))));
+        LSW_TRY(launch_pass(k_fa<R, L_>, pdl, dim3(gx, (nbatch + per - 1) / per), NT,
+                            sizeof(C) * lines * line_stride<C, L_, kblk<C>()>() + sizeof(R) * cols * LineCfg<L_>::N, st,
+                            u, dg, tab + line_table(1 << L_), adj, work, nbatch, per));
     })
     return LSW_OK;
 }
 
-// 512 threads: twice the rows, where they fit in shared memory and registers
+// 512 threads: twice the rows (FP64: four times), where they fit in shared memory and registers
 template <typename R, int LOGN> constexpr bool fb_wide() { return sizeof(R) == 4 || LineCfg<LOGN>::E < 32; }
 
 template <typename R, int NTB>
-lsw_status launch_fb(int lx, int bz, int nbatch, cudaStream_t st, typename Cx<R>::T* work,
+lsw_status launch_fb(int lx, bool pdl, int bz, int nbatch, cudaStream_t st, typename Cx<R>::T* work,
                      const typename Cx<R>::T* spt, const typename Cx<R>::T* tab) {
     typedef typename Cx<R>::T C;
     static std::atomic<bool> done[11];
     LSW_LOG_SWITCH(lx, {
-        constexpr int NT = fb_wide<R, L_>() ? NTB : 256, rows = NT / (2 * LineCfg<L_>::T);
+        constexpr int NT = fb_wide<R, L_>() ? NTB : fft_threads<R>(), rows = NT / (2 * LineCfg<L_>::T);
         LSW_TRY(set_smem(k_fb<R, L_, NT>, done[L_]));
-        LSW_TRY(launch_pdl(k_fb<R, L_, NT>, dim3((2 * bz + rows - 1) / rows, nbatch), NT,
-                           sizeof(C) * rows * (2 * line_stride<C, L_, rows>() + LineCfg<L_>::N + 1), st, work, bz, spt,
-                           tab + line_table(1 << L_)));
+        LSW_TRY(launch_pass(k_fb<R, L_, NT>, pdl, dim3((2 * bz + rows - 1) / rows, nbatch), NT,
+                            sizeof(C) * rows * (2 * line_stride<C, L_, rows>() + LineCfg<L_>::N + 1), st, work, bz, spt,
+                            tab + line_table(1 << L_)));
     })
     return LSW_OK;
 }
 
 template <typename R>
-lsw_status launch_fc(int lz, int nbatch, cudaStream_t st, const typename Cx<R>::T* work, const DevGeom& dg,
+lsw_status launch_fc(int lz, bool pdl, int nbatch, cudaStream_t st, const typename Cx<R>::T* work, const DevGeom& dg,
                      const typename Cx<R>::T* tab, int mode, const typename Cx<R>::T* u, const typename Cx<R>::T* u0,
                      typename Cx<R>::T* y) {
     typedef typename Cx<R>::T C;
     static std::atomic<bool> done[11];
     LSW_LOG_SWITCH(lz, {
-        constexpr int lines = kFftThreads / LineCfg<L_>::T, cols = lines / 2;
+        constexpr int NT = fft_threads<R>(), lines = NT / LineCfg<L_>::T, cols = lines / 2;
         LSW_TRY(set_smem(k_fc<R, L_>, done[L_]));
-        LSW_TRY(launch_pdl(k_fc<R, L_>, dim3((dg.bx + cols - 1) / cols, nbatch), kFftThreads,
-                           sizeof(C) * lines * line_stride<C, L_, kblk<C>()>(), st, work, dg, tab + line_table(1 << L_),
-                           mode, u, u0, y));
+        LSW_TRY(launch_pass(k_fc<R, L_>, pdl, dim3((dg.bx + cols - 1) / cols, nbatch), NT,
+                            sizeof(C) * lines * line_stride<C, L_, kblk<C>()>(), st, work, dg, tab + line_table(1 << L_),
+                            mode, u, u0, y));
     })
     return LSW_OK;
+}
+
+// Whether the passes start while their predecessors run.  It hides 2 to 3 us per
+// pass, but a pass that starts early lands on the SMs that its predecessor has
+// left free, and stays there: with CTAs for part of the SMs only, two and more of a
+// pass share an SM while others idle.  FP64, whose pipe is the bound, then loses
+// far more than it gains (8 fields of 128 x 128: 201 us against 100; one of 512 x 512 290
+// against 231; 16 x 1024, 8 fields 202 against 111), so it starts early only where
+// either kind of line has CTAs for four fifths of the SMs' slots (from there on
+// 7 to 10 us are gained: 128 x 128, 32 fields 307 against 315; 512 x 512, 2 fields 425 against
+// 433).  FP32 always does.
+template <typename R>
+bool start_early(int bz, int bx, int nbatch) {
+    if (sizeof(R) == 4) return true;
+    auto filled = [&](int side, long long lines) {      // lines of `side` cells, both parities
+        const int e = side >= 512 ? 32 : side >= 128 ? 16 : side >= 32 ? 8 : 4;                         // LineCfg
+        return lines * 2 * (side / e) / fft_threads<R>() * 5 >= 4LL * 152 * (e == 32 ? 2 : 4);          // fft_ctas
+    };
+    return filled(bz, (long long)bx * nbatch) && filled(bx, 2LL * bz * nbatch);
 }
 
 // The one-launch kernel's cluster: blocks per field, as many (at most 8) as
@@ -927,7 +951,7 @@ size_t small_cfg(int bz, int bx, int& cl) {
 
 // ---------------------------------------------------------- pass tuning
 // Variant of the operator passes per (2bz, 2bx, precision): 0 register FFT
-// with 256-thread row CTAs in pass B, 1 the same with 512-thread row CTAs,
+// with row CTAs of fft_threads in pass B, 1 the same with 512-thread row CTAs,
 // 2 the shared-memory Stockham passes.  Chosen by lsw_autotune.
 namespace {
 std::mutex g_tune_mu;
@@ -1022,10 +1046,11 @@ lsw_status op_apply(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, i
         KTimer kt(sizeof(R) == 8 ? "operator_c128" : "operator_c64", st, op_bytes(sizeof(C), bz, bx, nbatch, u0 != nullptr, mode),
                   op_flops(bz, bx, nbatch));
         const int lz = logpz - 1, lx = logpx - 1;
-        LSW_TRY(launch_fa<R>(lz, nbatch, st, u, dg, tab, mode == LSW_OP_ADJOINT, work));
-        if (variant == 1) LSW_TRY((launch_fb<R, 512>(lx, bz, nbatch, st, work, spt, tab)));
-        else LSW_TRY((launch_fb<R, 256>(lx, bz, nbatch, st, work, spt, tab)));
-        LSW_TRY(launch_fc<R>(lz, nbatch, st, work, dg, tab, mode, u, u0, y));
+        const bool pdl = start_early<R>(bz, bx, nbatch);
+        LSW_TRY(launch_fa<R>(lz, pdl, nbatch, st, u, dg, tab, mode == LSW_OP_ADJOINT, work));
+        if (variant == 1) LSW_TRY((launch_fb<R, 512>(lx, pdl, bz, nbatch, st, work, spt, tab)));
+        else LSW_TRY((launch_fb<R, fft_threads<R>()>(lx, pdl, bz, nbatch, st, work, spt, tab)));
+        LSW_TRY(launch_fc<R>(lz, pdl, nbatch, st, work, dg, tab, mode, u, u0, y));
         return LSW_OK;
     }
     // columns per CTA for passes A and C, rows per CTA for pass B
