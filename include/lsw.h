@@ -202,8 +202,8 @@ lsw_status lsw_point_sources(const lsw_green* g, const int32_t* positions, int n
  * (lsw_op_mode).  prec: LSW_C128 or LSW_C64 for u, u0 and y.  u0 may be
  * NULL for FORWARD and RESIDUAL (read as zero) and is ignored otherwise.
  * y must not alias u or u0.  Scratch: 2 * nbatch * nz * nx complex; none for
- * small fields (sides of 8 to 128, at most 8192 cells each and 32768 in all),
- * which take one launch. */
+ * small fields (sides of 4 to 128, at most 8192 cells each, 512 fields and
+ * 32768 cells in all), which take one launch. */
 lsw_status lsw_apply_operator(const lsw_green* g, int prec, const double* chi,
                               const void* u, const void* u0, void* y,
                               int nbatch, int mode, void* stream);

@@ -113,7 +113,7 @@ __device__ void smem_fft(C* s, int lstride, int nlines, int P, int logP,
 }
 
 // ------------------------------------------------------------------------
-// Line FFTs of N = 2^LOGN points (8 <= N <= 1024) held by T threads of one
+// Line FFTs of N = 2^LOGN points (4 <= N <= 1024) held by T threads of one
 // warp, E = N / T entries each, T <= E: thread t owns v[a] = x[T a + t].  The
 // transform is an E-point DFT in registers, one twiddle, one transpose
 // through shared memory inside the warp (no block barrier) and E / T T-point
@@ -223,10 +223,11 @@ __device__ __forceinline__ void rot_rows(C* y1, C* y2, C* y3) {
     }
 }
 
-// DFT of M entries (2, 4, 8, 16, 32) of a register array, in natural order
+// DFT of M entries (1, 2, 4, 8, 16, 32) of a register array, in natural order
 template <int M, bool INV, typename C>
 __device__ __forceinline__ void reg_dft(C* v) {
-    if constexpr (M == 2) {
+    if constexpr (M == 1) {
+    } else if constexpr (M == 2) {
         const C a = v[0];
         v[0] = vadd(a, v[1]);
         v[1] = vsub(a, v[1]);
@@ -328,8 +329,8 @@ __host__ __device__ inline bool parity_line(int line, int cols, int T, int& par,
     return col < cols;
 }
 
-// Tables of the line transforms, N = 8 .. 1024: three of N entries each.
-__host__ __device__ constexpr int line_table(int N) { return 3 * N - 24; }   // first entry of N's tables
+// Tables of the line transforms, N = 4 .. 1024: three of N entries each.
+__host__ __device__ constexpr int line_table(int N) { return 3 * N - 12; }   // first entry of N's tables
 constexpr int kLineTables = line_table(2048);                                // entries in all
 
 }  // namespace lsw

@@ -176,7 +176,7 @@ k_pass_c(const typename Cx<R>::T* __restrict__ T, DevGeom geo, int pz, int logpz
 
 // ------------------------------------------------- register-FFT passes
 // The same three passes with register-resident line FFTs, for box sides of
-// 8 .. 1024 cells.  A line of N cells zero-padded to 2N has the spectrum
+// 4 .. 1024 cells.  A line of N cells zero-padded to 2N has the spectrum
 //   X[2k] = DFT_N(x)[k],   X[2k + 1] = DFT_N(x w_2N^n)[k],
 // and the first N entries of an inverse transform of length 2N are
 //   y[n] = IDFT_N(Y[even])[n] + conj(w_2N^n) IDFT_N(Y[odd])[n],
@@ -650,6 +650,7 @@ k_small(const typename Cx<R>::T* __restrict__ u, DevGeom geo, int logrows, const
     const C* ltz = tab + line_table(bz);
 #define LSW_SMALL_SWITCH(n, ...)                                  \
     switch (n) {                                                  \
+        case 4: { constexpr int L_ = 2; __VA_ARGS__; break; }     \
         case 8: { constexpr int L_ = 3; __VA_ARGS__; break; }     \
         case 16: { constexpr int L_ = 4; __VA_ARGS__; break; }    \
         case 32: { constexpr int L_ = 5; __VA_ARGS__; break; }    \
@@ -671,7 +672,7 @@ k_small(const typename Cx<R>::T* __restrict__ u, DevGeom geo, int logrows, const
 // line twiddles and half-sample shifts of every line length (line_table)
 __global__ void k_line_tables(double2* t64, float2* t32) {
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kLineTables; e += gridDim.x * blockDim.x) {
-        int N = 8;
+        int N = 4;
         while (line_table(2 * N) <= e) N *= 2;
         const int E = N >= 512 ? 32 : N >= 128 ? 16 : N >= 32 ? 8 : 4, T = N / E;      // LineCfg
         const int i = e - line_table(N);
@@ -814,7 +815,7 @@ int grid_for(long long n, int bs = 256) {
 
 }  // namespace
 
-// Launch the register-FFT passes for a runtime log2 size (3..11).
+// Launch the register-FFT passes for a runtime log2 size (2..10).
 template <typename K>
 lsw_status set_smem(K k, std::atomic<bool>& done) {
     if (!done) {
@@ -826,6 +827,7 @@ lsw_status set_smem(K k, std::atomic<bool>& done) {
 
 #define LSW_LOG_SWITCH(lg, ...)                  \
     switch (lg) {                                \
+        case 2: { constexpr int L_ = 2; __VA_ARGS__; break; }   \
         case 3: { constexpr int L_ = 3; __VA_ARGS__; break; }   \
         case 4: { constexpr int L_ = 4; __VA_ARGS__; break; }   \
         case 5: { constexpr int L_ = 5; __VA_ARGS__; break; }   \
@@ -855,7 +857,7 @@ lsw_status launch_pass(K k, bool pdl, dim3 grid, int threads, size_t smem, cudaS
     return LSW_OK;
 }
 
-// log2 box sides lz, lx: 3 .. 10
+// log2 box sides lz, lx: 2 .. 10
 template <typename R>
 lsw_status launch_fa(int lz, bool pdl, int nbatch, cudaStream_t st, const typename Cx<R>::T* u, const DevGeom& dg,
                      const typename Cx<R>::T* tab, int adj, typename Cx<R>::T* work) {
@@ -941,6 +943,7 @@ size_t small_cfg(int bz, int bx, int& cl) {
         if (bz == 1 << L || bx == 1 << L)
             bufs = std::max(bufs, (size_t)(kSmallThreads / LineCfg<L>::T) * line_stride<C, L, kblk<C>()>());
     };
+    lines(std::integral_constant<int, 2>());
     lines(std::integral_constant<int, 3>());
     lines(std::integral_constant<int, 4>());
     lines(std::integral_constant<int, 5>());
@@ -983,14 +986,15 @@ void op_set_variant(int pz, int px, int rsize, int v) {
 // cells, 32768 cells in all.  Solvers keep a work array and replay their steps as
 // graphs; there the two are even: FGMRES in c64, 4 sources, 32 x 32 1.96 / 1.99 ms,
 // 64 x 64 5.34 / 5.29, 64 x 128 7.20 / 7.10; mixed with H 1.74 / 1.78, 2.85 / 2.87,
-// 2.74 / 2.69.  u and y must not overlap: one field's blocks may write y before
-// another's read u.
+// 2.74 / 2.69.  A field has a block of its own however small it is, so at most 512
+// fields: 2048 fields of 4 x 4 cells take 37 us in one launch, 23 in three.  u and y
+// must not overlap: one field's blocks may write y before another's read u.
 bool op_small(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, int rsize, int nbatch, const void* u,
               const void* y) {
     const int bz = geo.bz, bx = geo.bx;
-    if (!is_pow2(bz) || !is_pow2(bx) || bz < 8 || bx < 8 || bz > 128 || bx > 128 || bz * bx > 8192) return false;
+    if (!is_pow2(bz) || !is_pow2(bx) || bz < 4 || bx < 4 || bz > 128 || bx > 128 || bz * bx > 8192) return false;
     const long long cells = (long long)bz * bx * nbatch;
-    if (cells > (1 << 15) || !sp.t32 || !sp.t64 || op_variant(2 * bz, 2 * bx, rsize) == 2) return false;
+    if (cells > (1 << 15) || nbatch > 512 || !sp.t32 || !sp.t64 || op_variant(2 * bz, 2 * bx, rsize) == 2) return false;
     const char *pu = static_cast<const char*>(u), *py = static_cast<const char*>(y);
     return py + 2 * rsize * cells <= pu || pu + 2 * rsize * cells <= py;
 }
@@ -1040,7 +1044,7 @@ lsw_status op_apply(const lsw_green* g, const Spectrum& sp, const OpGeom& geo, i
         LSW_LAUNCH_CHECK();
         return LSW_OK;
     }
-    if (variant != 2 && bz >= 8 && bx >= 8 && bz <= 1024 && bx <= 1024 && sp.t32 && sp.t64) {
+    if (variant != 2 && bz >= 4 && bx >= 4 && bz <= 1024 && bx <= 1024 && sp.t32 && sp.t64) {
         const C* spt = reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)sp.t64 : (const void*)sp.t32);
         const C* tab = reinterpret_cast<const C*>(sizeof(R) == 8 ? (const void*)g->lt64 : (const void*)g->lt32);
         KTimer kt(sizeof(R) == 8 ? "operator_c128" : "operator_c64", st, op_bytes(sizeof(C), bz, bx, nbatch, u0 != nullptr, mode),
