@@ -669,21 +669,6 @@ k_small(const typename Cx<R>::T* __restrict__ u, DevGeom geo, int logrows, const
     cluster_wait();                          // no block leaves while its rows may be read
 }
 
-// line twiddles and half-sample shifts of every line length (line_table)
-__global__ void k_line_tables(double2* t64, float2* t32) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kLineTables; e += gridDim.x * blockDim.x) {
-        int N = 4;
-        while (line_table(2 * N) <= e) N *= 2;
-        const int E = N >= 512 ? 32 : N >= 128 ? 16 : N >= 32 ? 8 : 4, T = N / E;      // LineCfg
-        const int i = e - line_table(N);
-        double s, c;
-        const int which = i / N, cc = (i - which * N) / T, t = i % T;
-        sincospi(-(double)(which == 0 ? 2 * cc * t : which == 1 ? (2 * cc + 1) * t : cc * (2 * t + 1)) / N, &s, &c);
-        t64[e] = make_double2(c, s);
-        t32[e] = make_float2((float)c, (float)s);
-    }
-}
-
 // ------------------------------------------------ generic strided 1D FFTs
 // nlines lines of length P: element i of line l at data[l * lstep + i * estep].
 template <int NT>
@@ -761,10 +746,23 @@ __global__ void k_quarter(const double2* __restrict__ F, int bz, int bx, double2
     }
 }
 
+// exp(-2 pi i m / P), m < P, then the line twiddles and half-sample shifts of
+// every line length (line_table), in one launch
 __global__ void k_twiddles(double2* tw64, float2* tw32, int P) {
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < P; m += gridDim.x * blockDim.x) {
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < P + kLineTables; m += gridDim.x * blockDim.x) {
+        double turn;                    // in half turns
+        if (m < P) {
+            turn = -2.0 * m / P;
+        } else {
+            const int e = m - P;
+            int N = 4;
+            while (line_table(2 * N) <= e) N *= 2;
+            const int E = N >= 512 ? 32 : N >= 128 ? 16 : N >= 32 ? 8 : 4, T = N / E;      // LineCfg
+            const int i = e - line_table(N), which = i / N, c = (i - which * N) / T, t = i % T;
+            turn = -(double)(which == 0 ? 2 * c * t : which == 1 ? (2 * c + 1) * t : c * (2 * t + 1)) / N;
+        }
         double s, c;
-        sincospi(-2.0 * m / P, &s, &c);
+        sincospi(turn, &s, &c);
         tw64[m] = make_double2(c, s);
         tw32[m] = make_float2((float)c, (float)s);
     }
@@ -1155,9 +1153,7 @@ lsw_status green_init(lsw_green* g, cudaStream_t st) {
     LSW_CUDA(cudaMalloc(&g->tw32, (g->twP + kLineTables) * sizeof(float2)));
     g->lt64 = g->tw64 + g->twP;
     g->lt32 = g->tw32 + g->twP;
-    k_twiddles<<<grid_for(g->twP), 256, 0, st>>>(g->tw64, g->tw32, g->twP);
-    LSW_LAUNCH_CHECK();
-    k_line_tables<<<grid_for(kLineTables), 256, 0, st>>>(g->lt64, g->lt32);
+    k_twiddles<<<grid_for(g->twP + kLineTables), 256, 0, st>>>(g->tw64, g->tw32, g->twP);
     LSW_LAUNCH_CHECK();
     LSW_TRY(build_spectrum(g, g->nz, g->nx, &g->full, st));
     LSW_CUDA(cudaStreamSynchronize(st));

@@ -39,7 +39,7 @@ struct lsw_fno {
     float2* FxT = nullptr;       // nx x M   (F_x)^T
     float2* Fxc = nullptr;       // M x nx   conj(F_x)
     bool fast = false;           // truncated transforms by register DFTs (fno_passes.cuh)
-    float2* twz = nullptr;       // their line twiddles, nz and nx entries
+    float2* twz = nullptr;       // their line twiddles, nz and nx entries (inside Fz's and FxT's arrays)
     float2* twx = nullptr;
     // offsets into params
     long long oPT, op, oQT, oq;
@@ -618,7 +618,11 @@ lsw_status lsw_fno_create(const lsw_fno_params* p, void* stream, lsw_fno** out) 
         if (s == LSW_OK && cudaMalloc(ptr, sizeof(float2) * cnt) != cudaSuccess) s = LSW_ERR_OOM;
     };
     al(&f->params, f->np); al(&f->grads, f->np); al(&f->adam_m, f->np); al(&f->adam_v, f->np);
-    al(&f->Fz, (long long)f->M * f->nz); al(&f->FxT, (long long)f->M * f->nx); al(&f->Fxc, (long long)f->M * f->nx);
+    f->fast = fno_fast(f->nz, f->nx, f->M);
+    // the line twiddles of the register transforms lie behind Fz and FxT
+    al(&f->Fz, (long long)(f->M + f->fast) * f->nz);
+    al(&f->FxT, (long long)(f->M + f->fast) * f->nx);
+    al(&f->Fxc, (long long)f->M * f->nx);
     if (s != LSW_OK) { lsw_fno_destroy(f); return s; }
     cudaMemsetAsync(f->grads, 0, sizeof(float2) * f->np, st);
     cudaMemsetAsync(f->adam_m, 0, sizeof(float2) * f->np, st);
@@ -634,14 +638,10 @@ lsw_status lsw_fno_create(const lsw_fno_params* p, void* stream, lsw_fno** out) 
             k_conj<<<gridn((long long)f->M * f->nx), 256, 0, st>>>(tmp.as<float2>(), f->Fxc, (long long)f->M * f->nx);
         }
     }
-    f->fast = fno_fast(f->nz, f->nx, f->M);
     if (f->fast) {
-        al(&f->twz, f->nz);
-        al(&f->twx, f->nx);
-        if (s == LSW_OK) {
-            k_line_twiddles<<<gridn(f->nz), 256, 0, st>>>(f->twz, f->nz, f->M);
-            k_line_twiddles<<<gridn(f->nx), 256, 0, st>>>(f->twx, f->nx, f->M);
-        }
+        f->twz = f->Fz + (long long)f->M * f->nz;
+        f->twx = f->FxT + (long long)f->M * f->nx;
+        k_line_twiddles<<<gridn(f->nz + f->nx), 256, 0, st>>>(f->twz, f->nz, f->twx, f->nx, f->M);
     }
     // Gaussian initial weights (Philox), scaled per tensor by 1/sqrt(fan-in); biases zero
     if (s == LSW_OK) {
@@ -680,7 +680,7 @@ lsw_status lsw_fno_create(const lsw_fno_params* p, void* stream, lsw_fno** out) 
 
 lsw_status lsw_fno_destroy(lsw_fno* f) {
     if (!f) return LSW_ERR_INVALID_ARG;
-    for (float2* p : {f->params, f->grads, f->adam_m, f->adam_v, f->Fz, f->FxT, f->Fxc, f->twz, f->twx})
+    for (float2* p : {f->params, f->grads, f->adam_m, f->adam_v, f->Fz, f->FxT, f->Fxc})
         if (p) cudaFree(p);
     delete f;
     return LSW_OK;

@@ -17,15 +17,15 @@
 
 namespace lsw {
 
-// tw[a q + b] = w_n^(b k_a)
-__global__ void k_line_twiddles(float2* tw, int n, int M) {
-    const int q = n / M;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+// tw[a q + b] = w_n^(b k_a), for both axes
+__global__ void k_line_twiddles(float2* twz, int nz, float2* twx, int nx, int M) {
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < nz + nx; g += gridDim.x * blockDim.x) {
+        const int n = g < nz ? nz : nx, e = g < nz ? g : g - nz, q = n / M;
         const int a = e / q, b = e - a * q;
         const int k = a < M / 2 ? a : a - M;
         double s, c;
         sincospi(-2.0 * (double)(k * b) / n, &s, &c);
-        tw[e] = make_float2((float)c, (float)s);
+        (g < nz ? twz : twx)[e] = make_float2((float)c, (float)s);
     }
 }
 
