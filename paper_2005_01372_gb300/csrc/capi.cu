@@ -35,6 +35,19 @@ void set_last_error(cudaError_t e, const char* what, const char* file, int line)
     snprintf(g_last_error, sizeof g_last_error, "%s: %s (%s:%d)", what, cudaGetErrorString(e), file, line);
 }
 
+std::mutex& capture_mutex() {
+    static std::mutex mu;
+    return mu;
+}
+void device_wait() {
+    std::lock_guard<std::mutex> lk(capture_mutex());
+    if (cudaDeviceSynchronize() != cudaSuccess) cudaGetLastError();
+}
+void device_free(void* p) {
+    std::lock_guard<std::mutex> lk(capture_mutex());
+    if (cudaFree(p) != cudaSuccess) cudaGetLastError();
+}
+
 namespace {
 struct TimerState {
     std::mutex mu;
@@ -354,9 +367,9 @@ lsw_status lsw_build_green(const lsw_grid* grid, void* stream, lsw_green** out) 
 
 lsw_status lsw_destroy_green(lsw_green* g) {
     if (!g) return LSW_ERR_INVALID_ARG;
-    if (g->table) cudaFree(g->table);
-    if (g->tw64) cudaFree(g->tw64);
-    if (g->tw32) cudaFree(g->tw32);
+    if (g->table) device_free(g->table);
+    if (g->tw64) device_free(g->tw64);
+    if (g->tw32) device_free(g->tw32);
     free_spectrum(&g->full);
     delete g;
     return LSW_OK;

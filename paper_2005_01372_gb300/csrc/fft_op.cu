@@ -1135,8 +1135,8 @@ lsw_status build_spectrum(const lsw_green* g, int bz, int bx, Spectrum* out, cud
 }
 
 void free_spectrum(Spectrum* s) {
-    if (s->q64) cudaFree(s->q64);
-    if (s->q32) cudaFree(s->q32);
+    if (s->q64) device_free(s->q64);
+    if (s->q32) device_free(s->q32);
     s->q64 = nullptr;
     s->q32 = nullptr;
     s->t64 = nullptr;

@@ -681,7 +681,7 @@ lsw_status lsw_fno_create(const lsw_fno_params* p, void* stream, lsw_fno** out) 
 lsw_status lsw_fno_destroy(lsw_fno* f) {
     if (!f) return LSW_ERR_INVALID_ARG;
     for (float2* p : {f->params, f->grads, f->adam_m, f->adam_v, f->Fz, f->FxT, f->Fxc})
-        if (p) cudaFree(p);
+        if (p) device_free(p);
     delete f;
     return LSW_OK;
 }

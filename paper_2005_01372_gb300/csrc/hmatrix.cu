@@ -88,7 +88,7 @@ struct Tree {
 // Large H-matrix arrays come from the device's stream-ordered pool (which
 // keeps freed memory mapped: the next build of the same size reuses it
 // without new mappings).  The allocation is complete before the call
-// returns; a release first waits for the device, as cudaFree would.
+// returns; a release first waits for the device, as device_free would.
 inline lsw_status pool_alloc(void** p, size_t bytes) {
     if (cudaMallocAsync(p, bytes, 0) != cudaSuccess) {
         cudaGetLastError();
@@ -99,7 +99,7 @@ inline lsw_status pool_alloc(void** p, size_t bytes) {
     return LSW_OK;
 }
 inline void pool_free_all(std::initializer_list<const std::vector<void*>*> lists) {
-    cudaDeviceSynchronize();
+    device_wait();
     for (auto v : lists)
         for (void* p : *v)
             if (p) cudaFreeAsync(p, 0);
@@ -1619,10 +1619,10 @@ lsw_status lsw_destroy_hmatrix(lsw_hmatrix* h) {
     h->h32.release();
     h->h64.release();
     h->hb.release();
-    if (h->perm_d) cudaFree(h->perm_d);
-    if (h->smwU) cudaFree(h->smwU);
-    if (h->smwW) cudaFree(h->smwW);
-    if (h->smwZ) cudaFree(h->smwZ);
+    if (h->perm_d) device_free(h->perm_d);
+    if (h->smwU) device_free(h->smwU);
+    if (h->smwW) device_free(h->smwW);
+    if (h->smwZ) device_free(h->smwZ);
     delete h;
     return LSW_OK;
 }

@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <mutex>
 #include <stdint.h>
 
 #include <cstddef>
@@ -116,6 +118,14 @@ void timer_release(std::vector<TimedSpan>& spans);
 
 inline bool is_pow2(long long v) { return v > 0 && (v & (v - 1)) == 0; }
 inline int ilog2(long long v) { int l = 0; while ((1LL << l) < v) ++l; return l; }
+
+// Calls that wait for the whole device (cudaDeviceSynchronize, cudaFree) fail
+// while any thread captures a stream: then nothing is waited for, and the error
+// comes up at the calling thread's next launch.  So the library's captures (solve.cu)
+// hold this lock, and its device-wide calls go through the two below.
+std::mutex& capture_mutex();
+void device_wait();
+void device_free(void* p);
 
 // Stream-ordered scratch that frees itself.
 struct DevBuf {

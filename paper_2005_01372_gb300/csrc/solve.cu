@@ -294,15 +294,18 @@ struct StepGraph {
             failed = true;
             return body(st);
         }
+        std::unique_lock<std::mutex> no_device_wide_calls(capture_mutex());
         const unsigned long long l0 = launch_counter();
         if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
             cudaGetLastError();
             failed = true;
+            no_device_wide_calls.unlock();
             return body(st);
         }
         const lsw_status s = body(cs);
         cudaGraph_t gr = nullptr;
         const cudaError_t e = cudaStreamEndCapture(cs, &gr);
+        no_device_wide_calls.unlock();
         launches = (long long)(launch_counter() - l0);
         spans = timer_take_captured();
         if (s == LSW_OK && e == cudaSuccess && gr && cudaGraphInstantiate(&exec, gr, 0) != cudaSuccess) exec = nullptr;
