@@ -624,7 +624,9 @@ k_lr_partial_f32(LrLevels<float2, float2> lv, int m, int r, int k, const float2*
                        reinterpret_cast<float2*>(sm_raw), P + (long long)blockIdx.x * r * k);
 }
 
-// T[level q][block j] = sum over the block's chunks of the partials, in order.
+// T[level q][block j] = sum over the block's chunks of the partials, in order,
+// eight of them read at a time (64 one after the other take 15 us where 8 in
+// flight take 11).
 template <typename C, typename FT>
 __global__ void k_lr_reduce(LrLevels<C, FT> lv, int r, int k, const C* __restrict__ P, C* __restrict__ T) {
     const long long nout = (long long)r * k;
@@ -638,7 +640,15 @@ __global__ void k_lr_reduce(LrLevels<C, FT> lv, int r, int k, const C* __restric
         const int per = lv.nb[q] / lv.ch[q];
         const C* p = P + ((long long)lv.chunk0[q] + (long long)j * per) * nout + oi;
         C s = czero<C>();
-        for (int u = 0; u < per; ++u) s = cadd(s, p[(long long)u * nout]);
+        int u = 0;
+        for (; u + 8 <= per; u += 8) {
+            C v[8];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) v[w] = p[(long long)(u + w) * nout];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) s = cadd(s, v[w]);
+        }
+        for (; u < per; ++u) s = cadd(s, p[(long long)u * nout]);
         T[e] = s;
     }
 }
